@@ -3,6 +3,7 @@
 // state objects.  The hot path is in api_path.cu, ADAPT-VQE in api_vqe.cu,
 // the helpers they share in api_common.cu.
 #include "api_internal.h"
+#include "build_full.h"
 #include "dev.cuh"
 #include "grad.cuh"
 
@@ -487,6 +488,192 @@ extern "C" int tq_hf_index(int n_qubits, int n_electrons, int mapping, long long
 
 namespace {
 
+// Byte offsets of arrays packed into one allocation, 256-byte aligned (so
+// every array meets the alignment of the bulk copies), and the host image of
+// those that are uploaded.
+struct Packed {
+    size_t bytes = 0;
+    std::vector<unsigned char> image;
+    size_t room(size_t n) {
+        const size_t at = bytes;
+        bytes += (std::max<size_t>(n, 16) + 255) & ~(size_t)255;
+        return at;
+    }
+    template <typename T>
+    size_t put(const std::vector<T>& v) {
+        const size_t at = room(v.size() * sizeof(T));
+        image.resize(bytes);
+        if (!v.empty()) std::memcpy(image.data() + at, v.data(), v.size() * sizeof(T));
+        return at;
+    }
+};
+
+// The Pauli sum by X-mask: group masks, term offsets, terms, and apart from
+// them the diagonal (x = 0) terms.
+struct Grouped {
+    std::vector<uint32_t> gx, tz, dz;
+    std::vector<int> goff;
+    std::vector<double> tc, dc;
+    double maxc = 0.0;
+};
+
+Grouped group_terms(const std::vector<PauliTerm>& terms) {
+    Grouped q;
+    for (const auto& t : terms) {
+        q.maxc = std::max(q.maxc, std::fabs(t.c));
+        if (t.x == 0) {
+            q.dz.push_back((uint32_t)t.z);
+            q.dc.push_back(t.c);
+            continue;
+        }
+        if (q.gx.empty() || q.gx.back() != (uint32_t)t.x) {
+            q.gx.push_back((uint32_t)t.x);
+            q.goff.push_back((int)q.tz.size());
+        }
+        q.tz.push_back((uint32_t)t.z);
+        q.tc.push_back(t.c);
+    }
+    q.goff.push_back((int)q.tz.size());
+    return q;
+}
+
+unsigned long long double_bits(double v) {
+    unsigned long long b;
+    std::memcpy(&b, &v, sizeof b);
+    return b;
+}
+
+// Full space: diagonal, CSR and XOR-ELL from value tables (build_full.cu).
+// Two allocations: one for everything whose size is known beforehand, one
+// for the entries; what only the build needs lives in context scratch.
+void build_full(tq_ctx* c, tq_ham* h, const Grouped& q) {
+    HamView& v = h->view;
+    const long long D = h->D, B = (D + XELL_ROWS - 1) / XELL_ROWS;
+    const size_t vb = h->prec == TQ_C128 ? sizeof(double) : sizeof(float);
+    const BuildPlan plan = plan_build(h->nq, q.gx, q.goff, q.tz, q.dz);
+    const int G = v.G, W = (int)plan.wx.size(), H = (int)plan.hx.size();
+    Packed a;
+    const size_t a_gx = a.put(q.gx), a_goff = a.put(q.goff), a_tz = a.put(q.tz), a_tc = a.put(q.tc),
+                 a_dz = a.put(q.dz), a_dc = a.put(q.dc);
+    const size_t a_diag = a.room((size_t)D * sizeof(double)), a_row = a.room((size_t)(D + 1) * sizeof(int)),
+                 a_xptr = a.room((size_t)(B + 1) * sizeof(int));
+    v.n_blocks = B;
+    v.xgrid = xell_grid(B, h->prec, c->sm_count);
+    const size_t a_split = a.room((size_t)(v.xgrid + 1) * sizeof(int));
+    auto* base = static_cast<unsigned char*>(dev_alloc(a.bytes));
+    h->allocs.push_back(base);
+    TQ_CUDA(cudaMemcpy(base, a.image.data(), a.image.size(), cudaMemcpyHostToDevice));
+    v.gx = reinterpret_cast<uint32_t*>(base + a_gx);
+    v.goff = reinterpret_cast<int*>(base + a_goff);
+    v.tz = reinterpret_cast<uint32_t*>(base + a_tz);
+    v.tc = reinterpret_cast<double*>(base + a_tc);
+    v.dz = reinterpret_cast<uint32_t*>(base + a_dz);
+    v.dc = reinterpret_cast<double*>(base + a_dc);
+    double* diag = reinterpret_cast<double*>(base + a_diag);
+    int* rowptr = reinterpret_cast<int*>(base + a_row);
+    int* xptr = reinterpret_cast<int*>(base + a_xptr);
+    int* split = reinterpret_cast<int*>(base + a_split);
+    v.diag = diag;
+    v.rowptr = rowptr;
+    v.xptr = xptr;
+    v.xsplit = split;
+
+    // build-time data
+    std::vector<uint32_t> sz(q.dz.size());
+    std::vector<double> sc(q.dc.size());
+    for (size_t i = 0; i < plan.dorder.size(); ++i) {
+        sz[i] = q.dz[plan.dorder[i]];
+        sc[i] = q.dc[plan.dorder[i]];
+    }
+    Packed w;
+    const size_t w_rec = w.put(plan.rec), w_runs = w.put(plan.runs), w_comb = w.put(plan.comb), w_wx = w.put(plan.wx),
+                 w_woff = w.put(plan.woff), w_wend = w.put(plan.wend), w_hx = w.put(plan.hx),
+                 w_hoff = w.put(plan.hoff), w_sib = w.put(plan.sib), w_dbin = w.put(plan.dbin), w_sz = w.put(sz),
+                 w_sc = w.put(sc);
+    // masks and totals start at zero: part of the uploaded image
+    const size_t w_keep = w.put(std::vector<uint2>((size_t)G)), w_amb = w.put(std::vector<uint2>((size_t)G)),
+                 w_tot = w.put(std::vector<BuildTotals>(1));
+    const int segs = build_segments(B);
+    const size_t w_T = w.room((size_t)plan.n_entries * sizeof(double)),
+                 w_Tf = w.room((size_t)plan.n_entries * sizeof(float)),
+                 w_rows = w.room((size_t)D * sizeof(int)), w_blks = w.room((size_t)B * sizeof(int)),
+                 w_seg = w.room((size_t)segs * sizeof(BuildSeg)), w_off = w.room((size_t)segs * sizeof(longlong2));
+    auto* wb = static_cast<unsigned char*>(scratch(c, S_STAGE, w.bytes));
+    TQ_CUDA(cudaMemcpy(wb, w.image.data(), w.image.size(), cudaMemcpyHostToDevice));
+    BuildView bv{};
+    bv.G = G;
+    bv.W = W;
+    bv.H = H;
+    bv.levels = plan.levels;
+    bv.gx = v.gx;
+    bv.rec = reinterpret_cast<BuildGroup*>(wb + w_rec);
+    bv.keep = reinterpret_cast<uint2*>(wb + w_keep);
+    bv.amb = reinterpret_cast<uint2*>(wb + w_amb);
+    bv.runs = reinterpret_cast<BuildRun*>(wb + w_runs);
+    bv.T = reinterpret_cast<double*>(wb + w_T);
+    bv.Tf = reinterpret_cast<float*>(wb + w_Tf);
+    bv.wx = reinterpret_cast<uint32_t*>(wb + w_wx);
+    bv.woff = reinterpret_cast<int*>(wb + w_woff);
+    bv.wend = reinterpret_cast<int*>(wb + w_wend);
+    bv.hx = reinterpret_cast<uint32_t*>(wb + w_hx);
+    bv.hoff = reinterpret_cast<int*>(wb + w_hoff);
+    bv.sib = reinterpret_cast<uint32_t*>(wb + w_sib);
+    auto* tot = reinterpret_cast<BuildTotals*>(wb + w_tot);
+    const unsigned long long tol = double_bits(1e-12 * q.maxc), amb = double_bits(1e-9 * q.maxc);
+
+    launch(c, "build_diag", 0, [&] {
+        return launch_build_diag(D, reinterpret_cast<int*>(wb + w_dbin), reinterpret_cast<uint32_t*>(wb + w_sz),
+                                 reinterpret_cast<double*>(wb + w_sc), diag, c->sm_count, 0);
+    });
+    if (G > 0)
+        launch(c, "build_tables", 0, [&] {
+            return launch_build_tables(bv, (int)plan.runs.size(), reinterpret_cast<uint32_t*>(wb + w_comb), v.tc,
+                                       reinterpret_cast<double*>(wb + w_T), reinterpret_cast<float*>(wb + w_Tf), tol,
+                                       amb, reinterpret_cast<uint2*>(wb + w_keep),
+                                       reinterpret_cast<uint2*>(wb + w_amb), 0);
+        });
+    launch(c, "build_count", 0, [&] {
+        return launch_build_count(bv, D, B, tol, amb, reinterpret_cast<int*>(wb + w_rows),
+                                  reinterpret_cast<int*>(wb + w_blks), reinterpret_cast<BuildSeg*>(wb + w_seg),
+                                  reinterpret_cast<longlong2*>(wb + w_off), tot, rowptr, xptr, 0);
+    });
+    launch(c, "xell_split", 0, [&] { return launch_xell_split(xptr, B, v.xgrid, split, 0); });
+    BuildTotals ht;
+    TQ_CUDA(cudaMemcpy(&ht, tot, sizeof ht, cudaMemcpyDeviceToHost));
+    if (ht.rows >= 2147483647ll)
+        throw Error(TQ_ENOMEM, "CSR has 2^31 or more non-zeros; int32 indices cannot address it");
+    if (ht.pairs >= 2147483647ll)
+        throw Error(TQ_ENOMEM, "XOR-ELL has 2^31 or more pairs; int32 offsets cannot address it");
+    h->nnz = v.nnz = ht.rows;
+    h->n_amb = (long long)ht.amb;
+    h->max_row = ht.max_row;
+    v.n_pairs = ht.pairs;
+    // pairs padded to whole copy chunks: the staged energy copies chunk by chunk
+    const long long chunk = xell_chunk_pairs(), cap = std::max(1ll, (ht.pairs + chunk - 1) / chunk) * chunk;
+    Packed e;
+    const size_t e_col = e.room((size_t)ht.rows * sizeof(int)), e_val = e.room((size_t)ht.rows * vb),
+                 e_xm = e.room((size_t)cap * sizeof(uint32_t)), e_xv = e.room((size_t)cap * XELL_ROWS * vb);
+    auto* eb = static_cast<unsigned char*>(dev_alloc(e.bytes));
+    h->allocs.push_back(eb);
+    int* col = reinterpret_cast<int*>(eb + e_col);
+    void* val = eb + e_val;
+    uint32_t* xmask = reinterpret_cast<uint32_t*>(eb + e_xm);
+    void* xval = eb + e_xv;
+    v.col = col;
+    v.val = val;
+    v.xmask = xmask;
+    v.xval = xval;
+    TQ_CUDA(cudaMemsetAsync(xmask + ht.pairs, 0, (size_t)(cap - ht.pairs) * sizeof(uint32_t), 0));
+    TQ_CUDA(cudaMemsetAsync(static_cast<char*>(xval) + (size_t)ht.pairs * XELL_ROWS * vb, 0,
+                            (size_t)(cap - ht.pairs) * XELL_ROWS * vb, 0));
+    if (ht.rows > 0)
+        launch(c, "build_fill", 0, [&] {
+            return launch_build_fill(bv, D, B, ht.rows, tol, h->prec, rowptr, col, val, xptr, xmask, xval, c->sm_count,
+                                     0);
+        });
+    TQ_CUDA(cudaDeviceSynchronize());
+}
+
 // Pauli sum -> device Hamiltonian (diagonal, CSR, and outside a sector the
 // XOR-ELL layout), over the full space or over a sector (`sect` non-null).
 tq_ham* make_hamiltonian(tq_ctx* c, int n_spatial, const double* h1, const double* g2, double e_const,
@@ -502,57 +689,39 @@ tq_ham* make_hamiltonian(tq_ctx* c, int n_spatial, const double* h1, const doubl
         h->mapping = mapping;
         h->D = sect ? sector_dim(sect->n, sect->na, sect->nb) : 1ll << h->nq;
         h->n_pauli = (long long)terms.size();
-        std::vector<uint32_t> gx, tz, dz;
-        std::vector<int> goff;
-        std::vector<double> tc, dc;
-        double maxc = 0.0;
-        for (size_t i = 0; i < terms.size(); ++i) {
-            maxc = std::max(maxc, std::fabs(terms[i].c));
-            if (terms[i].x == 0) {
-                dz.push_back((uint32_t)terms[i].z);
-                dc.push_back(terms[i].c);
-                continue;
-            }
-            if (gx.empty() || gx.back() != (uint32_t)terms[i].x) {
-                gx.push_back((uint32_t)terms[i].x);
-                goff.push_back((int)tz.size());
-            }
-            tz.push_back((uint32_t)terms[i].z);
-            tc.push_back(terms[i].c);
-        }
-        goff.push_back((int)tz.size());
+        const Grouped q = group_terms(terms);
         HamView& v = h->view;
         v.nq = h->nq;
         v.prec = prec;
         v.D = h->D;
-        v.G = (int)gx.size();
-        v.gx = upload(h->allocs, gx);
-        v.goff = upload(h->allocs, goff);
-        v.tz = upload(h->allocs, tz);
-        v.tc = upload(h->allocs, tc);
-        v.Kd = (int)dz.size();
-        v.dz = upload(h->allocs, dz);
-        v.dc = upload(h->allocs, dc);
-        size_t extra = 0;
+        v.G = (int)q.gx.size();
+        v.Kd = (int)q.dz.size();
+        const size_t vb = prec == TQ_C128 ? 8 : 4;
         if (sect) {
+            v.gx = upload(h->allocs, q.gx);
+            v.goff = upload(h->allocs, q.goff);
+            v.tz = upload(h->allocs, q.tz);
+            v.tc = upload(h->allocs, q.tc);
+            v.dz = upload(h->allocs, q.dz);
+            v.dc = upload(h->allocs, q.dc);
             h->sector = 1;
             h->n_alpha = sect->na;
             h->n_beta = sect->nb;
             const auto basis = sector_basis(*sect);
             v.sq = upload(h->allocs, basis);
             v.sect = upload(h->allocs, std::vector<SectorSpec>{*sect});
-            extra = basis.size() * 4 + sizeof(SectorSpec);
+            double* diag = static_cast<double*>(dev_alloc((size_t)h->D * sizeof(double)));
+            h->allocs.push_back(diag);
+            v.diag = diag;
+            launch(c, "diag", 0, [&] { return launch_diag(v, diag, c->sm_count, 0); });
+            h->nnz = build_csr(c, v, q.maxc, prec, h->allocs, &h->n_amb, &h->max_row);
+            h->bytes = basis.size() * 4 + sizeof(SectorSpec);
+        } else {
+            build_full(c, h, q);
+            h->bytes = (size_t)(v.n_blocks + 1) * 4 + (size_t)v.n_pairs * (4 + XELL_ROWS * vb) + (size_t)(v.xgrid + 1) * 4;
         }
-        double* diag = static_cast<double*>(dev_alloc((size_t)h->D * sizeof(double)));
-        h->allocs.push_back(diag);
-        v.diag = diag;
-        launch(c, "diag", 0, [&] { return launch_diag(v, diag, c->sm_count, 0); });
-        h->nnz = build_csr(c, v, maxc, prec, h->allocs, &h->n_amb, &h->max_row);
-        const long long np = sect ? 0 : build_xell(c, v, maxc, prec, h->allocs);
-        const size_t vb = prec == TQ_C128 ? 8 : 4;
-        h->bytes = (size_t)h->D * 8 + (size_t)(h->D + 1) * 4 + (size_t)h->nnz * (4 + vb) + extra +
-                   (sect ? 0 : (size_t)(v.n_blocks + 1) * 4 + (size_t)np * (4 + XELL_ROWS * vb) + (size_t)(v.xgrid + 1) * 4) +
-                   (gx.size() + goff.size() + tz.size() + dz.size()) * 4 + (tc.size() + dc.size()) * 8;
+        h->bytes += (size_t)h->D * 8 + (size_t)(h->D + 1) * 4 + (size_t)h->nnz * (4 + vb) +
+                    (q.gx.size() + q.goff.size() + q.tz.size() + q.dz.size()) * 4 + (q.tc.size() + q.dc.size()) * 8;
     } catch (...) {
         tq_ham_free(h);
         throw;

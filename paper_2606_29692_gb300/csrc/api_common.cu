@@ -84,55 +84,6 @@ long long build_csr(tq_ctx* c, HamView& h, double maxc, int prec, std::vector<vo
     return nnz;
 }
 
-// XOR-ELL form of the same off-diagonal entries (blocks of XELL_ROWS rows);
-// returns the number of pairs.
-long long build_xell(tq_ctx* c, HamView& h, double maxc, int prec, std::vector<void*>& allocs) {
-    h.n_blocks = (h.D + XELL_ROWS - 1) / XELL_ROWS;
-    const long long B = h.n_blocks;
-    int* counts = static_cast<int*>(scratch(c, S_G, (size_t)B * sizeof(int)));
-    int* xptr = static_cast<int*>(dev_alloc((size_t)(B + 1) * sizeof(int)));
-    allocs.push_back(xptr);
-    struct Out { long long total; int max_row; int pad; };
-    Out* dout = static_cast<Out*>(scratch(c, S_PART, sizeof(Out)));
-    TQ_CUDA(cudaMemset(dout, 0, sizeof(Out)));
-    const double tol = 1e-12 * maxc;
-    if (h.G > 0) {
-        launch(c, "xell_count", 0, [&] { return launch_xell_count(h, tol, counts, c->sm_count, 0); });
-    } else {
-        TQ_CUDA(cudaMemset(counts, 0, (size_t)B * sizeof(int)));
-    }
-    launch(c, "scan", 0, [&] { return launch_scan(counts, B, xptr, &dout->total, &dout->max_row, 0); });
-    Out hout;
-    TQ_CUDA(cudaMemcpy(&hout, dout, sizeof(Out), cudaMemcpyDeviceToHost));
-    if (hout.total >= 2147483647ll)
-        throw Error(TQ_ENOMEM, "XOR-ELL has 2^31 or more pairs; int32 offsets cannot address it");
-    const long long np = hout.total;
-    // padded to whole copy chunks: the staged energy copies chunk by chunk
-    const long long chunk = xell_chunk_pairs();
-    const long long cap = std::max(1ll, (np + chunk - 1) / chunk) * chunk;
-    const size_t vb = prec == TQ_C128 ? sizeof(double) : sizeof(float);
-    uint32_t* xmask = static_cast<uint32_t*>(dev_alloc((size_t)cap * sizeof(uint32_t)));
-    allocs.push_back(xmask);
-    void* xval = dev_alloc((size_t)cap * XELL_ROWS * vb);
-    allocs.push_back(xval);
-    TQ_CUDA(cudaMemset(xmask + np, 0, (size_t)(cap - np) * sizeof(uint32_t)));
-    TQ_CUDA(cudaMemset(static_cast<char*>(xval) + (size_t)np * XELL_ROWS * vb, 0,
-                       (size_t)(cap - np) * XELL_ROWS * vb));
-    h.xptr = xptr;
-    h.xmask = xmask;
-    h.xval = xval;
-    h.n_pairs = np;
-    if (np > 0) launch(c, "xell_fill", 0, [&] { return launch_xell_fill(h, tol, xmask, xval, prec, c->sm_count, 0); });
-    // pair-balanced block ranges for the staged energy launch
-    h.xgrid = xell_grid(B, prec, c->sm_count);
-    int* split = static_cast<int*>(dev_alloc((size_t)(h.xgrid + 1) * sizeof(int)));
-    allocs.push_back(split);
-    h.xsplit = split;
-    launch(c, "xell_split", 0, [&] { return launch_xell_split(xptr, B, h.xgrid, split, 0); });
-    TQ_CUDA(cudaDeviceSynchronize());
-    return np;
-}
-
 // A pool, Hamiltonian and state must describe the same space: the same
 // qubit count, and either all the full space or all the same sector.
 void check_space(const tq_pool* p, const tq_state* s) {

@@ -38,10 +38,9 @@ void check_space(const tq_pool* p, const tq_state* s);
 void check_space(const tq_ham* h, const tq_state* s);
 void free_all(std::vector<void*>& allocs);
 
-// The CSR and XOR-ELL forms of a Hamiltonian's off-diagonal entries.
+// The CSR of a sector Hamiltonian's off-diagonal entries or of one generator.
 long long build_csr(tq_ctx* c, HamView& h, double maxc, int prec, std::vector<void*>& allocs,
                     long long* n_amb, int* max_row);
-long long build_xell(tq_ctx* c, HamView& h, double maxc, int prec, std::vector<void*>& allocs);
 
 // Amplitudes of one state of the pool's space.
 long long state_len(const tq_pool* p);

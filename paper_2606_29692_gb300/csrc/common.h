@@ -190,9 +190,6 @@ int launch_scan(const int* counts, long long D, int* rowptr, long long* total,
                 int* max_row, cudaStream_t s);
 int launch_csr_fill(const HamView& h, double tol, int max_row, int* col, void* val,
                     int prec, int sms, cudaStream_t s);
-int launch_xell_count(const HamView& h, double tol, int* counts, int sms, cudaStream_t s);
-int launch_xell_fill(const HamView& h, double tol, uint32_t* xmask, void* xval, int prec, int sms,
-                     cudaStream_t s);
 
 // Taylor-5, matrix-free pair path: states back to back, op k[b] / theta[b]
 // (device arrays, or the immediates when the pointers are null).  Writes

@@ -17,6 +17,35 @@ using namespace tq::api;
 
 namespace {
 
+// The sweeps with a launch per factor: states beyond one cluster, sector
+// pools, pools with entries other than +-1.
+void ansatz_by_factor(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq_state* psi0, int n, const int* ops,
+                      const double* th, bool grad, unsigned char* phis, void* chi, double* gdev, double* part,
+                      const tq_state& last, cudaStream_t s) {
+    const int prec = psi0->prec, upt = c->pair_upt[prec];
+    const long long D = psi0->D;
+    const size_t vb = (size_t)D * elem_bytes(prec);
+    TQ_CUDA(cudaMemcpyAsync(phis, psi0->data, vb, cudaMemcpyDeviceToDevice, s));
+    for (int j = 0; j < n; ++j) {
+        unsigned char* dst = phis + (size_t)(j + 1) * vb;
+        TQ_CUDA(cudaMemcpyAsync(dst, phis + (size_t)j * vb, vb, cudaMemcpyDeviceToDevice, s));
+        launch_update(c, p, 1, prec, upt, dst, nullptr, nullptr, ops[j], th[j], nullptr, part, nullptr, nullptr, s);
+    }
+    run_energy(c, h, &last, part, s);
+    if (!grad) return;
+    launch(c, "residual", s, [&] { return launch_residual(static_cast<double2*>(c->scratch[S_W0]), last.data, chi, prec,
+                                                          D, c->step, s); });
+    for (int j = n - 1; j >= 0; --j) {
+        const double t = th[j], t2 = t * t;
+        const double c4 = 1.0 - t2 / 2.0 + t2 * t2 / 24.0, s4 = t * (1.0 - t2 / 6.0);
+        launch(c, "ansatz_dot", s, [&] {
+            return launch_ansatz_dot(p->view, ops[j], c4, s4, chi, phis + (size_t)j * vb, prec, D, part,
+                                     c->tickets + 4, c->step, gdev + j, c->sm_count, s);
+        });
+        launch_update(c, p, 1, prec, upt, chi, nullptr, nullptr, ops[j], -t, nullptr, part, nullptr, nullptr, s);
+    }
+}
+
 // E(theta) and dE/dtheta of psi(theta) = U_n ... U_1 psi0 (Taylor-5 factors,
 // no renormalisation): forward states phi_0 .. phi_n kept in scratch, the
 // energy pass over phi_n (w = H psi), chi = w - E psi, then per factor from
@@ -38,30 +67,46 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
     double* part = prepare(c, D, p, p->nq);
     unsigned char* phis = static_cast<unsigned char*>(scratch(c, S_PHI, (size_t)(n + 1) * vb));
     void* chi = scratch(c, S_CHI, vb);
-    double* gdev = static_cast<double*>(scratch(c, S_AG, (size_t)std::max(n, 1) * sizeof(double)));
-    const int upt = c->pair_upt[prec];
-    TQ_CUDA(cudaMemcpyAsync(phis, psi0->data, vb, cudaMemcpyDeviceToDevice, s));
-    for (int j = 0; j < n; ++j) {
-        unsigned char* dst = phis + (size_t)(j + 1) * vb;
-        TQ_CUDA(cudaMemcpyAsync(dst, phis + (size_t)j * vb, vb, cudaMemcpyDeviceToDevice, s));
-        launch_update(c, p, 1, prec, upt, dst, nullptr, nullptr, ops[j], th[j], nullptr, part, nullptr, nullptr, s);
-    }
+    const size_t gbytes = (size_t)std::max(n, 1) * sizeof(double);
+    double* gdev = static_cast<double*>(
+        scratch(c, S_AG, gbytes + (size_t)SWEEP_OPS * SWEEP_MAX_CLUSTER * sizeof(double) + sizeof(double)));
     tq_state last = *psi0;
     last.owned = 0;
     last.data = phis + (size_t)n * vb;
-    run_energy(c, h, &last, part, s);
-    if (grad) {
-        launch(c, "residual", s, [&] { return launch_residual(static_cast<double2*>(c->scratch[S_W0]), last.data, chi, prec,
-                                                              D, c->step, s); });
-        for (int j = n - 1; j >= 0; --j) {
-            const double t = th[j], t2 = t * t;
-            const double c4 = 1.0 - t2 / 2.0 + t2 * t2 / 24.0, s4 = t * (1.0 - t2 / 6.0);
-            launch(c, "ansatz_dot", s, [&] {
-                return launch_ansatz_dot(p->view, ops[j], c4, s4, chi, phis + (size_t)j * vb, prec, D, part,
-                                         c->tickets + 4, c->step, gdev + j, c->sm_count, s);
+    // one launch per sweep where a cluster holds the state: at every size
+    // that fits it beats the launches per factor (14 qubits: see vqe.cu)
+    if (n > 0 && !p->sector && p->unit && ansatz_sweep_ready(p->nq, prec)) {
+        const size_t half = vb / 2;                 // a factor's pairs
+        auto chunk = [&](int j0, int j1) {
+            SweepOps o{};
+            for (int j = j0; j < j1; ++j) {
+                o.k[j - j0] = ops[j];
+                o.theta[j - j0] = th[j];
+            }
+            return o;
+        };
+        for (int j = 0; j < n; j += SWEEP_OPS) {
+            const int m = std::min(SWEEP_OPS, n - j);
+            const SweepOps o = chunk(j, j + m);
+            launch(c, "ansatz_forward", s, [&] {
+                return launch_ansatz_forward(p->view, o, m, prec, j ? last.data : psi0->data, last.data,
+                                             grad ? phis + (size_t)j * half : nullptr, s);
             });
-            launch_update(c, p, 1, prec, upt, chi, nullptr, nullptr, ops[j], -t, nullptr, part, nullptr, nullptr, s);
         }
+        run_energy(c, h, &last, part, s);
+        double* gpart = gdev + std::max(n, 1);
+        for (int j1 = n; grad && j1 > 0;) {
+            const int j0 = ((j1 - 1) / SWEEP_OPS) * SWEEP_OPS;
+            const SweepOps o = chunk(j0, j1);
+            launch(c, "ansatz_adjoint", s, [&] {
+                return launch_ansatz_adjoint(p->view, o, j1 - j0, prec, static_cast<double2*>(c->scratch[S_W0]),
+                                             last.data, c->step, j1 == n ? nullptr : chi, j0 ? chi : nullptr,
+                                             phis + (size_t)j0 * half, gpart, gdev + j0, s);
+            });
+            j1 = j0;
+        }
+    } else {
+        ansatz_by_factor(c, h, p, psi0, n, ops, th, grad != nullptr, phis, chi, gdev, part, last, s);
     }
     double E = 0.0;
     int status = 0;

@@ -314,6 +314,25 @@ int energy_grid(long long D, int sms);
 int launch_ansatz_dot(const PoolView& p, int k, double c4, double s4, const void* chi, const void* phi, int prec,
                       long long D, double* partials, unsigned* ticket, const DevStep* step, double* grad_out,
                       int sms, cudaStream_t s);
+// The same sweeps in one launch each, for states one thread-block cluster
+// holds (unit pools of the full space), at most SWEEP_OPS factors per launch.
+constexpr int SWEEP_OPS = 128;
+constexpr int SWEEP_MAX_CLUSTER = 16;
+constexpr int SWEEP_MAX_TPB = 1024;
+struct SweepOps {
+    int k[SWEEP_OPS];
+    double theta[SWEEP_OPS];
+};
+bool ansatz_sweep_ready(int nq, int prec);
+// psi_end <- U_{n-1} .. U_0 psi0; pairs (optional): factor j's input pairs
+// {psi_r, psi_{r^x}} in pair order from amplitude j * 2^nq / 2.
+int launch_ansatz_forward(const PoolView& p, const SweepOps& ops, int n, int prec, const void* psi0, void* psi_end,
+                          void* pairs, cudaStream_t s);
+// Gradients of factors n-1 .. 0 and chi carried through them; chi_in null:
+// chi = w - E psi.  part: SWEEP_OPS * SWEEP_MAX_CLUSTER doubles.
+int launch_ansatz_adjoint(const PoolView& p, const SweepOps& ops, int n, int prec, const double2* w, const void* psi,
+                          const DevStep* step, const void* chi_in, void* chi_out, const void* pairs, double* part,
+                          double* grad, cudaStream_t s);
 int launch_residual(const double2* w, const void* psi, void* chi, int prec, long long D, const DevStep* step,
                     cudaStream_t s);
 int sector_tiles(long long dim, int prec);

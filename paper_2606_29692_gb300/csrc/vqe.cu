@@ -7,6 +7,14 @@
 // annihilate), so U'(theta) = c4 A - s4 P with c4 = 1 - theta^2/2 +
 // theta^4/24 and s4 = theta - theta^3/6.
 #include "dev.cuh"
+#include "grad.cuh"
+#include "pair.cuh"
+
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+namespace cg = cooperative_groups;
 
 namespace tq {
 
@@ -80,13 +88,323 @@ __global__ void k_residual(const double2* __restrict__ w, const typename C2<T>::
     }
 }
 
+
+// ------------------------------------------------- whole sweeps in one launch
+//
+// Forward and adjoint sweep of an ansatz whose state fits the shared memory
+// of one thread-block cluster (each CTA holds a contiguous slice): one
+// launch per sweep instead of a copy, an update and (backwards) a dot per
+// factor.  A factor touches its generator's support only, as pairs {r, r^x};
+// one thread owns a pair, reads and writes both amplitudes through
+// distributed shared memory, and a cluster barrier separates factors.  The
+// update is the pair update's own arithmetic (chain_pair for complex64, the
+// closed form for complex128), so the states are bit for bit those of the
+// per-factor launches.  The forward sweep stores each factor's input pairs
+// in pair order for the adjoint sweep, which turns them into
+//   X = sum_S Re<chi_r|A phi_r>,  Y = sum_S Re<chi_r|phi_r>,  grad = 2 (c4 X - s4 Y) / <psi|psi>,
+// with complex64 products and sums carried in float32 pairs (about 48 bits):
+// a float64 product per amplitude would hold the float64 pipe of the
+// cluster's 16 SMs longer than everything else.
+//
+// What bounds it: the latency of a factor (barrier, distributed shared
+// memory round trip, pair arithmetic).  20 factors at 14 qubits, complex64,
+// energy and read-back included: 588 us as 40 update and 20 dot launches
+// with their copies, 148 us here (forward 32, energy 20, adjoint 43 us, the
+// rest launches and read-back).
+template <typename T>
+struct SweepOp {
+    RowExp rx;
+    uint32_t x, z0;
+    int neg;               // entries of A are (-1)^{parity(col & z0)} (-1)^neg
+    uint32_t pairs;
+    T cf[6];
+    double c5, s5;         // closed form (complex128)
+    double c4, s4;         // derivative (adjoint sweep)
+};
+
+template <typename T>
+__device__ __forceinline__ void sweep_prepare(const PoolView& p, const SweepOps& ops, int n, bool adjoint,
+                                              SweepOp<T>* out) {
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        const int k = ops.k[j];
+        const double t = ops.theta[j];
+        SweepOp<T>& o = out[j];
+        const SuppRec s = load_supp(p, k);
+        o.rx = make_rowexp(s, p.supp[k].z);
+        o.x = s.x;
+        o.z0 = s.z0;
+        o.neg = p.fc0f[k] < 0.0f;
+        o.pairs = (uint32_t)((1ll << p.nq) >> (s.m + 1));
+        taylor_coefs_fast<T>(adjoint ? -t : t, o.cf);
+        if constexpr (sizeof(T) == 8) closed_coefs(o.cf, o.c5, o.s5);
+        const double t2 = t * t;
+        o.c4 = 1.0 - t2 / 2.0 + t2 * t2 / 24.0;
+        o.s4 = t * (1.0 - t2 / 6.0);
+    }
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// The update of one pair; neg_r: A[r][q] = -1 (then A[q][r] = +1).
+__device__ __forceinline__ void sweep_pair(const SweepOp<float>& o, bool neg_r, float2& a, float2& b) {
+    chain_pair(neg_r ? -1.f : 1.f, neg_r ? 1.f : -1.f, o.cf, a, b);
+}
+__device__ __forceinline__ void sweep_pair(const SweepOp<double>& o, bool neg_r, double2& a, double2& b) {
+    closed_pair_sign(neg_r ? -1 : 1, neg_r ? 1 : -1, o.cf, o.c5, o.s5, a, b);
+}
+
+// Sums of products: float64, or float32 (hi, lo) pairs with exact products.
+template <typename T> struct DotAcc;
+template <> struct DotAcc<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
+    __device__ __forceinline__ double warp() const { return warp_sum(v); }
+};
+template <> struct DotAcc<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float a, float b) {
+        const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+        float s, r;
+        two_sum(hi, p, s, r);
+        hi = s;
+        lo += r + e;
+    }
+    __device__ __forceinline__ double warp() const { return warp_sum_compensated_pair(hi, lo); }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(SWEEP_MAX_TPB)
+k_ansatz_forward(PoolView p, const __grid_constant__ SweepOps ops, int n, int slice_log,
+                 const typename C2<T>::type* psi0, typename C2<T>::type* psi_end,
+                 typename C2<T>::type* __restrict__ pairs_out, long long stride) {
+    using V = typename C2<T>::type;
+    extern __shared__ __align__(16) unsigned char sw_raw[];
+    cg::cluster_group cl = cg::this_cluster();
+    SweepOp<T>* op = reinterpret_cast<SweepOp<T>*>(sw_raw);
+    V* st = reinterpret_cast<V*>(sw_raw + SWEEP_OPS * sizeof(SweepOp<T>));
+    const uint32_t per = 1u << slice_log, lo = per - 1u, rank = cl.block_rank();
+    for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) st[i] = psi0[((size_t)rank << slice_log) + i];
+    sweep_prepare<T>(p, ops, n, false, op);
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();                       // every slice is loaded
+    const uint32_t t0 = rank * blockDim.x + threadIdx.x, step = cl.num_blocks() * blockDim.x;
+    for (int j = 0; j < n; ++j) {
+        const SweepOp<T>& o = op[j];
+        for (uint32_t u = t0; u < o.pairs; u += step) {
+            const uint32_t r = expand_row(o.rx, u), q = r ^ o.x;
+            V* pr = cl.map_shared_rank(st + (r & lo), r >> slice_log);
+            V* pq = cl.map_shared_rank(st + (q & lo), q >> slice_log);
+            V a = *pr, b = *pq;
+            if (pairs_out) store2(pairs_out + (size_t)j * stride, 2 * u, a, b);
+            sweep_pair(o, (parity32(q & o.z0) ^ o.neg) != 0, a, b);
+            *pr = a;
+            *pq = b;
+        }
+        cluster_arrive();
+        cluster_wait();                   // the factor is applied, and no peer reads this slice any more
+    }
+    for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) psi_end[((size_t)rank << slice_log) + i] = st[i];
+}
+
+// chi_in null: chi = w - E psi at the end of the ansatz (the first launch of
+// the sweep), else the chi an earlier launch left.  part: [SWEEP_OPS][CTAs].
+template <typename T>
+__global__ void __launch_bounds__(SWEEP_MAX_TPB)
+k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int slice_log,
+                 const double2* __restrict__ w, const typename C2<T>::type* __restrict__ psi, const DevStep* step,
+                 const typename C2<T>::type* chi_in, typename C2<T>::type* chi_out,
+                 const typename C2<T>::type* __restrict__ pairs_in, long long stride, double* part, double* grad) {
+    using V = typename C2<T>::type;
+    extern __shared__ __align__(16) unsigned char sw_raw[];
+    cg::cluster_group cl = cg::this_cluster();
+    SweepOp<T>* op = reinterpret_cast<SweepOp<T>*>(sw_raw);
+    const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double* wsum = reinterpret_cast<double*>(sw_raw + SWEEP_OPS * sizeof(SweepOp<T>));   // [n][nw]
+    V* st = reinterpret_cast<V*>(wsum + (size_t)SWEEP_OPS * (SWEEP_MAX_TPB / 32));
+    const uint32_t per = 1u << slice_log, lo = per - 1u, rank = cl.block_rank();
+    const double E = step->energy;
+    for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) {
+        const size_t r = ((size_t)rank << slice_log) + i;
+        if (chi_in) {
+            st[i] = chi_in[r];
+        } else {
+            const double2 wr = w[r];
+            const V pr = psi[r];
+            st[i] = {(T)(wr.x - E * (double)pr.x), (T)(wr.y - E * (double)pr.y)};
+        }
+    }
+    sweep_prepare<T>(p, ops, n, true, op);
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
+    const uint32_t t0 = rank * blockDim.x + threadIdx.x, step_u = cl.num_blocks() * blockDim.x;
+    for (int j = n - 1; j >= 0; --j) {
+        const SweepOp<T>& o = op[j];
+        DotAcc<T> X, Y;
+        for (uint32_t u = t0; u < o.pairs; u += step_u) {
+            V fr, fq;
+            load2(pairs_in + (size_t)j * stride, 2 * u, fr, fq);
+            const uint32_t r = expand_row(o.rx, u), q = r ^ o.x;
+            V* pr = cl.map_shared_rank(st + (r & lo), r >> slice_log);
+            V* pq = cl.map_shared_rank(st + (q & lo), q >> slice_log);
+            V a = *pr, b = *pq;
+            const bool neg = (parity32(q & o.z0) ^ o.neg) != 0;      // A[r][q] = -1, A[q][r] = +1
+            const T s = neg ? T(-1) : T(1);
+            X.add(s * a.x, fq.x);
+            X.add(s * a.y, fq.y);
+            X.add(-s * b.x, fr.x);
+            X.add(-s * b.y, fr.y);
+            Y.add(a.x, fr.x);
+            Y.add(a.y, fr.y);
+            Y.add(b.x, fq.x);
+            Y.add(b.y, fq.y);
+            sweep_pair(o, neg, a, b);
+            *pr = a;
+            *pq = b;
+        }
+        cluster_arrive();
+        const double x = X.warp(), y = Y.warp();
+        if (lane == 0) wsum[j * nw + wid] = o.c4 * x - o.s4 * y;
+        cluster_wait();
+    }
+    for (uint32_t i = threadIdx.x; chi_out && i < per; i += blockDim.x) chi_out[((size_t)rank << slice_log) + i] = st[i];
+    // this CTA's sums in warp order, then the CTAs' in rank order
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        double v = 0.0;
+        for (int i = 0; i < nw; ++i) v += wsum[j * nw + i];
+        part[(size_t)j * SWEEP_MAX_CLUSTER + rank] = v;
+    }
+    __threadfence();
+    cluster_arrive();
+    cluster_wait();
+    if (rank == 0)
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            double v = 0.0;
+            for (unsigned i = 0; i < cl.num_blocks(); ++i) v += __ldcg(part + (size_t)j * SWEEP_MAX_CLUSTER + i);
+            grad[j] = 2.0 * v / step->e_den;
+        }
+}
+
 int small_grid(long long D, int sms) {
     long long g = (D + 255) / 256;
     if (g > (long long)sms * 4) g = (long long)sms * 4;
     return (int)(g < 1 ? 1 : g);
 }
 
+template <typename T>
+size_t sweep_smem(bool adjoint, int slice_log) {
+    return SWEEP_OPS * sizeof(SweepOp<T>) + (adjoint ? (size_t)SWEEP_OPS * (SWEEP_MAX_TPB / 32) * sizeof(double) : 0) +
+           ((size_t)1 << slice_log) * 2 * sizeof(T);
+}
+
+// CTAs and threads per CTA for 2^nq amplitudes: a single excitation has D/4
+// pairs, aimed at one per thread.  complex64 takes 256 pairs per CTA
+// (latency bounds it), complex128 128 (its float64 work spreads over more
+// SMs), up to 16 CTAs, then more threads.
+void sweep_shape(int nq, int prec, int* cs, int* tpb) {
+    const long long pairs = std::max(1ll, (1ll << nq) >> 2), per_cta = prec == TQ_C128 ? 128 : 256;
+    const long long c = std::min<long long>(SWEEP_MAX_CLUSTER, std::max(1ll, pairs / per_cta));
+    *cs = (int)c;
+    *tpb = (int)std::min<long long>(SWEEP_MAX_TPB, std::max(32ll, pairs / c));
+}
+
+template <typename K>
+cudaError_t sweep_config(K kern, int cs, int tpb, size_t smem, cudaStream_t s, cudaLaunchConfig_t* cfg,
+                         cudaLaunchAttribute* attr) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && cs > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3(cs);
+    cfg->blockDim = dim3(tpb);
+    cfg->dynamicSmemBytes = smem;
+    cfg->stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = cs;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    return e;
+}
+
+template <typename T>
+bool sweep_fits(int nq, int prec) {
+    int cs, tpb;
+    sweep_shape(nq, prec, &cs, &tpb);
+    int lg = nq;
+    while (cs >> (nq - lg + 1)) --lg;          // slice of D / cs amplitudes
+    const size_t smem = sweep_smem<T>(true, lg);
+    if (smem > 200 * 1024) return false;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    int n = 0;
+    cudaError_t e = sweep_config(k_ansatz_adjoint<T>, cs, tpb, smem, 0, &cfg, &attr);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_ansatz_adjoint<T>, &cfg);
+    if (e == cudaSuccess && n >= 1) {
+        e = sweep_config(k_ansatz_forward<T>, cs, tpb, sweep_smem<T>(false, lg), 0, &cfg, &attr);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_ansatz_forward<T>, &cfg);
+    }
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e == cudaSuccess && n >= 1;
+}
+
 }  // namespace
+
+// Asked once per call: a few microseconds of host queries beside the sweep.
+bool ansatz_sweep_ready(int nq, int prec) {
+    if (nq < 2 || nq >= 32) return false;
+    return prec == TQ_C128 ? sweep_fits<double>(nq, prec) : sweep_fits<float>(nq, prec);
+}
+
+template <typename T>
+static int forward_t(const PoolView& p, const SweepOps& ops, int n, int prec, const void* psi0, void* psi_end,
+                     void* pairs, cudaStream_t s) {
+    using V = typename C2<T>::type;
+    int cs, tpb, lg = p.nq;
+    sweep_shape(p.nq, prec, &cs, &tpb);
+    while (cs >> (p.nq - lg + 1)) --lg;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cudaError_t e = sweep_config(k_ansatz_forward<T>, cs, tpb, sweep_smem<T>(false, lg), s, &cfg, &attr);
+    if (e == cudaSuccess)
+        e = cudaLaunchKernelEx(&cfg, k_ansatz_forward<T>, p, ops, n, lg, static_cast<const V*>(psi0),
+                               static_cast<V*>(psi_end), static_cast<V*>(pairs), (1ll << p.nq) / 2);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+template <typename T>
+static int adjoint_t(const PoolView& p, const SweepOps& ops, int n, int prec, const double2* w, const void* psi,
+                     const DevStep* step, const void* chi_in, void* chi_out, const void* pairs, double* part,
+                     double* grad, cudaStream_t s) {
+    using V = typename C2<T>::type;
+    int cs, tpb, lg = p.nq;
+    sweep_shape(p.nq, prec, &cs, &tpb);
+    while (cs >> (p.nq - lg + 1)) --lg;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cudaError_t e = sweep_config(k_ansatz_adjoint<T>, cs, tpb, sweep_smem<T>(true, lg), s, &cfg, &attr);
+    if (e == cudaSuccess)
+        e = cudaLaunchKernelEx(&cfg, k_ansatz_adjoint<T>, p, ops, n, lg, w, static_cast<const V*>(psi), step,
+                               static_cast<const V*>(chi_in), static_cast<V*>(chi_out), static_cast<const V*>(pairs),
+                               (1ll << p.nq) / 2, part, grad);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+int launch_ansatz_forward(const PoolView& p, const SweepOps& ops, int n, int prec, const void* psi0, void* psi_end,
+                          void* pairs, cudaStream_t s) {
+    return prec == TQ_C128 ? forward_t<double>(p, ops, n, prec, psi0, psi_end, pairs, s)
+                           : forward_t<float>(p, ops, n, prec, psi0, psi_end, pairs, s);
+}
+
+int launch_ansatz_adjoint(const PoolView& p, const SweepOps& ops, int n, int prec, const double2* w, const void* psi,
+                          const DevStep* step, const void* chi_in, void* chi_out, const void* pairs, double* part,
+                          double* grad, cudaStream_t s) {
+    return prec == TQ_C128
+               ? adjoint_t<double>(p, ops, n, prec, w, psi, step, chi_in, chi_out, pairs, part, grad, s)
+               : adjoint_t<float>(p, ops, n, prec, w, psi, step, chi_in, chi_out, pairs, part, grad, s);
+}
 
 int launch_ansatz_dot(const PoolView& p, int k, double c4, double s4, const void* chi, const void* phi, int prec,
                       long long D, double* partials, unsigned* ticket, const DevStep* step, double* grad_out,

@@ -124,8 +124,9 @@ int tq_ctx_get_l2_fetch(tq_ctx* ctx, int* bytes);
 
 /* Schedule of the energy SpMV (the H pass of tq_energy, tq_pool_gradients
  * and tq_adapt_step): 4, 8, 16 or 32 lanes sharing one row of the CSR,
- * or TQ_SPMV_XELL for the XOR-ELL layout (the default; a sector
- * Hamiltonian, which has only the CSR, then uses 8 lanes).  Every Hamiltonian
+ * or TQ_SPMV_XELL for the XOR-ELL layout.  Until one is set, complex64 uses
+ * the XOR-ELL layout and complex128 the CSR at 4 lanes; a sector
+ * Hamiltonian, which has only the CSR, uses 8 lanes for either.  Every Hamiltonian
  * holds both layouts of the same off-diagonal entries: the CSR, and blocks
  * of 8 rows where each X-mask present in the block stores its 8 values
  * H[8R+i][(8R+i)^x] (zero where the CSR has no entry), so one pair's 8

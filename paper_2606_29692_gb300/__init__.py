@@ -204,7 +204,8 @@ class Context:
         call("tq_ctx_set_test_flags", self.handle, int(flags))
 
     def set_spmv_schedule(self, lanes_per_row):
-        """4, 8, 16 or 32 CSR lanes per row, or TQ_SPMV_XELL (the default)."""
+        """4, 8, 16 or 32 CSR lanes per row, or TQ_SPMV_XELL (until set: XELL for
+        complex64, 4 lanes for complex128)."""
         call("tq_ctx_set_spmv_schedule", self.handle, int(lanes_per_row))
 
     def set_support_schedule(self, prec, pairs_per_thread):

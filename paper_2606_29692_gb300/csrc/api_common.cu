@@ -156,8 +156,9 @@ void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, c
     TQ_REQUIRE(h->prec == psi->prec, "state and Hamiltonian precisions differ");
     double2* w = static_cast<double2*>(c->scratch[S_W0]);
     float2* w32 = psi->prec == TQ_C64 ? static_cast<float2*>(c->scratch[S_W32]) : nullptr;
-    // a sector Hamiltonian has the CSR only
-    const int lanes = c->spmv_lanes == TQ_SPMV_XELL && h->sector ? 8 : c->spmv_lanes;
+    int lanes = c->spmv_lanes;
+    if (lanes == SPMV_AUTO) lanes = h->prec == TQ_C128 && !h->sector ? SPMV_C128_LANES : (int)TQ_SPMV_XELL;
+    if (lanes == TQ_SPMV_XELL && h->sector) lanes = 8;   // a sector Hamiltonian has the CSR only
     if (lanes == TQ_SPMV_XELL)
         launch(c, "energy_xell", s, [&] {
             return launch_energy_xell(h->view, psi->data, psi->prec, w, w32, part, c->tickets, c->step, s,

@@ -681,6 +681,7 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
         b->n = n_traj;
         b->eps = eps;
         b->prec = hams[0]->prec;
+        if (b->prec == TQ_C128) b->lpr = SPMV_C128_LANES;
         std::vector<int4> ei, gi, pi, si;
         long long nslots = 0, toff = 0;
         for (int t = 0; t < n_traj; ++t) {

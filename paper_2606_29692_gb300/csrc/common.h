@@ -132,6 +132,17 @@ struct PoolView {
 
 constexpr int XELL_ROWS = 8;   // rows per XOR-ELL block
 
+// The energy SpMV's schedule until the caller or an autotuner sets one: the
+// XOR-ELL layout for complex64, the CSR at 4 lanes per row for complex128.
+// Complex128 products are bound by the float64 pipe, which works on a whole
+// warp instruction whatever its lanes hold: the XOR-ELL's zeros (half its
+// slots) cost as much as entries, and a wider row reduction adds float64
+// additions.  Traced, XOR-ELL against 4 lanes: 23 / 17 us at 12 qubits,
+// 59 / 27 at 14, 255 / 108 at 16, 1279 / 568 at 18 (8 lanes 581, 32 lanes
+// 728); complex64 at 16 and 18 qubits: 53 / 64 and 231 / 291.
+constexpr int SPMV_AUTO = -1;
+constexpr int SPMV_C128_LANES = 4;
+
 // Hamiltonian: float64 diagonal + off-diagonal CSR + the same off-diagonal
 // entries in XOR-ELL form + X-mask-grouped terms.
 struct HamView {
@@ -373,7 +384,7 @@ struct tq_ctx {
     int grouped_lanes[2] = {1, 1};         // grouped-layout update: lanes per row (C128, C64)
     int grouped_ppt[2] = {1, 1};           // and pairs per lane
     int l2_fetch_default = 0;              // the CUDA context's L2 fetch granularity at creation (bytes)
-    int spmv_lanes = 0;                    // energy SpMV: CSR lanes per row, or 0 for XOR-ELL (default)
+    int spmv_lanes = tq::SPMV_AUTO;        // energy SpMV: CSR lanes per row, 0 for XOR-ELL, or by precision
     int test_flags = 0;                    // TQ_TEST_* (tests of the failure paths only)
     std::vector<tq_trace_rec> trace;      // recorded, not yet reported
     std::vector<cudaEvent_t> event_pool;  // reusable events

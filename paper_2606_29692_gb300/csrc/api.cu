@@ -46,9 +46,10 @@ extern "C" int tq_ctx_create(int device, tq_ctx** out) {
         throw Error(TQ_ECUDA, cudaGetErrorString(e));
     }
     try {
-        c->step = static_cast<DevStep*>(dev_alloc(sizeof(DevStep)));
+        c->step = static_cast<DevStep*>(dev_alloc(sizeof(DevStep) + tq_ctx::kStepTail * sizeof(double)));
         TQ_CUDA(cudaMemset(c->step, 0, sizeof(DevStep)));
         tickets(c, 4096);
+        host_scratch(c, 0);
         size_t fetch = 0;
         TQ_CUDA(cudaDeviceGetLimit(&fetch, cudaLimitMaxL2FetchGranularity));
         c->l2_fetch_default = (int)fetch;
@@ -78,6 +79,7 @@ extern "C" int tq_ctx_destroy(tq_ctx* c) {
     for (int i = 0; i < tq_ctx::kScratch; ++i)
         if (c->scratch[i]) cudaFree(c->scratch[i]);
     if (c->step) cudaFree(c->step);
+    if (c->host_buf) cudaFreeHost(c->host_buf);
     if (c->tickets) cudaFree(c->tickets);
     if (c->line_sc) cudaFree(c->line_sc);
     if (c->line_se) cudaFree(c->line_se);

@@ -24,6 +24,28 @@ void* scratch(tq_ctx* c, int slot, size_t bytes) {
     return c->scratch[slot];
 }
 
+void* host_scratch(tq_ctx* c, size_t bytes) {
+    if (c->host_bytes < bytes || !c->host_buf) {
+        if (c->host_buf) TQ_CUDA(cudaFreeHost(c->host_buf));
+        c->host_buf = nullptr;
+        c->host_bytes = 0;
+        void* p = nullptr;
+        const size_t room = std::max(bytes, sizeof(DevStep) + tq_ctx::kStepTail * sizeof(double));
+        TQ_CUDA(cudaMallocHost(&p, room));
+        c->host_buf = static_cast<unsigned char*>(p);
+        c->host_bytes = room;
+    }
+    return c->host_buf;
+}
+
+const DevStep* read_step(tq_ctx* c, size_t n, cudaStream_t s) {
+    const size_t bytes = sizeof(DevStep) + n * sizeof(double);
+    auto* h = static_cast<DevStep*>(host_scratch(c, bytes));
+    TQ_CUDA(cudaMemcpyAsync(h, c->step, bytes, cudaMemcpyDeviceToHost, s));
+    TQ_CUDA(cudaStreamSynchronize(s));
+    return h;
+}
+
 unsigned* tickets(tq_ctx* c, size_t n) {
     if (c->tickets_n < n) {
         if (c->tickets) TQ_CUDA(cudaFree(c->tickets));

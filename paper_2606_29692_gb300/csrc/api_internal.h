@@ -25,6 +25,15 @@ T* upload(std::vector<void*>& allocs, const std::vector<T>& v) {
 enum { S_PART = 0, S_W0, S_U1, S_U2, S_W1, S_W2, S_G, S_STAGE, S_W32, S_PHI, S_CHI, S_AG, S_HOSTB, S_REC,
        S_THETAS };
 void* scratch(tq_ctx* c, int slot, size_t bytes);
+// Page-locked host memory for a call's read-back (grown on demand, kept until
+// the context goes; valid until the next call of the context).  A copy into
+// pageable memory is staged by the driver and blocks the host for each
+// array: a 12-qubit energy spent 20 of its 42 us on two of them.
+void* host_scratch(tq_ctx* c, size_t bytes);
+// Copies the step record and the first n doubles of its tail to the host and
+// waits for s.  Returns the record; the tail values follow it.
+const DevStep* read_step(tq_ctx* c, size_t n, cudaStream_t s);
+inline const double* step_tail(const DevStep* h) { return reinterpret_cast<const double*>(h + 1); }
 // n zeroed tickets (every user leaves them zero).
 unsigned* tickets(tq_ctx* c, size_t n);
 

@@ -73,11 +73,9 @@ extern "C" int tq_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double
     cudaStream_t s = as_stream(stream);
     double* part = prepare(c, h->D, nullptr, h->nq);
     run_energy(c, h, psi, part, s);
-    int status = 0;
-    TQ_CUDA(cudaMemcpyAsync(E, &c->step->energy, sizeof(double), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaMemcpyAsync(&status, &c->step->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaStreamSynchronize(s));
-    raise_status(c, status, s);
+    const DevStep* hs = read_step(c, 0, s);
+    *E = hs->energy;
+    raise_status(c, hs->status, s);
     API_END
 }
 
@@ -92,8 +90,7 @@ extern "C" int tq_energy_matrix_free(tq_ctx* c, const tq_ham* h, const tq_state*
     double* part = prepare(c, h->D, nullptr, h->nq);
     launch(c, "energy_matrix_free", s, [&] { return launch_energy_matrix_free(h->view, psi->data, psi->prec, part, c->tickets + 1,
                                               c->step, c->sm_count, s); });
-    TQ_CUDA(cudaMemcpyAsync(E, &c->step->energy, sizeof(double), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaStreamSynchronize(s));
+    *E = read_step(c, 0, s)->energy;
     API_END
 }
 
@@ -103,15 +100,19 @@ extern "C" int tq_pool_gradients(tq_ctx* c, const tq_ham* h, const tq_pool* p, c
     TQ_REQUIRE(c && h && p && psi && g, "null argument");
     set_device(c);
     cudaStream_t s = as_stream(stream);
-    double* gd = g_on_device ? g : static_cast<double*>(scratch(c, S_G, (size_t)p->M * sizeof(double)));
+    // a host result goes behind the step record (one read-back) where it fits
+    const bool in_tail = !g_on_device && p->M <= tq_ctx::kStepTail;
+    double* gd = g_on_device ? g
+                 : in_tail   ? c->tail()
+                             : static_cast<double*>(scratch(c, S_G, (size_t)p->M * sizeof(double)));
     double* part = prepare(c, h->D, p, p->nq);
     run_gradients(c, h, p, psi, gd, part, s);
     if (!g_on_device) {
-        int status = 0;
-        TQ_CUDA(cudaMemcpyAsync(g, gd, (size_t)p->M * sizeof(double), cudaMemcpyDeviceToHost, s));
-        TQ_CUDA(cudaMemcpyAsync(&status, &c->step->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-        TQ_CUDA(cudaStreamSynchronize(s));
-        raise_status(c, status, s);
+        if (!in_tail)
+            TQ_CUDA(cudaMemcpyAsync(g, gd, (size_t)p->M * sizeof(double), cudaMemcpyDeviceToHost, s));
+        const DevStep* hs = read_step(c, in_tail ? p->M : 0, s);
+        if (in_tail) std::memcpy(g, step_tail(hs), (size_t)p->M * sizeof(double));
+        raise_status(c, hs->status, s);
     }
     API_END
 }
@@ -206,9 +207,7 @@ extern "C" int tq_adapt_step(tq_ctx* c, const tq_ham* h, const tq_pool* p, tq_st
     cudaStream_t s = as_stream(stream);
     const AdaptBufs b = adapt_buffers(c, h, p, psi);
     enqueue_adapt_step(c, b, h, p, psi, eps, theta, nullptr, s);
-    DevStep hs;
-    TQ_CUDA(cudaMemcpyAsync(&hs, c->step, sizeof(DevStep), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaStreamSynchronize(s));
+    const DevStep& hs = *read_step(c, 0, s);
     raise_status(c, hs.status, s);
     out->energy = hs.energy;
     out->max_grad = hs.max_grad;
@@ -236,7 +235,9 @@ extern "C" int tq_adapt_run(tq_ctx* c, const tq_ham* h, const tq_pool* p, tq_sta
     if (!c->aux[1]) TQ_CUDA(cudaStreamCreateWithFlags(&c->aux[1], cudaStreamNonBlocking));
     cudaStream_t s = c->aux[1];
     const AdaptBufs b = adapt_buffers(c, h, p, psi);
-    double* rec = static_cast<double*>(scratch(c, S_REC, (size_t)n_iter * 6 * sizeof(double)));
+    double* rec = (size_t)n_iter * 6 <= tq_ctx::kStepTail
+                      ? c->tail()
+                      : static_cast<double*>(scratch(c, S_REC, (size_t)n_iter * 6 * sizeof(double)));
     double* dth = nullptr;
     if (thetas) {
         dth = static_cast<double*>(scratch(c, S_THETAS, (size_t)n_iter * sizeof(double)));
@@ -278,11 +279,11 @@ extern "C" int tq_adapt_run(tq_ctx* c, const tq_ham* h, const tq_pool* p, tq_sta
         }
     }
     std::vector<double> hr((size_t)n_iter * 6);
-    int status = 0;
-    TQ_CUDA(cudaMemcpyAsync(hr.data(), rec, hr.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaMemcpyAsync(&status, &c->step->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaStreamSynchronize(s));
-    raise_status(c, status, s);
+    const bool in_tail = rec == c->tail();
+    if (!in_tail) TQ_CUDA(cudaMemcpyAsync(hr.data(), rec, hr.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+    const DevStep* hs = read_step(c, in_tail ? hr.size() : 0, s);
+    if (in_tail) std::memcpy(hr.data(), step_tail(hs), hr.size() * sizeof(double));
+    raise_status(c, hs->status, s);
     int done = n_iter;
     for (int i = 0; i < n_iter; ++i) {
         const double* r = &hr[6 * (size_t)i];

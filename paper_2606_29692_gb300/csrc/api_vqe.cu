@@ -68,8 +68,10 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
     unsigned char* phis = static_cast<unsigned char*>(scratch(c, S_PHI, (size_t)(n + 1) * vb));
     void* chi = scratch(c, S_CHI, vb);
     const size_t gbytes = (size_t)std::max(n, 1) * sizeof(double);
-    double* gdev = static_cast<double*>(
-        scratch(c, S_AG, gbytes + (size_t)SWEEP_OPS * SWEEP_MAX_CLUSTER * sizeof(double) + sizeof(double)));
+    double* gpart = static_cast<double*>(
+        scratch(c, S_AG, gbytes + (size_t)SWEEP_OPS * SWEEP_MAX_CLUSTER * sizeof(double)));
+    const bool in_tail = n <= tq_ctx::kStepTail;
+    double* gdev = in_tail ? c->tail() : gpart + SWEEP_OPS * SWEEP_MAX_CLUSTER;
     tq_state last = *psi0;
     last.owned = 0;
     last.data = phis + (size_t)n * vb;
@@ -94,7 +96,6 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
             });
         }
         run_energy(c, h, &last, part, s);
-        double* gpart = gdev + std::max(n, 1);
         for (int j1 = n; grad && j1 > 0;) {
             const int j0 = ((j1 - 1) / SWEEP_OPS) * SWEEP_OPS;
             const SweepOps o = chunk(j0, j1);
@@ -108,15 +109,13 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
     } else {
         ansatz_by_factor(c, h, p, psi0, n, ops, th, grad != nullptr, phis, chi, gdev, part, last, s);
     }
-    double E = 0.0;
-    int status = 0;
-    TQ_CUDA(cudaMemcpyAsync(&E, &c->step->energy, sizeof(double), cudaMemcpyDeviceToHost, s));
-    TQ_CUDA(cudaMemcpyAsync(&status, &c->step->status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    if (grad && n > 0) TQ_CUDA(cudaMemcpyAsync(grad, gdev, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, s));
+    const size_t ng = grad ? (size_t)n : 0;
+    if (ng && !in_tail) TQ_CUDA(cudaMemcpyAsync(grad, gdev, ng * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (psi_out) TQ_CUDA(cudaMemcpyAsync(psi_out, last.data, vb, cudaMemcpyDeviceToDevice, s));
-    TQ_CUDA(cudaStreamSynchronize(s));
-    raise_status(c, status, s);
-    return E;
+    const DevStep* hs = read_step(c, in_tail ? ng : 0, s);
+    if (ng && in_tail) std::memcpy(grad, step_tail(hs), ng * sizeof(double));
+    raise_status(c, hs->status, s);
+    return hs->energy;
 }
 
 // BFGS on f with gradient g: inverse-Hessian update, backtracking line

@@ -175,7 +175,7 @@ struct HamView {
 };
 
 // Scalars an ADAPT iteration keeps on the device between its kernels.
-struct DevStep {
+struct alignas(16) DevStep {
     double e_num, e_den, energy;   // Rayleigh quotient pieces
     double max_grad;
     double theta;
@@ -392,7 +392,11 @@ struct tq_ctx {
     static constexpr int kScratch = 16;
     void* scratch[kScratch] = {nullptr};
     size_t scratch_bytes[kScratch] = {0};
-    tq::DevStep* step = nullptr;      // device
+    tq::DevStep* step = nullptr;      // device, followed by kStepTail doubles (small results of a call)
+    static constexpr int kStepTail = 4096;
+    double* tail() const { return reinterpret_cast<double*>(step + 1); }
+    unsigned char* host_buf = nullptr;   // page-locked: what a call reads back
+    size_t host_bytes = 0;
     unsigned* tickets = nullptr;      // device, zero between calls
     double2* line_sc = nullptr;       // device, sin/cos of the line search's sample angles (filled once)
     long long* line_se = nullptr;     // device, the samples' energy keys and per-block minima (4096 + 16)

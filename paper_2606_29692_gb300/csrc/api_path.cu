@@ -33,6 +33,14 @@ extern "C" int tq_evolve_taylor5(tq_ctx* c, const tq_pool* p, int k, double thet
         });
         return TQ_OK;
     }
+    if (!p->sector && p->unit && p->nq >= 2) {
+        auto* parts = static_cast<double2*>(scratch(c, S_PART, (size_t)large_parts(c->sm_count) * sizeof(double2)));
+        launch(c, "taylor5_large", s, [&] {
+            return launch_taylor5_large(p->view, psi->prec, k, theta, nullptr, psi->data, renormalize, parts,
+                                        renormalize ? &c->step->norm2 : nullptr, c->sm_count, s);
+        });
+        return TQ_OK;
+    }
     const int upt = c->pair_upt[psi->prec];
     const int tiles = update_tiles(p, psi->prec, upt);
     double* part = static_cast<double*>(scratch(c, S_PART, (size_t)tiles * sizeof(double)));
@@ -176,6 +184,13 @@ void enqueue_adapt_step(tq_ctx* c, const AdaptBufs& b, const tq_ham* h, const tq
         // the update, its norm and the rescale in one launch
         launch(c, "taylor5_single_gated", s, [&] {
             return launch_taylor5_single(p->view, psi->prec, p->unit, 0, 0.0, c->step, psi->data, 1, &c->step->norm2, s);
+        });
+        return;
+    }
+    if (!p->sector && p->unit && p->nq >= 2) {
+        launch(c, "taylor5_large_gated", s, [&] {
+            return launch_taylor5_large(p->view, psi->prec, 0, 0.0, c->step, psi->data, 1,
+                                        reinterpret_cast<double2*>(b.part), &c->step->norm2, c->sm_count, s);
         });
         return;
     }

@@ -308,6 +308,11 @@ int launch_step_record(DevStep* step, double* rec, int n, cudaStream_t s);
 bool taylor5_single_ready(int nq, int prec);
 int launch_taylor5_single(const PoolView& p, int prec, bool unit_pool, int k, double theta, const DevStep* gate,
                           void* psi, int renorm, double* norm2, cudaStream_t s);
+// States no cluster holds (nq >= 2, pools with entries +-1): norm and update
+// launches; part: large_parts(sms) double2 of scratch.
+int large_parts(int sms);
+int launch_taylor5_large(const PoolView& p, int prec, int k, double theta, const DevStep* gate, void* psi, int renorm,
+                         double2* part, double* norm2, int sms, cudaStream_t s);
 int launch_taylor5_pair_gated(const PoolView& p, int prec, int upt, void* psi, const DevStep* step,
                               double* partials, int sms, cudaStream_t s);
 int launch_scale_gated(void* psi, int prec, long long D, const double* norm2,

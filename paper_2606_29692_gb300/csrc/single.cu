@@ -26,6 +26,8 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 namespace cg = cooperative_groups;
 
 namespace tq {
@@ -288,6 +290,210 @@ k_taylor5_single_closed(PoolView p, int k_imm, double th_imm, const DevStep* gat
     }
 }
 
+// ---------------------------------------- states beyond one cluster
+//
+// Two launches for a pool whose entries are +-1 (A^2 = -I on the support S,
+// so the new norm follows from the input state, as in
+// k_taylor5_single_closed):
+//   k_large_norm:   sum |psi|^2 and sum_S |psi|^2, one partial pair per CTA;
+//   k_large_update: the update and the rescale in one pass, after every CTA
+//                   has added the partials in CTA order.
+// The state is read twice and written once (update, norm reduction and
+// rescale as three launches read and write it twice).  Programmatic launch:
+// the norm kernel lets the update kernel start once its own wait is over,
+// so the update's amplitudes are loaded and its series summed while the norm
+// is still being reduced; it only stores after its wait.  Before that wait it
+// reads nothing the norm kernel writes, and what it does read was complete
+// before the norm kernel's wait ended.
+//
+// What bounds it: launch latency and the L2 (a 20-qubit complex64 state, 8 MB,
+// stays there); in complex128 the float64 pipe.  Renormalised, as three
+// launches and here: complex64 at 18, 20, 22, 24 qubits 24.6 / 9.1,
+// 43.1 / 8.8, 115 / 23.6, 430 / 96 us; complex128 24.6 / 20.8, 49.2 / 31.2,
+// 132 / 100, 521 / 361 us.
+constexpr int LARGE_BS = 256;
+constexpr int LARGE_UPT = 2;         // units of 4 amplitudes per thread
+constexpr int LARGE_NORM_BS = 512;
+constexpr int LARGE_NORM_PER_SM = 2;
+
+// The two running sums (all rows, rows on S).  complex64 carries them as
+// float32 (hi, lo) pairs all the way to the last addition: every float64
+// warp instruction holds its SM quarter's pipe for 64 cycles, and float64
+// shuffle trees in every warp took 6 of the first version's 18 us.
+template <typename T> struct NormPair;
+template <> struct NormPair<double> {
+    double a = 0.0, s = 0.0;
+    __device__ __forceinline__ void add(double na, double ns) {
+        a += na;
+        s += ns;
+    }
+    __device__ __forceinline__ void add_slot(const double2* slot) {
+        const double2 v = __ldcg(slot);
+        add(v.x, v.y);
+    }
+    __device__ __forceinline__ void warp() {
+        a = warp_sum(a);
+        s = warp_sum(s);
+    }
+    __device__ __forceinline__ void store(double2* slot) const { *slot = make_double2(a, s); }
+    __device__ __forceinline__ void load(const double2* slot) {
+        a = slot->x;
+        s = slot->y;
+    }
+    __device__ __forceinline__ double all() const { return a; }
+    __device__ __forceinline__ double on() const { return s; }
+};
+template <> struct NormPair<float> {
+    float ah = 0.f, al = 0.f, sh = 0.f, sl = 0.f;
+    __device__ __forceinline__ void acc(float& hi, float& lo, float h2, float l2) {
+        float sum, err;
+        two_sum(hi, h2, sum, err);
+        hi = sum;
+        lo += l2 + err;
+    }
+    __device__ __forceinline__ void add(float na, float ns) {
+        acc(ah, al, na, 0.f);
+        acc(sh, sl, ns, 0.f);
+    }
+    __device__ __forceinline__ void add_slot(const double2* slot) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(slot));
+        acc(ah, al, v.x, v.y);
+        acc(sh, sl, v.z, v.w);
+    }
+    __device__ __forceinline__ void warp() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_down_sync(0xffffffffu, ah, o), l = __shfl_down_sync(0xffffffffu, al, o);
+            const float h2 = __shfl_down_sync(0xffffffffu, sh, o), l2 = __shfl_down_sync(0xffffffffu, sl, o);
+            acc(ah, al, h, l);
+            acc(sh, sl, h2, l2);
+        }
+    }
+    __device__ __forceinline__ void store(double2* slot) const {
+        *reinterpret_cast<float4*>(slot) = make_float4(ah, al, sh, sl);
+    }
+    __device__ __forceinline__ void load(const double2* slot) {
+        const float4 v = *reinterpret_cast<const float4*>(slot);
+        ah = v.x;
+        al = v.y;
+        sh = v.z;
+        sl = v.w;
+    }
+    __device__ __forceinline__ double all() const { return (double)ah + (double)al; }
+    __device__ __forceinline__ double on() const { return (double)sh + (double)sl; }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(LARGE_NORM_BS)
+k_large_norm(PoolView p, int k_imm, const DevStep* gate, const typename C2<T>::type* __restrict__ psi,
+             double2* __restrict__ part) {
+    constexpr int NW = LARGE_NORM_BS / 32;
+    static_assert(NW <= 32, "one lane per warp in the last tree");
+    __shared__ __align__(16) double2 red[NW];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (gate && gate->converged) return;
+    const int k = gate ? gate->selected : k_imm;
+    const OpRec<T> op = make_rec<T>(p, k);
+    const uint32_t D = 1u << p.nq, step = gridDim.x * LARGE_NORM_BS * 2;
+    const int flip = (op.dcode >> 4) & 7;                    // parity codes of delta = 1
+    const int cx = (op.dcode >> 8) & 7;                      // and of x: col = r ^ x
+    NormPair<T> sum;
+    // four rounds of two consecutive rows in flight, summed plainly (8
+    // squares) before they join the running pair
+    for (uint32_t r0 = (blockIdx.x * LARGE_NORM_BS + threadIdx.x) * 2; r0 < D; r0 += 4 * step) {
+        typename C2<T>::type a[4], b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            a[j] = b[j] = typename C2<T>::type{};
+            const uint32_t r = r0 + j * step;
+            if (r < D && r >= r0) load2(psi, r, a[j], b[j]);
+        }
+        T all = T(0), on = T(0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int code = (base_code(op, r0 + j * step) & 7) ^ cx;
+            const T na = a[j].x * a[j].x + a[j].y * a[j].y, nb = b[j].x * b[j].x + b[j].y * b[j].y;
+            all += na + nb;
+            on += (code == op.t ? na : T(0)) + ((code ^ flip) == op.t ? nb : T(0));
+        }
+        sum.add(all, on);
+    }
+    sum.warp();
+    if ((threadIdx.x & 31) == 0) sum.store(&red[threadIdx.x >> 5]);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        NormPair<T> t;
+        if (threadIdx.x < NW) t.load(&red[threadIdx.x]);
+        t.warp();
+        if (threadIdx.x == 0) t.store(part + blockIdx.x);
+    }
+}
+
+// Units of 4 amplitudes (PairUnit).  n_part: the norm kernel's CTAs, 0 when
+// the state is not renormalised.
+template <typename T>
+__global__ void __launch_bounds__(LARGE_BS)
+k_large_update(PoolView p, int k_imm, double th_imm, const DevStep* gate, typename C2<T>::type* psi,
+               const double2* __restrict__ part, int n_part, double* norm2_out) {
+    using V = typename C2<T>::type;
+    __shared__ double scale_sh;
+    if (!n_part) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (gate && gate->converged) return;
+    const int k = gate ? gate->selected : k_imm;
+    const double theta = gate ? gate->theta : th_imm;
+    const OpRec<T> op = make_rec<T>(p, k);
+    const uint32_t x = op.x;
+    const int hb = 31 - __clz(x);
+    const uint32_t units = (1u << p.nq) >> 2;
+    PairUnit<V> w[LARGE_UPT];
+    bool ok[LARGE_UPT];
+    T unused = T(0);
+#pragma unroll
+    for (int j = 0; j < LARGE_UPT; ++j) {
+        const uint32_t u = (blockIdx.x * LARGE_UPT + j) * LARGE_BS + threadIdx.x;
+        ok[j] = u < units;
+        if (ok[j]) unit_load(psi, x, hb, u, w[j]);
+    }
+    T cf[6];
+    taylor_coefs_fast<T>(theta, cf);
+    double c5 = 0.0, s5 = 0.0;
+    if constexpr (sizeof(T) == 8) closed_coefs(cf, c5, s5);
+#pragma unroll
+    for (int j = 0; j < LARGE_UPT; ++j)
+        if (ok[j]) unit_update<T>(op, hb, cf, c5, s5, w[j], unused);
+    T sc = T(1);
+    if (n_part) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (threadIdx.x < 32) {
+            NormPair<T> t;
+            for (int i = threadIdx.x; i < n_part; i += 32) t.add_slot(part + i);
+            t.warp();
+            if (threadIdx.x == 0) {
+                const double t2 = theta * theta, t6 = t2 * t2 * t2;   // c5^2 + s5^2 - 1 in closed form
+                const double n = fma(t6 * fma(t2, fma(t2, 1.0 / 14400.0, -1.0 / 960.0), 1.0 / 360.0), t.on(), t.all());
+                scale_sh = rsqrt(n);
+                if (blockIdx.x == 0 && norm2_out) *norm2_out = n;
+            }
+        }
+        __syncthreads();
+        sc = (T)scale_sh;
+    }
+#pragma unroll
+    for (int j = 0; j < LARGE_UPT; ++j) {
+        if (!ok[j]) continue;
+        if (n_part) {
+            V* v[4] = {&w[j].a0, &w[j].a1, &w[j].b0, &w[j].b1};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                v[i]->x *= sc;
+                v[i]->y *= sc;
+            }
+        }
+        unit_store(psi, x, hb, w[j]);
+    }
+}
+
 // Cluster size and units per thread for a state of 2^nq amplitudes: the
 // fewest units per thread whose cluster fits; 0 when no configuration does.
 int single_shape(int nq, int max_cluster, int* upt_out) {
@@ -482,6 +688,46 @@ bool single_config(int nq, int prec, int* cs_out, int* upt_out) {
 bool taylor5_single_ready(int nq, int prec) {
     int cs = 0, upt = 0;
     return single_config(nq, prec, &cs, &upt);
+}
+
+int large_parts(int sms) { return LARGE_NORM_PER_SM * sms; }
+
+namespace {
+
+template <typename T>
+int launch_large_t(const PoolView& p, int k, double theta, const DevStep* gate, void* psi, int renorm, double2* part,
+                   double* norm2, int sms, cudaStream_t s) {
+    using V = typename C2<T>::type;
+    const long long units = (1ll << p.nq) >> 2;
+    const long long need = ((1ll << p.nq) + 2 * LARGE_NORM_BS - 1) / (2 * LARGE_NORM_BS);
+    const int n = renorm ? (int)std::min<long long>(need, large_parts(sms)) : 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaSuccess;
+    if (n) {
+        cfg.gridDim = dim3(n);
+        cfg.blockDim = dim3(LARGE_NORM_BS);
+        e = cudaLaunchKernelEx(&cfg, k_large_norm<T>, p, k, gate, static_cast<const V*>(psi), part);
+    }
+    cfg.gridDim = dim3((unsigned)((units + LARGE_BS * LARGE_UPT - 1) / (LARGE_BS * LARGE_UPT)));
+    cfg.blockDim = dim3(LARGE_BS);
+    if (e == cudaSuccess)
+        e = cudaLaunchKernelEx(&cfg, k_large_update<T>, p, k, theta, gate, static_cast<V*>(psi),
+                               static_cast<const double2*>(part), n, norm2);
+    return e == cudaSuccess ? (n ? 2 : 1) : -1;
+}
+
+}  // namespace
+
+int launch_taylor5_large(const PoolView& p, int prec, int k, double theta, const DevStep* gate, void* psi, int renorm,
+                         double2* part, double* norm2, int sms, cudaStream_t s) {
+    return prec == TQ_C128 ? launch_large_t<double>(p, k, theta, gate, psi, renorm, part, norm2, sms, s)
+                           : launch_large_t<float>(p, k, theta, gate, psi, renorm, part, norm2, sms, s);
 }
 
 int launch_taylor5_single(const PoolView& p, int prec, bool unit_pool, int k, double theta, const DevStep* gate,

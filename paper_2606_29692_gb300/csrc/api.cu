@@ -205,9 +205,8 @@ extern "C" int tq_autotune_support(tq_ctx* c, const tq_pool* p, int prec, int n_
     set_device(c);
     const long long D = 1ll << p->nq;
     const size_t sb = (size_t)D * elem_bytes(prec);
-    size_t parts = 0;
-    for (int u : {1, 2, 4, 8})
-        parts = std::max(parts, (size_t)n_states * support_parts(support_tiles(p->nq, n_states, u, c->sm_count)));
+    const int tps = support_tiles(p->nq, prec, n_states, c->sm_count);
+    const size_t parts = (size_t)n_states * support_parts(tps);
     const int cands[8] = {1, 2, 4, 8, -1, -2, -4, -8};
     unsigned char* buf = static_cast<unsigned char*>(
         scratch(c, S_STAGE, (size_t)n_states * sb + (size_t)n_states * (sizeof(int) + 2 * sizeof(double)) +
@@ -233,7 +232,6 @@ extern "C" int tq_autotune_support(tq_ctx* c, const tq_pool* p, int prec, int n_
     int best = c->supp_ppt[prec];
     float best_t = 1e30f;
     for (int u : cands) {
-        const int tps = support_tiles(p->nq, n_states, u, c->sm_count);
         auto once = [&] {
             launch(c, "autotune_support", 0, [&] {
                 return launch_taylor5_support(p->view, n_states, prec, u, psi, dk, dth, part, tps, dn, c->sm_count, 0,

@@ -352,7 +352,7 @@ extern "C" int tq_evolve_taylor5_batch_support(tq_ctx* c, const tq_pool* p, int 
     set_device(c);
     cudaStream_t s = as_stream(stream);
     const int ppt = c->supp_ppt[prec];
-    const int tps = support_tiles(p->nq, n_states, ppt, c->sm_count);
+    const int tps = support_tiles(p->nq, prec, n_states, c->sm_count);
     const int parts = support_parts(tps);
     double* part = static_cast<double*>(scratch(c, S_PART, (size_t)n_states * parts * sizeof(double)));
     launch(c, "taylor5_support", s, [&] {
@@ -377,7 +377,7 @@ extern "C" int tq_evolve_taylor5_batch_support_touch(tq_ctx* c, const tq_pool* p
     set_device(c);
     cudaStream_t s = as_stream(stream);
     const int ppt = c->supp_ppt[prec] < 0 ? c->supp_ppt[prec] : -c->supp_ppt[prec];
-    const int tps = support_tiles(p->nq, n_states, ppt, c->sm_count);
+    const int tps = support_tiles(p->nq, prec, n_states, c->sm_count);
     const int parts = support_parts(tps);
     double* part = static_cast<double*>(scratch(c, S_PART, (size_t)n_states * parts * sizeof(double)));
     // theta is read by the tile set-up and not used: any finite values
@@ -414,7 +414,7 @@ extern "C" int tq_evolve_taylor5_batch_support_host(tq_ctx* c, const tq_pool* p,
     if (!s) TQ_CUDA(cudaStreamCreateWithFlags(&c->aux[0], cudaStreamNonBlocking));
     s = c->aux[0];
     const int ppt = c->supp_ppt[prec];
-    const int tps = support_tiles(p->nq, n_states, ppt, c->sm_count);
+    const int tps = support_tiles(p->nq, prec, n_states, c->sm_count);
     const int parts = support_parts(tps);
     unsigned char* buf = static_cast<unsigned char*>(
         scratch(c, S_HOSTB, (size_t)n_states * (sizeof(int) + 2 * sizeof(double)) + 64));

@@ -7,8 +7,8 @@
 //   energy   items (t, row block): w_t = H_t psi_t, <psi|w>, <psi|psi>
 //            (the trajectory's last item sums its items' parts);
 //   grads    items (t, op, chunk): the chunk's part of 2 Re<w_t|A_k psi_t>;
-//   select   one warp per t: g_t[k] (divided by <psi|psi>) summed from the
-//            chunk parts in a fixed order, k*, max|g|, convergence, angle,
+//   select   one block per t: its energy, g_t[k] (divided by <psi|psi>)
+//            summed from the chunk parts in a fixed order, k*, max|g|, convergence, angle,
 //            record, and the iteration counter advanced; the last block
 //            numbers the active trajectories' energy items for the next
 //            iteration (prefix counts);
@@ -46,6 +46,7 @@ namespace tq {
 struct TrajDev {
     int nq, M, len, nch, chunk;
     int eoff, ecnt;          // energy items of this trajectory
+    int nslab, wslab;        // slabs of SLAB_ROWS rows and their mean entries (kb_energy_smem)
     int pcnt;                // pair tiles (8 norm partials each)
     long long D;
     long long hf;
@@ -310,6 +311,149 @@ kbx_energy(const TrajDev* tr, TrajState* ts, const int4* items, const int2* pre,
     }
 }
 
+// Energy of every active trajectory, complex64, CSR, with the trajectory's
+// state in shared memory (states of up to `room` amplitudes; larger ones are
+// gathered from global memory).  A row's 32 partial sums are those of the
+// 32-lane schedule (entry e in partial (e - first) mod 32, each in entry
+// order, then the same butterfly), here on 8 lanes with four sums each, so
+// the results are that schedule's bit for bit with 6 shuffles per four rows
+// instead of 40 and four independent chains per lane.
+//
+// What bounds the CSR form: a warp gather of 32 amplitudes touches 32 lines,
+// and the L1 serves about one line a cycle; 24 trajectories of 10 to 14
+// qubits (2.3e7 entries) took 96 us per iteration.  From shared memory the
+// same gather costs a few cycles, and what is left is the matrix stream
+// (8 bytes per entry): 61 us against 91 with the L1 gathers.
+//
+// The matrix entries of the active trajectories are cut evenly over the CTAs
+// (one per SM): wpre[t] counts entries before trajectory t in slabs of
+// SLAB_ROWS rows at the trajectory's mean, CTA c takes the slabs that start in
+// [c W / G, (c + 1) W / G).  A CTA and a trajectory it touches make a segment;
+// its sums go to seg[c + rank[t]] (a step along the cut advances either the
+// CTA or the trajectory, so the place is its own), and the select launch adds
+// a trajectory's segments in CTA order.
+constexpr int KBS_BS = 1024;
+constexpr int SLAB_ROWS = 32;
+constexpr int KBS_CHUNK = 1024;      // rows finished together, one per thread
+
+__device__ __forceinline__ long long cta_bound(long long W, int c, int G) { return W * c / G; }
+
+// Off-diagonal sums of the four rows r .. r + 3 of a warp (8 lanes each);
+// `x` is the state (shared or global).
+__device__ __forceinline__ float2 rows4(const int* __restrict__ rowptr, const int* __restrict__ col,
+                                        const float* __restrict__ val, const float2* x, int r, int r1) {
+    const int lane = threadIdx.x & 31, l = lane & 7, row = r + (lane >> 3);
+    int e = 0, e1 = 0;
+    if (row < r1) {
+        e = rowptr[row];
+        e1 = rowptr[row + 1];
+    }
+    const int rounds = __reduce_max_sync(0xffffffffu, (unsigned)(e1 - e + 31) >> 5);
+    e += l;
+    float2 acc[4];
+    int c[4];
+    float a[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        acc[j] = make_float2(0.f, 0.f);
+        const bool in = e + 8 * j < e1;
+        c[j] = in ? col[e + 8 * j] : -1;
+        a[j] = in ? val[e + 8 * j] : 0.f;
+    }
+    for (int k = 0; k < rounds; ++k) {
+        e += 32;
+        int nc[4];
+        float na[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const bool in = e + 8 * j < e1;
+            nc[j] = in ? col[e + 8 * j] : -1;
+            na[j] = in ? val[e + 8 * j] : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (c[j] >= 0) acc[j] = __ffma2_rn(make_float2(a[j], a[j]), x[c[j]], acc[j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            c[j] = nc[j];
+            a[j] = na[j];
+        }
+    }
+    // lanes xor 16 and 8 of the 32-lane butterfly are sums of this lane
+    float sx = (acc[0].x + acc[2].x) + (acc[1].x + acc[3].x);
+    float sy = (acc[0].y + acc[2].y) + (acc[1].y + acc[3].y);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        sy += __shfl_xor_sync(0xffffffffu, sy, o);
+    }
+    return make_float2(sx, sy);
+}
+
+__global__ void __launch_bounds__(KBS_BS, 1)
+kb_energy_smem(const TrajDev* tr, const long long* __restrict__ wpre, const int* __restrict__ rank, int n, int room,
+               double2* seg) {
+    extern __shared__ __align__(16) unsigned char kbs_raw[];
+    float2* ps = reinterpret_cast<float2*>(kbs_raw);
+    float2* rs = ps + room;                                   // off-diagonal sums of a chunk's rows
+    __shared__ double sh[2 * KBS_BS / 32];
+    const int c = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const long long W = wpre[n], lo = cta_bound(W, c, G), hi = cta_bound(W, c + 1, G);
+    if (lo >= hi) return;
+    int t = 0;
+    for (int up = n; up - t > 1;) {                           // last t with wpre[t] <= lo
+        const int mid = (t + up) >> 1;
+        if (wpre[mid] <= lo) t = mid;
+        else up = mid;
+    }
+    for (; t < n && wpre[t] < hi; ++t) {
+        const long long w0 = wpre[t], w1 = wpre[t + 1];
+        if (w1 <= lo || w1 == w0) continue;
+        const TrajDev& d = tr[t];
+        const long long from = (lo > w0 ? lo : w0) - w0;
+        const int i0 = (int)((from + d.wslab - 1) / d.wslab);
+        const int i1 = (int)min((long long)d.nslab, (hi - w0 + d.wslab - 1) / d.wslab);
+        double num = 0.0, den = 0.0;
+        if (i0 < i1) {
+            const int r0 = i0 * SLAB_ROWS, r1 = (int)min((long long)i1 * SLAB_ROWS, d.D);
+            const float2* psi = static_cast<const float2*>(d.psi);
+            const float2* x = psi;
+            if (d.D <= room) {
+                __syncthreads();                              // the previous segment is done with ps
+                for (int i = tid; i < (int)(d.D >> 1); i += KBS_BS)
+                    reinterpret_cast<float4*>(ps)[i] = reinterpret_cast<const float4*>(psi)[i];
+                __syncthreads();
+                x = ps;
+            }
+            const float* val = static_cast<const float*>(d.val);
+            const int chunks = (r1 - r0 + KBS_CHUNK - 1) / KBS_CHUNK;
+            const int len = ((r1 - r0 + chunks - 1) / chunks + 3) & ~3;
+            for (int q0 = r0; q0 < r1; q0 += len) {
+                const int q1 = min(q0 + len, r1);
+                for (int r = q0 + 4 * wid; r < q1; r += 4 * (KBS_BS / 32)) {
+                    const float2 s = rows4(d.rowptr, d.col, val, x, r, q1);
+                    const int row = r + (lane >> 3);
+                    if ((lane & 7) == 0 && row < q1) rs[row - q0] = s;
+                }
+                __syncthreads();
+                const int row = q0 + tid;
+                if (row < q1) {
+                    const float2 pv = x[row], s = rs[tid];
+                    const double px = (double)pv.x, py = (double)pv.y, dg = d.diag[row];
+                    const double wx = fma(dg, px, (double)s.x), wy = fma(dg, py, (double)s.y);
+                    d.w32[row] = make_float2((float)wx, (float)wy);
+                    num += px * wx + py * wy;
+                    den += px * px + py * py;
+                }
+                __syncthreads();
+            }
+        }
+        double v[2] = {num, den};
+        block_sum<2>(v, sh);
+        if (tid == 0) seg[c + rank[t]] = make_double2(v[0], v[1]);
+    }
+}
+
 // Gradient item: (t, op, chunk of the op's support rows).
 template <typename T>
 __global__ void __launch_bounds__(GRAD_TPB)
@@ -337,102 +481,189 @@ kb_grad(const TrajDev* tr, const TrajState* ts, const int4* items, int n_items) 
     }
 }
 
-// Numbers the energy items of the active trajectories for the next energy
-// launch (n + 1 entries, as active_traj reads them), in one block: thread i
-// owns a run of consecutive trajectories.
-__device__ void number_active(const TrajDev* tr, const TrajState* ts, int n, int2* pre) {
-    __shared__ int wsum[32];
+// What the energy launch needs to know of the trajectories still active:
+// their items numbered (pre, as active_traj reads them), their matrix
+// entries before trajectory t (wpre) and their rank (kb_energy_smem).
+struct Active {
+    int2* pre;          // [n + 1]
+    long long* wpre;    // [n + 1]
+    int* rank;          // [n]
+};
+
+// Renews it for the next iteration, in one block: thread i owns a run of
+// consecutive trajectories.
+__device__ void number_active(const TrajDev* tr, const TrajState* ts, int n, const Active& act) {
+    __shared__ int wsum[32], asum[32];
+    __shared__ long long lsum[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int c = (n + blockDim.x - 1) / blockDim.x;
     const int a = min(n, (int)threadIdx.x * c), b = min(n, a + c);
-    int own = 0;
+    int own = 0, own_a = 0;
+    long long own_w = 0;
     for (int t = a; t < b; ++t)
-        if (__ldcg(&ts[t].active)) own += tr[t].ecnt;
-    int inc = own;                             // inclusive scan over the warp
+        if (__ldcg(&ts[t].active)) {
+            own += tr[t].ecnt;
+            own_w += (long long)tr[t].nslab * tr[t].wslab;
+            ++own_a;
+        }
+    int inc = own, inc_a = own_a;              // inclusive scans over the warp
+    long long inc_w = own_w;
     for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += x;
+        const int x = __shfl_up_sync(0xffffffffu, inc, o), y = __shfl_up_sync(0xffffffffu, inc_a, o);
+        const long long z = __shfl_up_sync(0xffffffffu, inc_w, o);
+        if (lane >= o) {
+            inc += x;
+            inc_a += y;
+            inc_w += z;
+        }
     }
-    if (lane == 31) wsum[wid] = inc;
+    if (lane == 31) {
+        wsum[wid] = inc;
+        asum[wid] = inc_a;
+        lsum[wid] = inc_w;
+    }
     __syncthreads();
-    int before = 0, total = 0;
+    int e = inc - own, r = inc_a - own_a, total = 0;   // exclusive prefixes of this thread's run
+    long long l = inc_w - own_w, total_w = 0;
     for (int w = 0; w < nw; ++w) {
-        if (w < wid) before += wsum[w];
+        if (w < wid) {
+            e += wsum[w];
+            r += asum[w];
+            l += lsum[w];
+        }
         total += wsum[w];
+        total_w += lsum[w];
     }
-    int e = before + inc - own;                // exclusive prefix of this thread's run
     for (int t = a; t < b; ++t) {
         const TrajDev& d = tr[t];
-        pre[t] = make_int2(e, d.eoff - e);
-        if (__ldcg(&ts[t].active)) e += d.ecnt;
+        act.pre[t] = make_int2(e, d.eoff - e);
+        act.wpre[t] = l;
+        act.rank[t] = r;
+        if (__ldcg(&ts[t].active)) {
+            e += d.ecnt;
+            l += (long long)d.nslab * d.wslab;
+            ++r;
+        }
     }
-    if (threadIdx.x == 0) pre[n] = make_int2(total, 0);
+    if (threadIdx.x == 0) {
+        act.pre[n] = make_int2(total, 0);
+        act.wpre[n] = total_w;
+    }
 }
 
-// One warp per trajectory: each gradient from its op's chunk partials
-// (Eq. (5), divided by <psi|psi>), then choice, convergence, angle, record,
-// and the iteration counter advanced.  The last block to finish numbers the
-// next iteration's energy items.
-__global__ void kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, int2* pre,
-                          unsigned* ticket) {
+// One block per trajectory: its energy from the segments' sums (seg set), each
+// gradient from its op's chunk partials (Eq. (5), divided by <psi|psi>), then
+// choice, convergence, angle, record, and the iteration counter advanced.
+// The last block to finish renews the active trajectories' numbering.  Maxima
+// and thresholds compare bit patterns (a non-negative double orders like
+// them), off the float64 pipe.
+constexpr int SEL_BS = 128;
+__global__ void __launch_bounds__(SEL_BS)
+kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, Active act, const double2* seg, int seg_ctas,
+          unsigned* ticket) {
+    constexpr int NW = SEL_BS / 32;
+    constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;
     __shared__ bool last;
-    const int lane = threadIdx.x & 31;
-    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (t < n) {
-        TrajState& s = ts[t];
-        if (!s.active) {
-            if (lane == 0) s.do_update = 0;
-        } else {
-            const TrajDev& d = tr[t];
-            const double inv = 1.0 / s.e_den;
-            double m = 0.0;
-            // the lane's ops k = lane + 32 j, four at a time so that their
-            // bounds and first chunks load together; each op's chunks are
-            // summed in item order (every op has at least one)
-            for (int k0 = lane; k0 < d.M; k0 += 32 * SEL_U) {
-                int f[SEL_U], e[SEL_U];
-                double acc[SEL_U];
-#pragma unroll
-                for (int u = 0; u < SEL_U; ++u) {
-                    const int k = k0 + 32 * u;
-                    f[u] = k < d.M ? d.gfirst[k] : 0;
-                    e[u] = k < d.M ? d.gfirst[k + 1] : 0;
-                }
-#pragma unroll
-                for (int u = 0; u < SEL_U; ++u) acc[u] = k0 + 32 * u < d.M ? d.gpart[f[u]] : 0.0;
-#pragma unroll
-                for (int u = 0; u < SEL_U; ++u) {
-                    const int k = k0 + 32 * u;
-                    if (k < d.M) {
-                        for (int i = f[u] + 1; i < e[u]; ++i) acc[u] += d.gpart[i];
-                        const double g = 2.0 * acc[u] * inv;
-                        d.g[k] = g;            // read back below by this lane only
-                        m = fmax(m, fabs(g));
+    __shared__ double e_sh[2];
+    __shared__ unsigned long long smax[NW];
+    __shared__ int smin[NW];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = blockIdx.x;
+    TrajState& s = ts[t];
+    if (!s.active) {
+        if (threadIdx.x == 0) s.do_update = 0;
+    } else {
+        const TrajDev& d = tr[t];
+        if (wid == 0) {
+            double num = 0.0, den = 0.0;
+            if (seg) {
+                const long long W = act.wpre[n], w0 = act.wpre[t], w1 = act.wpre[t + 1];
+                for (int c = lane; c < seg_ctas; c += 32) {
+                    const long long lo = cta_bound(W, c, seg_ctas), hi = cta_bound(W, c + 1, seg_ctas);
+                    if (lo < hi && hi > w0 && lo < w1) {
+                        const double2 v = seg[c + act.rank[t]];
+                        num += v.x;
+                        den += v.y;
                     }
                 }
+                num = warp_sum(num);
+                den = warp_sum(den);
+            } else {
+                num = s.e_num;
+                den = s.e_den;
             }
-            for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-            const double tau = prec == TQ_C128 ? 1e-9 * fmax(1.0, m) : 1e-5;
-            int best = d.M;
-            for (int k = lane; k < d.M; k += 32)
-                if (fabs(d.g[k]) >= m - tau && k < best) best = k;
-            for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
             if (lane == 0) {
-                const int it = s.iter;
-                s.selected = best < d.M ? best : 0;
-                s.max_grad = m;
-                s.converged = m < eps ? 1 : 0;
-                s.theta = s.converged ? 0.0 : d.thetas[it];
-                s.do_update = !s.converged;
-                if (s.do_update) s.updated = 1;
-                d.res_e[it] = s.energy;
-                d.res_g[it] = m;
-                d.res_sel[it] = s.selected;
-                d.res_th[it] = s.theta;
-                s.iter = it + 1;
-                s.active = (!s.converged && it + 1 < d.len) ? 1 : 0;
-                __threadfence();
+                e_sh[0] = num / den;
+                e_sh[1] = 1.0 / den;
             }
+        }
+        // the thread's ops k = tid + SEL_BS j, SEL_U at a time so that their
+        // bounds and first chunks load together; each op's chunks are summed
+        // in item order (every op has at least one)
+        unsigned long long m = 0;
+        for (int k0 = threadIdx.x; k0 < d.M; k0 += SEL_BS * SEL_U) {
+            int f[SEL_U], e[SEL_U];
+            double acc[SEL_U];
+#pragma unroll
+            for (int u = 0; u < SEL_U; ++u) {
+                const int k = k0 + SEL_BS * u;
+                f[u] = k < d.M ? d.gfirst[k] : 0;
+                e[u] = k < d.M ? d.gfirst[k + 1] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < SEL_U; ++u) acc[u] = k0 + SEL_BS * u < d.M ? d.gpart[f[u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < SEL_U; ++u) {
+                const int k = k0 + SEL_BS * u;
+                if (k < d.M) {
+                    for (int i = f[u] + 1; i < e[u]; ++i) acc[u] += d.gpart[i];
+                    d.g[k] = acc[u];           // scaled and read back below by this thread only
+                }
+            }
+        }
+        __syncthreads();                       // e_sh
+        const double inv = e_sh[1];
+        for (int k = threadIdx.x; k < d.M; k += SEL_BS) {
+            const double g = 2.0 * d.g[k] * inv;
+            d.g[k] = g;
+            const unsigned long long a = (unsigned long long)__double_as_longlong(g) & kAbs;
+            if (a <= kInf && a > m) m = a;     // NaN gradients are skipped
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+            m = v > m ? v : m;
+        }
+        if (lane == 0) smax[wid] = m;
+        __syncthreads();
+        for (int i = 0; i < NW; ++i) m = smax[i] > m ? smax[i] : m;
+        const double gmax = __longlong_as_double((long long)m);
+        const double tau = prec == TQ_C128 ? 1e-9 * fmax(1.0, gmax) : 1e-5;
+        const double cut = gmax - tau;
+        const unsigned long long thr = cut > 0.0 ? (unsigned long long)__double_as_longlong(cut) : 0ull;
+        int best = d.M;
+        for (int k = threadIdx.x; k < d.M; k += SEL_BS) {
+            const unsigned long long a = (unsigned long long)__double_as_longlong(d.g[k]) & kAbs;
+            if (a <= kInf && a >= thr && k < best) best = k;
+        }
+        best = __reduce_min_sync(0xffffffffu, best);
+        if (lane == 0) smin[wid] = best;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < NW; ++i) best = min(best, smin[i]);
+            const int it = s.iter;
+            s.energy = e_sh[0];
+            s.selected = best < d.M ? best : 0;
+            s.max_grad = gmax;
+            s.converged = gmax < eps ? 1 : 0;
+            s.theta = s.converged ? 0.0 : d.thetas[it];
+            s.do_update = !s.converged;
+            if (s.do_update) s.updated = 1;
+            d.res_e[it] = s.energy;
+            d.res_g[it] = gmax;
+            d.res_sel[it] = s.selected;
+            d.res_th[it] = s.theta;
+            s.iter = it + 1;
+            s.active = (!s.converged && it + 1 < d.len) ? 1 : 0;
+            __threadfence();
         }
     }
     __syncthreads();
@@ -440,7 +671,7 @@ __global__ void kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, i
     __syncthreads();
     if (!last) return;
     __threadfence();
-    number_active(tr, ts, n, pre);
+    number_active(tr, ts, n, act);
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
@@ -539,8 +770,12 @@ struct tq_batch {
     int n_e = 0, n_g = 0, n_p = 0, n_s = 0;
     double* epart = nullptr;
     double* npart = nullptr;
-    int2* pre = nullptr;            // the active trajectories' energy items, numbered (n + 1 entries)
-    int2* pre0 = nullptr;           // the same before the first iteration
+    Active act{};                   // the active trajectories, numbered (one block, act.pre first)
+    unsigned char* act0 = nullptr;  // the same block before the first iteration
+    size_t act_bytes = 0;
+    double2* seg = nullptr;         // energy segments (kb_energy_smem)
+    int room = 0;                   // amplitudes it holds in shared memory
+    bool by_segments() const { return prec == TQ_C64 && lpr == 32; }
     unsigned* nticket = nullptr;    // blocks of the select launch done
     unsigned char* res = nullptr;   // results block (see tq_batch_create)
     size_t res_len = 0;             // iterations of all trajectories
@@ -575,16 +810,30 @@ T* dupload(tq_batch* b, const std::vector<T>& v) {
     return p;
 }
 
+// States of at most KBS_ROOM amplitudes are staged (128 KB).
+constexpr int KBS_ROOM = 1 << 14;
+size_t kbs_smem(int room) { return ((size_t)room + KBS_CHUNK) * sizeof(float2); }
+
 template <typename T, typename VT>
 int launch_energy(tq_batch* b, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4) {
+        if (b->by_segments()) {
+            kb_energy_smem<<<b->ctx->sm_count, KBS_BS, kbs_smem(b->room), s>>>(b->d_td, b->act.wpre, b->act.rank, b->n,
+                                                                              b->room, b->seg);
+            return 1;
+        }
+    }
     switch (b->lpr) {
         case TQ_SPMV_XELL:
-            kbx_energy<T, VT><<<b->grid_x, BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->pre, b->n, b->epart);
+            kbx_energy<T, VT><<<b->grid_x, BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->act.pre, b->n, b->epart);
             break;
-        case 4: kb_energy<T, VT, 4><<<b->grid_e[0], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->pre, b->n, b->epart); break;
-        case 8: kb_energy<T, VT, 8><<<b->grid_e[1], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->pre, b->n, b->epart); break;
-        case 16: kb_energy<T, VT, 16><<<b->grid_e[2], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->pre, b->n, b->epart); break;
-        default: kb_energy<T, VT, 32><<<b->grid_e[3], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->pre, b->n, b->epart); break;
+        case 4: kb_energy<T, VT, 4><<<b->grid_e[0], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->act.pre, b->n, b->epart); break;
+        case 8: kb_energy<T, VT, 8><<<b->grid_e[1], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->act.pre, b->n, b->epart); break;
+        case 16: kb_energy<T, VT, 16><<<b->grid_e[2], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->act.pre, b->n, b->epart); break;
+        default:
+            if constexpr (sizeof(T) == 8)
+                kb_energy<T, VT, 32><<<b->grid_e[3], BT_BS, 0, s>>>(b->d_td, b->d_ts, b->eitems, b->act.pre, b->n, b->epart);
+            break;
     }
     return 1;
 }
@@ -596,7 +845,8 @@ void compute_grids(tq_batch* b) {
     b->grid_e[0] = std::min(b->n_e, resident_grid(kb_energy<T, VT, 4>, BT_BS, sms));
     b->grid_e[1] = std::min(b->n_e, resident_grid(kb_energy<T, VT, 8>, BT_BS, sms));
     b->grid_e[2] = std::min(b->n_e, resident_grid(kb_energy<T, VT, 16>, BT_BS, sms));
-    b->grid_e[3] = std::min(b->n_e, resident_grid(kb_energy<T, VT, 32>, BT_BS, sms));
+    if constexpr (sizeof(T) == 8) b->grid_e[3] = std::min(b->n_e, resident_grid(kb_energy<T, VT, 32>, BT_BS, sms));
+    else TQ_CUDA(cudaFuncSetAttribute(kb_energy_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kbs_smem(KBS_ROOM)));
     b->grid_x = std::min(b->n_e, resident_grid(kbx_energy<T, VT>, BT_BS, sms));
     b->grid_g = std::min(b->n_g, resident_grid(kb_grad<T>, GRAD_TPB, sms));
     b->grid_p = std::min(b->n_p, resident_grid(kb_pair<T>, PAIR_BS, sms));
@@ -619,8 +869,8 @@ void enqueue_iteration(tq_batch* b, cudaStream_t s) {
         return 1;
     });
     launch(c, "batch_select", s, [&] {
-        kb_select<<<(b->n * 32 + 255) / 256, 256, 0, s>>>(b->d_td, b->d_ts, b->n, b->eps, b->prec, b->pre,
-                                                          b->nticket);
+        kb_select<<<b->n, SEL_BS, 0, s>>>(b->d_td, b->d_ts, b->n, b->eps, b->prec, b->act,
+                                          b->by_segments() ? b->seg : nullptr, c->sm_count, b->nticket);
         return 1;
     });
     launch(c, "batch_taylor5_pair", s, [&] {
@@ -653,7 +903,7 @@ void enqueue_all(tq_batch* b, cudaStream_t s) {
 }
 
 void reset(tq_batch* b, cudaStream_t s) {
-    TQ_CUDA(cudaMemcpyAsync(b->pre, b->pre0, (size_t)(b->n + 1) * sizeof(int2), cudaMemcpyDeviceToDevice, s));
+    TQ_CUDA(cudaMemcpyAsync(b->act.pre, b->act0, b->act_bytes, cudaMemcpyDeviceToDevice, s));
     launch(b->ctx, "batch_reset", s, [&] {
         return b->prec == TQ_C128 ? launch_reset<double>(b, s) : launch_reset<float>(b, s);
     });
@@ -720,6 +970,9 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
             for (long long r = 0; r < d.D; r += ROWS_PER_ITEM)
                 ei.push_back(make_int4(t, (int)r, (int)std::min<long long>(ROWS_PER_ITEM, d.D - r), 0));
             d.ecnt = (int)ei.size() - d.eoff;
+            d.nslab = (int)((d.D + SLAB_ROWS - 1) / SLAB_ROWS);
+            d.wslab = (int)std::max<long long>(1, h->nnz / d.nslab);
+            if (d.D <= KBS_ROOM) b->room = std::max(b->room, (int)d.D);
             d.gbase = (int)gi.size();
             // the pool's own item table: op k's chunks are items gf[k] .. gf[k + 1] - 1
             std::vector<int> gf((size_t)d.M + 1);
@@ -779,16 +1032,35 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
         b->npart = dalloc<double>(b, (size_t)nslots);
         {
             // before the first iteration the active trajectories are those of length > 0
-            std::vector<int2> p0((size_t)n_traj + 1);
-            int e = 0;
+            const size_t np = (size_t)n_traj + 1;
+            b->act_bytes = np * (sizeof(int2) + sizeof(long long)) + (size_t)n_traj * sizeof(int);
+            std::vector<unsigned char> img(b->act_bytes);
+            auto view = [&](unsigned char* base) {
+                Active v;
+                v.pre = reinterpret_cast<int2*>(base);
+                v.wpre = reinterpret_cast<long long*>(base + np * sizeof(int2));
+                v.rank = reinterpret_cast<int*>(base + np * (sizeof(int2) + sizeof(long long)));
+                return v;
+            };
+            const Active h0 = view(img.data());
+            int e = 0, r = 0;
+            long long w = 0;
             for (int t = 0; t < n_traj; ++t) {
                 const TrajDev& d = b->td[t];
-                p0[t] = make_int2(e, d.eoff - e);
-                if (d.len > 0) e += d.ecnt;
+                h0.pre[t] = make_int2(e, d.eoff - e);
+                h0.wpre[t] = w;
+                h0.rank[t] = r;
+                if (d.len > 0) {
+                    e += d.ecnt;
+                    w += (long long)d.nslab * d.wslab;
+                    ++r;
+                }
             }
-            p0[n_traj] = make_int2(e, 0);
-            b->pre0 = dupload(b, p0);
-            b->pre = dupload(b, p0);
+            h0.pre[n_traj] = make_int2(e, 0);
+            h0.wpre[n_traj] = w;
+            b->act0 = dupload(b, img);
+            b->act = view(dupload(b, img));
+            b->seg = dalloc<double2>(b, (size_t)c->sm_count + n_traj);
             b->nticket = dalloc<unsigned>(b, 1);
             TQ_CUDA(cudaMemset(b->nticket, 0, sizeof(unsigned)));
         }

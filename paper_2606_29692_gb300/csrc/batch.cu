@@ -46,7 +46,8 @@ namespace tq {
 struct TrajDev {
     int nq, M, len, nch, chunk;
     int eoff, ecnt;          // energy items of this trajectory
-    int nslab, wslab;        // slabs of SLAB_ROWS rows and their mean entries (kb_energy_smem)
+    int nslab, wslab;        // slabs of about wslab units of work each (kb_energy_smem):
+    const int* cut;          // slab i is rows cut[i] .. cut[i + 1] - 1
     int pcnt;                // pair tiles (8 norm partials each)
     long long D;
     long long hf;
@@ -315,79 +316,116 @@ kbx_energy(const TrajDev* tr, TrajState* ts, const int4* items, const int2* pre,
 // state in shared memory (states of up to `room` amplitudes; larger ones are
 // gathered from global memory).  A row's 32 partial sums are those of the
 // 32-lane schedule (entry e in partial (e - first) mod 32, each in entry
-// order, then the same butterfly), here on 8 lanes with four sums each, so
-// the results are that schedule's bit for bit with 6 shuffles per four rows
-// instead of 40 and four independent chains per lane.
+// order, then the same butterfly), four rows at a time, so the results are
+// that schedule's bit for bit with 12 shuffles per four rows instead of 40
+// and four independent chains per lane.
 //
 // What bounds the CSR form: a warp gather of 32 amplitudes touches 32 lines,
 // and the L1 serves about one line a cycle; 24 trajectories of 10 to 14
 // qubits (2.3e7 entries) took 96 us per iteration.  From shared memory the
 // same gather costs a few cycles, and what is left is the matrix stream
-// (8 bytes per entry): 61 us against 91 with the L1 gathers.
+// (8 bytes per entry), the gathers' bank conflicts and latency: 55 us against
+// 91 with the L1 gathers.
 //
-// The matrix entries of the active trajectories are cut evenly over the CTAs
-// (one per SM): wpre[t] counts entries before trajectory t in slabs of
-// SLAB_ROWS rows at the trajectory's mean, CTA c takes the slabs that start in
+// The work of the active trajectories (entries and rows) is cut evenly over
+// the CTAs (one per SM): a trajectory's rows are cut once into slabs of equal
+// work (k_cut_slabs), wpre[t] counts the work before trajectory t, and CTA c
+// takes the slabs that start in
 // [c W / G, (c + 1) W / G).  A CTA and a trajectory it touches make a segment;
 // its sums go to seg[c + rank[t]] (a step along the cut advances either the
 // CTA or the trajectory, so the place is its own), and the select launch adds
 // a trajectory's segments in CTA order.
 constexpr int KBS_BS = 1024;
-constexpr int SLAB_ROWS = 32;
+constexpr int KBS_SLABS = 1024;      // most slabs of a trajectory
+constexpr int KBS_AHEAD = 2;
+// A row costs about as much as this many entries (its float64 finish, row
+// sums and the unfilled last round): what a slab is cut by.
+constexpr int KBS_ROW = 32;
 constexpr int KBS_CHUNK = 1024;      // rows finished together, one per thread
 
 __device__ __forceinline__ long long cta_bound(long long W, int c, int G) { return W * c / G; }
 
-// Off-diagonal sums of the four rows r .. r + 3 of a warp (8 lanes each);
-// `x` is the state (shared or global).
+// Off-diagonal sums of the four rows r .. r + 3 of a warp, all 32 lanes on
+// each (whole lines of columns and values), their chains interleaved; lane l
+// returns row r + (l >> 3).  `x` is the state (shared or global).  The
+// butterfly over the rows' partial sums scatters as it goes: each half keeps
+// two rows at distance 16, each quarter one at distance 8.
 __device__ __forceinline__ float2 rows4(const int* __restrict__ rowptr, const int* __restrict__ col,
                                         const float* __restrict__ val, const float2* x, int r, int r1) {
-    const int lane = threadIdx.x & 31, l = lane & 7, row = r + (lane >> 3);
-    int e = 0, e1 = 0;
-    if (row < r1) {
-        e = rowptr[row];
-        e1 = rowptr[row + 1];
+    const int lane = threadIdx.x & 31;
+    const int at = lane <= 4 ? rowptr[min(r + lane, r1)] : 0;
+    int first[4], left[4], most = 0;                 // first entry of this lane, entries of the row past it
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int b = __shfl_sync(0xffffffffu, at, q), n = __shfl_sync(0xffffffffu, at, q + 1) - b;
+        most = max(most, n);
+        first[q] = b + lane;
+        left[q] = n - lane;
     }
-    const int rounds = __reduce_max_sync(0xffffffffu, (unsigned)(e1 - e + 31) >> 5);
-    e += l;
+    // a row's entries k + lane; KBS_AHEAD rounds of loads in flight
     float2 acc[4];
-    int c[4];
-    float a[4];
+    int c[KBS_AHEAD + 1][4];
+    float a[KBS_AHEAD + 1][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        acc[j] = make_float2(0.f, 0.f);
-        const bool in = e + 8 * j < e1;
-        c[j] = in ? col[e + 8 * j] : -1;
-        a[j] = in ? val[e + 8 * j] : 0.f;
-    }
-    for (int k = 0; k < rounds; ++k) {
-        e += 32;
-        int nc[4];
-        float na[4];
+    for (int q = 0; q < 4; ++q) acc[q] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool in = e + 8 * j < e1;
-            nc[j] = in ? col[e + 8 * j] : -1;
-            na[j] = in ? val[e + 8 * j] : 0.f;
+    for (int s = 0; s < KBS_AHEAD; ++s)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool in = 32 * s < left[q];
+            c[s][q] = in ? col[first[q] + 32 * s] : -1;
+            a[s][q] = in ? val[first[q] + 32 * s] : 0.f;
+        }
+    for (int k = 0; k < most; k += 32) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int at2 = k + 32 * KBS_AHEAD;
+            const bool in = at2 < left[q];
+            c[KBS_AHEAD][q] = in ? col[first[q] + at2] : -1;
+            a[KBS_AHEAD][q] = in ? val[first[q] + at2] : 0.f;
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (c[j] >= 0) acc[j] = __ffma2_rn(make_float2(a[j], a[j]), x[c[j]], acc[j]);
+        for (int q = 0; q < 4; ++q)
+            if (c[0][q] >= 0) acc[q] = __ffma2_rn(make_float2(a[0][q], a[0][q]), x[c[0][q]], acc[q]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            c[j] = nc[j];
-            a[j] = na[j];
-        }
+        for (int s = 0; s < KBS_AHEAD; ++s)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                c[s][q] = c[s + 1][q];
+                a[s][q] = a[s + 1][q];
+            }
     }
-    // lanes xor 16 and 8 of the 32-lane butterfly are sums of this lane
-    float sx = (acc[0].x + acc[2].x) + (acc[1].x + acc[3].x);
-    float sy = (acc[0].y + acc[2].y) + (acc[1].y + acc[3].y);
+    float2 k2[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float2 give = (lane & 16) ? acc[i] : acc[i + 2], keep = (lane & 16) ? acc[i + 2] : acc[i];
+        k2[i].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16);
+        k2[i].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16);
+    }
+    const float2 give = (lane & 8) ? k2[0] : k2[1], keep = (lane & 8) ? k2[1] : k2[0];
+    float sx = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8);
+    float sy = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
         sx += __shfl_xor_sync(0xffffffffu, sx, o);
         sy += __shfl_xor_sync(0xffffffffu, sy, o);
     }
     return make_float2(sx, sy);
+}
+
+// cut[i]: the first row whose work before it (entries, and KBS_ROW per row)
+// reaches i / nslab of the trajectory's.
+__global__ void k_cut_slabs(const int* __restrict__ rowptr, long long D, long long nnz, int nslab, int* cut) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i > nslab) return;
+    const long long target = (nnz + KBS_ROW * D) * i / nslab;
+    long long lo = 0, hi = D;
+    while (lo < hi) {
+        const long long mid = (lo + hi) >> 1;
+        if (rowptr[mid] + KBS_ROW * mid >= target) hi = mid;
+        else lo = mid + 1;
+    }
+    cut[i] = i == 0 ? 0 : i == nslab ? (int)D : (int)lo;
 }
 
 __global__ void __launch_bounds__(KBS_BS, 1)
@@ -415,7 +453,7 @@ kb_energy_smem(const TrajDev* tr, const long long* __restrict__ wpre, const int*
         const int i1 = (int)min((long long)d.nslab, (hi - w0 + d.wslab - 1) / d.wslab);
         double num = 0.0, den = 0.0;
         if (i0 < i1) {
-            const int r0 = i0 * SLAB_ROWS, r1 = (int)min((long long)i1 * SLAB_ROWS, d.D);
+            const int r0 = d.cut[i0], r1 = d.cut[i1];
             const float2* psi = static_cast<const float2*>(d.psi);
             const float2* x = psi;
             if (d.D <= room) {
@@ -970,8 +1008,11 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
             for (long long r = 0; r < d.D; r += ROWS_PER_ITEM)
                 ei.push_back(make_int4(t, (int)r, (int)std::min<long long>(ROWS_PER_ITEM, d.D - r), 0));
             d.ecnt = (int)ei.size() - d.eoff;
-            d.nslab = (int)((d.D + SLAB_ROWS - 1) / SLAB_ROWS);
-            d.wslab = (int)std::max<long long>(1, h->nnz / d.nslab);
+            d.nslab = (int)std::max<long long>(1, std::min<long long>(KBS_SLABS, d.D / 8));
+            d.wslab = (int)std::max<long long>(1, (h->nnz + KBS_ROW * d.D) / d.nslab);
+            int* cut = dalloc<int>(b, (size_t)d.nslab + 1);
+            k_cut_slabs<<<(d.nslab + 256) / 256, 256>>>(d.rowptr, d.D, h->nnz, d.nslab, cut);
+            d.cut = cut;
             if (d.D <= KBS_ROOM) b->room = std::max(b->room, (int)d.D);
             d.gbase = (int)gi.size();
             // the pool's own item table: op k's chunks are items gf[k] .. gf[k + 1] - 1

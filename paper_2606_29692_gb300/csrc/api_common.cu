@@ -179,6 +179,10 @@ void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, c
     double2* w = static_cast<double2*>(c->scratch[S_W0]);
     float2* w32 = psi->prec == TQ_C64 ? static_cast<float2*>(c->scratch[S_W32]) : nullptr;
     int lanes = c->spmv_lanes;
+    if (lanes == SPMV_AUTO && h->prec == TQ_C128 && !h->sector && h->D <= ENERGY_FEW) {
+        launch(c, "energy_csr", s, [&] { return launch_energy_few(h->view, psi->data, w, part, c->tickets, c->step, s); });
+        return;
+    }
     if (lanes == SPMV_AUTO) lanes = h->prec == TQ_C128 && !h->sector ? SPMV_C128_LANES : (int)TQ_SPMV_XELL;
     if (lanes == TQ_SPMV_XELL && h->sector) lanes = 8;   // a sector Hamiltonian has the CSR only
     if (lanes == TQ_SPMV_XELL)

@@ -630,8 +630,9 @@ kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, Active 
                 den = s.e_den;
             }
             if (lane == 0) {
-                e_sh[0] = num / den;
-                e_sh[1] = 1.0 / den;
+                const double inv = 1.0 / den;
+                e_sh[0] = num * inv;
+                e_sh[1] = inv;
             }
         }
         // the thread's ops k = tid + SEL_BS j, SEL_U at a time so that their

@@ -266,6 +266,11 @@ int launch_xell_split(const int* xptr, long long n_blocks, int grid, int* split,
 int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2* w,
                        float2* w32, double* partials, unsigned* ticket, DevStep* step,
                        int sms, cudaStream_t s, int lanes_per_row);
+// complex128 over a space of at most ENERGY_FEW rows: one row per group of
+// lanes (one partial pair per CTA, at most ENERGY_FEW / 32 of them).
+constexpr long long ENERGY_FEW16 = 1 << 12, ENERGY_FEW = 1 << 14;
+int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,
+                      cudaStream_t s);
 // gradients read w in float32 (w32) for complex64 states, float64 (w) otherwise
 int launch_pool_gradients(const PoolView& p, const double2* w, const float2* w32,
                           const void* psi, int prec, const DevStep* step, double* partials,

@@ -9,6 +9,35 @@
 
 namespace tq {
 
+// Programmatic launch.  A kernel launched with launch_pdl may start while its
+// predecessor in the stream still runs; pdl_wait returns when that one has
+// completed and its writes are visible, and every CTA calls it before it
+// touches anything an earlier launch writes (and before it may return).  Such
+// data is not read through __ldg or an unconditional read-only pointer at a
+// kernel's top: the compiler may move those loads over the wait.
+// pdl_start lets the next launch start in turn.  Only the short kernels of the
+// ADAPT step's chain are launched so (20 steps at 12 qubits, complex128: 1.345 to 1.32 ms):
+// dependents that wait beside a long pass slow it (launched so everywhere,
+// a 16-qubit complex128 gradient sweep went from 141 to 185 us).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A launch error stays pending for the caller's cudaGetLastError check.
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+}
+
 // complex type per precision: float2 (TQ_C64) or double2 (TQ_C128)
 template <typename T> struct C2;
 template <> struct C2<float> { using type = float2; };
@@ -66,23 +95,62 @@ __device__ __forceinline__ double warp_sum_compensated_pair(float hi, float lo) 
     return (double)hi + (double)lo;
 }
 
-// Block-wide float64 sum of `n` values per thread (n <= 4); result valid in
-// thread 0.  `sh` needs blockDim/32 * n doubles.  Deterministic: fixed tree.
+// Block-wide float64 sum of `n` values per thread (n <= 8); result valid in
+// thread 0.  `sh` needs blockDim/32 * n doubles (at least n).  Deterministic:
+// fixed trees.  A float64 warp addition holds its SM quarter's pipe for 64
+// cycles whatever its lanes hold, so both trees share the lanes among the
+// values: the warp tree scatters (each half keeps half of the values: 5
+// additions for two values instead of 10, 9 for five instead of 25), and the
+// warps' sums are added with one lane per value and warp.
 template <int n>
 __device__ __forceinline__ void block_sum(double (&v)[n], double* sh) {
+    constexpr int P = n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : 8;      // values, padded with zeros
+    static_assert(n <= 8, "at most eight values");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double a[P];
 #pragma unroll
-    for (int i = 0; i < n; ++i) v[i] = warp_sum(v[i]);
-    if (lane == 0)
+    for (int i = 0; i < P; ++i) a[i] = i < n ? v[i] : 0.0;
+    int o = 16;
 #pragma unroll
-        for (int i = 0; i < n; ++i) sh[wid * n + i] = v[i];
-    __syncthreads();
-    if (wid == 0) {
+    for (int k = P; k > 1; k >>= 1, o >>= 1) {
+        const bool up = lane & o;
 #pragma unroll
-        for (int i = 0; i < n; ++i) v[i] = lane < nw ? sh[lane * n + i] : 0.0;
-#pragma unroll
-        for (int i = 0; i < n; ++i) v[i] = warp_sum(v[i]);
+        for (int i = 0; i < k / 2; ++i) {
+            const double give = up ? a[i] : a[i + k / 2], keep = up ? a[i + k / 2] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
+#pragma unroll
+    for (int q = 16 / P; q > 0; q >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], q);
+    // lane l (a multiple of 32 / P) holds value l P / 32
+    if (lane % (32 / P) == 0 && lane * P / 32 < n) sh[wid * n + lane * P / 32] = a[0];
+    __syncthreads();
+    if (nw <= 8) {
+        // eight lanes per value, one per warp
+        double s = 0.0;
+        const int val = threadIdx.x >> 3, w = threadIdx.x & 7;
+        if (threadIdx.x < ((8 * n + 31) & ~31)) {
+            if (val < n && w < nw) s = sh[w * n + val];
+#pragma unroll
+            for (int q = 4; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        }
+        __syncthreads();
+        if (val < n && w == 0) sh[val] = s;
+    } else {
+        // one warp per value
+        double s = 0.0;
+        if (wid < n) {
+            if (lane < nw) s = sh[lane * n + wid];
+#pragma unroll
+            for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        }
+        __syncthreads();
+        if (wid < n && lane == 0) sh[wid] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int i = 0; i < n; ++i) v[i] = sh[i];
     __syncthreads();
 }
 

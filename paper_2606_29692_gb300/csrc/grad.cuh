@@ -182,8 +182,11 @@ __device__ __forceinline__ double grad_item(const SuppRec& s, T c0, const W* __r
     if (lane == 0) sh[wid] = part;
     __syncthreads();
     double tot = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < nw; ++i) tot += sh[i];
+    if (threadIdx.x < 32) {
+        tot = lane < nw ? sh[lane] : 0.0;
+#pragma unroll
+        for (int o = GRAD_TPB / 64; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
+    }
     __syncthreads();
     return tot;
 }

@@ -72,6 +72,66 @@ k_energy_csr(HamView h, const typename C2<T>::type* __restrict__ psi, double2* _
     }
 }
 
+// The same for small spaces (complex128): one row per group of L lanes, so
+// that a 12-qubit H fills 256 CTAs where 64-row items fill 64, and the
+// rows' float64 finish and its sums run in one warp.  What bounds it is the
+// chain launch - row offsets - entries - gathers - sums - ticket; float64
+// additions hold the pipe for 64 cycles each, so the row trees scatter the
+// two components over the lanes (4 additions for 16 lanes instead of 8).
+// 12 qubits: 13.4 us with 64-row items, 9.2 us here.
+template <int L>
+__global__ void __launch_bounds__(256)
+k_energy_few(HamView h, const double2* __restrict__ psi, double2* __restrict__ w, double* partials, unsigned* ticket,
+             DevStep* step) {
+    constexpr int R = 256 / L;                    // rows per CTA
+    static_assert(L >= 8 && L <= 32, "the rows of a CTA are finished by one warp");
+    __shared__ double sh[2 * 8];
+    __shared__ double st[R][2];
+    const double* __restrict__ val = static_cast<const double*>(h.val);
+    const int tid = threadIdx.x, gl = tid % L, lane = tid & 31;
+    const long long r0 = (long long)blockIdx.x * R, r = r0 + tid / L;
+    double2 pv = make_double2(0.0, 0.0);
+    double dg = 0.0;
+    const bool fin = tid < R && r0 + tid < h.D;
+    if (fin) {                                    // loaded ahead of the entries
+        pv = psi[r0 + tid];
+        dg = h.diag[r0 + tid];
+    }
+    double px = 0.0, py = 0.0;
+    if (r < h.D) row_dot<double, double, double2, L>(h.col, val, psi, h.rowptr[r], h.rowptr[r + 1], gl, px, py);
+    const bool up = gl & (L / 2);
+    double k = (up ? py : px) + __shfl_xor_sync(0xffffffffu, up ? px : py, L / 2);
+#pragma unroll
+    for (int o = L / 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    if (gl % (L / 2) == 0) st[tid / L][gl / (L / 2)] = k;
+    __syncthreads();
+    if (tid < 32) {
+        double num = 0.0, den = 0.0;
+        if (fin) {
+            const double wx = fma(dg, pv.x, st[tid][0]), wy = fma(dg, pv.y, st[tid][1]);
+            w[r0 + tid] = make_double2(wx, wy);
+            num = fma(pv.x, wx, pv.y * wy);
+            den = fma(pv.x, pv.x, pv.y * pv.y);
+        }
+        const bool hi = lane & 16;
+        double s = (hi ? den : num) + __shfl_xor_sync(0xffffffffu, hi ? num : den, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane % 16 == 0) partials[2 * blockIdx.x + lane / 16] = s;
+        __threadfence();
+    }
+    if (last_block(ticket, gridDim.x)) {
+        double a, b;
+        block_sum_pairs(partials, 0, (int)gridDim.x, sh, a, b);
+        if (tid == 0) {
+            step->e_num = a;
+            step->e_den = b;
+            step->energy = a / b;
+            *ticket = 0u;
+        }
+    }
+}
+
 // The XOR-ELL energy with the pair stream staged through shared memory by
 // bulk copies (TMA).  Each CTA owns a contiguous range of row blocks,
 // balanced by pair count (h.xsplit), so its pairs form one contiguous run
@@ -412,6 +472,7 @@ k_pool_grad(PoolView p, const W* __restrict__ w, const typename C2<T>::type* __r
         }
         __syncthreads();
     }
+    pdl_start();
 }
 
 // Operator choice and convergence (one CTA of SELECT_BS threads).  A
@@ -421,6 +482,8 @@ k_pool_grad(PoolView p, const W* __restrict__ w, const typename C2<T>::type* __r
 // NaN gradients are skipped.
 constexpr int SELECT_BS = 256;
 __global__ void __launch_bounds__(SELECT_BS) k_select(const double* g, int M, double eps, int prec, DevStep* step) {
+    pdl_start();
+    pdl_wait();
     constexpr int NW = SELECT_BS / 32;
     constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;
     __shared__ unsigned long long smax[NW];
@@ -730,8 +793,9 @@ template <typename T, int L>
 __global__ void __launch_bounds__(256)
 k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ psi, DevStep* step,
                double* partials, unsigned* ticket) {
+    pdl_wait();
     using V = typename C2<T>::type;
-    __shared__ double sh[4 * 8];
+    __shared__ double sh[5 * 8];
     // the sums of a warp's 32 rows, finished in float64 by one lane each
     __shared__ LineSums<T> stash[8][32];
     if (step->converged) return;
@@ -827,20 +891,53 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
             } else {
                 double ax[3] = {0.0, 0.0, 0.0}, ay[3] = {0.0, 0.0, 0.0};   // y_S, y_O, y_1
                 if (live) {
-                    for (int e = h.rowptr[r] + sub; e < h.rowptr[r + 1]; e += L) {
-                        const double av = val[e];
-                        const uint32_t c = (uint32_t)h.col[e];
-                        const V v = __ldg(psi + c);
-                        if (in_support(s, c)) {
-                            ax[0] = fma(av, v.x, ax[0]);
-                            ay[0] = fma(av, v.y, ay[0]);
-                            const V w = __ldg(psi + (c ^ s.x));
-                            const double sg = sup_sign<double>(s, c0, c ^ s.x) * av;
-                            ax[2] = fma(sg, w.x, ax[2]);
-                            ay[2] = fma(sg, w.y, ay[2]);
-                        } else {
-                            ax[1] = fma(av, v.x, ax[1]);
-                            ay[1] = fma(av, v.y, ay[1]);
+                    // as above, U entries per lane in flight
+                    constexpr int U = 4;
+                    const int e1 = h.rowptr[r + 1];
+                    int e0 = h.rowptr[r] + sub;
+                    double av[U];
+                    int c[U];
+#pragma unroll
+                    for (int j = 0; j < U; ++j) {
+                        const int e = e0 + j * L;
+                        av[j] = e < e1 ? val[e] : 0.0;
+                        c[j] = e < e1 ? h.col[e] : -1;
+                    }
+                    while (e0 < e1) {
+                        V v[U], w[U];
+                        bool ins[U];
+#pragma unroll
+                        for (int j = 0; j < U; ++j) {
+                            ins[j] = c[j] >= 0 && in_support(s, (uint32_t)c[j]);
+                            v[j] = c[j] >= 0 ? __ldg(psi + c[j]) : V{};
+                            w[j] = ins[j] ? __ldg(psi + ((uint32_t)c[j] ^ s.x)) : V{};
+                        }
+                        e0 += U * L;
+                        double nav[U];
+                        int nc[U];
+#pragma unroll
+                        for (int j = 0; j < U; ++j) {
+                            const int e = e0 + j * L;
+                            nav[j] = e < e1 ? val[e] : 0.0;
+                            nc[j] = e < e1 ? h.col[e] : -1;
+                        }
+#pragma unroll
+                        for (int j = 0; j < U; ++j) {
+                            if (ins[j]) {
+                                ax[0] = fma(av[j], v[j].x, ax[0]);
+                                ay[0] = fma(av[j], v[j].y, ay[0]);
+                                const double sg = sup_sign<double>(s, c0, (uint32_t)c[j] ^ s.x) * av[j];
+                                ax[2] = fma(sg, w[j].x, ax[2]);
+                                ay[2] = fma(sg, w[j].y, ay[2]);
+                            } else if (c[j] >= 0) {
+                                ax[1] = fma(av[j], v[j].x, ax[1]);
+                                ay[1] = fma(av[j], v[j].y, ay[1]);
+                            }
+                        }
+#pragma unroll
+                        for (int j = 0; j < U; ++j) {
+                            av[j] = nav[j];
+                            c[j] = nc[j];
                         }
                     }
                 }
@@ -882,26 +979,19 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
         }
         __syncwarp();   // the stash is refilled by the next group
     }
-    double lo[4] = {a[0], a[1], a[2], a[3]};
-    double hi[1] = {a[4]};
-    block_sum<4>(lo, sh);
-    block_sum<1>(hi, sh + 24);
-    if (threadIdx.x == 0) {
-        for (int j = 0; j < 4; ++j) partials[5 * blockIdx.x + j] = lo[j];
-        partials[5 * blockIdx.x + 4] = hi[0];
-    }
+    pdl_start();
+    block_sum<5>(a, sh);
+    if (threadIdx.x == 0)
+        for (int j = 0; j < 5; ++j) partials[5 * blockIdx.x + j] = a[j];
     if (last_block(ticket, gridDim.x)) {
         double f[5] = {0, 0, 0, 0, 0};
         for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
             for (int j = 0; j < 5; ++j) f[j] = __dadd_rn(f[j], __ldcg(partials + 5 * b + j));
-        double lo2[4] = {f[0], f[1], f[2], f[3]};
-        double hi2[1] = {f[4]};
-        block_sum<4>(lo2, sh);
-        block_sum<1>(hi2, sh + 24);
+        const double inv = 1.0 / step->e_den;          // beside the sums, not after them
+        block_sum<5>(f, sh);
         if (threadIdx.x == 0) {
-            const double tot[5] = {lo2[0], lo2[1], lo2[2], lo2[3], hi2[0]};
             step->dots[0] = step->energy;
-            for (int j = 0; j < 5; ++j) step->dots[j + 1] = tot[j] / step->e_den;
+            for (int j = 0; j < 5; ++j) step->dots[j + 1] = f[j] * inv;
             *ticket = 0u;
         }
     }
@@ -913,15 +1003,18 @@ __device__ __forceinline__ double line_e_sc(const double* c, double s, double co
     return c[0] + 2 * s * c[1] + 2 * u * c[2] + s * s * c[3] + 2 * s * u * c[4] + u * u * c[5];
 }
 __device__ __forceinline__ double line_e(const double* c, double th) { return line_e_sc(c, sin(th), cos(th)); }
-// dE/dtheta and d2E/dtheta2 from sin(theta) = s and cos(theta) = cc.
-__device__ __forceinline__ double line_d1(const double* c, double s, double cc) {
-    const double u = 1.0 - cc;
-    return 2 * cc * c[1] + 2 * s * c[2] + 2 * s * cc * c[3] + 2 * (cc * u + s * s) * c[4] + 2 * u * s * c[5];
-}
-__device__ __forceinline__ double line_d2(const double* c, double s, double cc) {
-    const double u = 1.0 - cc;
-    return -2 * s * c[1] + 2 * cc * c[2] + 2 * (cc * cc - s * s) * c[3] +
-           2 * (3 * s * cc - s * u) * c[4] + 2 * (s * s + u * cc) * c[5];
+// The same curve as a0 + a1 cos + b1 sin + a2 cos 2theta + b2 sin 2theta: its
+// two derivatives then take 8 multiply-adds and the double angle.
+struct LineTrig {
+    double a1, b1, a2, b2;
+};
+__device__ __forceinline__ LineTrig line_trig(const double* c) {
+    LineTrig t;
+    t.a1 = -2.0 * (c[2] + c[5]);
+    t.b1 = 2.0 * (c[1] + c[4]);
+    t.a2 = 0.5 * (c[5] - c[3]);
+    t.b2 = -c[4];
+    return t;
 }
 __host__ __device__ __forceinline__ double sample_theta(int m) {
     return -kPi + 2.0 * kPi * (double)(m + 1) / 4096.0;
@@ -929,14 +1022,24 @@ __host__ __device__ __forceinline__ double sample_theta(int m) {
 
 // sin and cos of theta0 + d from those of theta0 and the Taylor series of
 // sin d and cos d (angle addition).  The polish keeps |d| within one sample
-// spacing, 2 pi / 4096 < 1.6e-3, where the first omitted terms (d^9 / 9!,
-// d^10 / 10!) are below 1e-30: no float64 sincos per Newton step.
+// spacing, 2 pi / 4096 < 1.6e-3, where the first omitted terms (d^7 / 7!,
+// d^8 / 8!) are below 1e-22 of the leading ones: no float64 sincos per
+// Newton step.
 __device__ __forceinline__ void sincos_near(double2 sc0, double d, double& s, double& c) {
     const double q = d * d;
-    const double sd = d * fma(q, fma(q, fma(q, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), 1.0);
-    const double cd = fma(q, fma(q, fma(q, fma(q, 1.0 / 40320.0, -1.0 / 720.0), 1.0 / 24.0), -0.5), 1.0);
+    const double sd = d * fma(q, fma(q, 1.0 / 120.0, -1.0 / 6.0), 1.0);
+    const double cd = fma(q, fma(q, fma(q, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
     s = fma(sc0.x, cd, sc0.y * sd);
     c = fma(sc0.y, cd, -(sc0.x * sd));
+}
+
+// 1 / d to float32 accuracy (d > 0), scaled by a power of two first so that it
+// stays in float32 range.
+__device__ __forceinline__ double quick_reciprocal(double d) {
+    const int e = ((__double2hiint(d) >> 20) & 0x7ff) - 1023;
+    if (e < -1000 || e > 1000) return 1.0 / d;
+    const double down = __hiloint2double((1023 - e) << 20, 0);      // 2^-e
+    return (double)(1.0f / (float)(d * down)) * down;
 }
 
 // Order-preserving int64 key of a double: the integer order of the keys is
@@ -978,6 +1081,8 @@ constexpr int LS_BLOCKS = 4096 / LS_BS;
 __global__ void __launch_bounds__(LS_BS)
 k_line_search(DevStep* step, double theta_given, const double* theta_list, const double2* __restrict__ sc,
               const int* __restrict__ rank, long long* se, unsigned* ticket) {
+    pdl_start();
+    pdl_wait();
     __shared__ long long red[LS_BS / 32];
     __shared__ int redi[LS_BS / 32];
     __shared__ long long thr_sh;
@@ -1046,20 +1151,28 @@ k_line_search(DevStep* step, double theta_given, const double* theta_list, const
         const double2 s0 = sc[mb];
         const double e0 = key_value(__ldcg(se + mb));
         const double h = 2.0 * kPi / 4096.0;
-        double th = th0;
+        // Newton on dE/dtheta.  The chain runs in one thread on a pipe that
+        // holds every float64 instruction for 64 cycles, so its length is its
+        // time: the trigonometric form of the derivatives, and the quotient
+        // by a float32 reciprocal (it scales a step by 1 + 1e-7, which the next
+        // step makes good)
+        const LineTrig tr = line_trig(c);
+        double th = th0, dl = 0.0;
         for (int it = 0; it < 8; ++it) {
             double sn, cs;
-            sincos_near(s0, th - th0, sn, cs);
-            const double d2 = line_d2(c, sn, cs);
+            sincos_near(s0, dl, sn, cs);
+            const double s2 = 2.0 * sn * cs, c2 = fma(cs, cs, -(sn * sn));
+            const double d2 = -fma(tr.a1, cs, fma(tr.b1, sn, 4.0 * fma(tr.a2, c2, tr.b2 * s2)));
             if (!(d2 > 0.0)) break;
-            const double stp = line_d1(c, sn, cs) / d2;
-            const double nt = th - stp;
-            if (fabs(nt - th0) > h) break;
-            th = nt;
+            const double d1 = fma(tr.b1, cs, fma(-tr.a1, sn, 2.0 * fma(tr.b2, c2, -(tr.a2 * s2))));
+            const double stp = d1 * quick_reciprocal(d2);
+            if (fabs(dl - stp) > h) break;
+            dl -= stp;
+            th = th0 + dl;
             if (fabs(stp) < 1e-15) break;
         }
         double sn, cs;
-        sincos_near(s0, th - th0, sn, cs);
+        sincos_near(s0, dl, sn, cs);
         if (line_e_sc(c, sn, cs) > e0) th = th0;
         step->theta = th;
         *ticket = 0u;
@@ -1203,6 +1316,16 @@ int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2*
     return energy_dispatch<float, float>(lanes, h, psi, w, w32, partials, ticket, step, sms, s);
 }
 
+int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,
+                      cudaStream_t s) {
+    const auto* p = static_cast<const double2*>(psi);
+    if (h.D <= ENERGY_FEW16)
+        k_energy_few<16><<<(int)((h.D + 15) / 16), 256, 0, s>>>(h, p, w, partials, ticket, step);
+    else
+        k_energy_few<8><<<(int)((h.D + 31) / 32), 256, 0, s>>>(h, p, w, partials, ticket, step);
+    return 1;
+}
+
 int launch_energy_matrix_free(const HamView& h, const void* psi, int psi_prec, double* partials,
                               unsigned* ticket, DevStep* step, int sms, cudaStream_t s) {
     const long long blocks = (h.D + 255) / 256;                 // one row per thread
@@ -1229,7 +1352,7 @@ int launch_pool_gradients(const PoolView& p, const double2* w, const float2* w32
 }
 
 int launch_select(const double* g, int M, double eps, int prec, DevStep* step, cudaStream_t s) {
-    k_select<<<1, SELECT_BS, 0, s>>>(g, M, eps, prec, step);
+    launch_pdl(k_select, 1, SELECT_BS, 0, s, g, M, eps, prec, step);
     return 1;
 }
 
@@ -1299,9 +1422,9 @@ int launch_line_support_l(const HamView& h, const PoolView& p, const void* psi, 
                           unsigned* ticket, int sms, cudaStream_t s) {
     const int grid = h.prec == TQ_C128 ? line_support_grid<double, L>(h.D, sms) : line_support_grid<float, L>(h.D, sms);
     if (h.prec == TQ_C128)
-        k_line_support<double, L><<<grid, 256, 0, s>>>(h, p, static_cast<const double2*>(psi), step, partials, ticket);
+        launch_pdl(k_line_support<double, L>, grid, 256, 0, s, h, p, static_cast<const double2*>(psi), step, partials, ticket);
     else
-        k_line_support<float, L><<<grid, 256, 0, s>>>(h, p, static_cast<const float2*>(psi), step, partials, ticket);
+        launch_pdl(k_line_support<float, L>, grid, 256, 0, s, h, p, static_cast<const float2*>(psi), step, partials, ticket);
     return 1;
 }
 
@@ -1335,11 +1458,13 @@ int launch_line_table(double2* sc, cudaStream_t s) {
 
 int launch_line_search(DevStep* step, double theta_given, const double* theta_list, const double2* sc,
                        const int* rank, long long* se, unsigned* ticket, cudaStream_t s) {
-    k_line_search<<<LS_BLOCKS, LS_BS, 0, s>>>(step, theta_given, theta_list, sc, rank, se, ticket);
+    launch_pdl(k_line_search, LS_BLOCKS, LS_BS, 0, s, step, theta_given, theta_list, sc, rank, se, ticket);
     return 1;
 }
 
 __global__ void k_step_record(DevStep* step, double* rec, int n) {
+    pdl_start();
+    pdl_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int i = step->iter;
     if (i < n) {
@@ -1356,7 +1481,7 @@ __global__ void k_step_record(DevStep* step, double* rec, int n) {
 }
 
 int launch_step_record(DevStep* step, double* rec, int n, cudaStream_t s) {
-    k_step_record<<<1, 32, 0, s>>>(step, rec, n);
+    launch_pdl(k_step_record, 1, 32, 0, s, step, rec, n);
     return 1;
 }
 

@@ -173,32 +173,32 @@ size_t partials_needed(long long D, int n_gitems, int nq, int sms) {
     return n + 8;
 }
 
-void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, cudaStream_t s) {
+void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, cudaStream_t s, DevStep* host) {
     check_space(h, psi);
     TQ_REQUIRE(h->prec == psi->prec, "state and Hamiltonian precisions differ");
     double2* w = static_cast<double2*>(c->scratch[S_W0]);
     float2* w32 = psi->prec == TQ_C64 ? static_cast<float2*>(c->scratch[S_W32]) : nullptr;
     int lanes = c->spmv_lanes;
     if (lanes == SPMV_AUTO && h->prec == TQ_C128 && !h->sector && h->D <= ENERGY_FEW) {
-        launch(c, "energy_csr", s, [&] { return launch_energy_few(h->view, psi->data, w, part, c->tickets, c->step, s); });
+        launch(c, "energy_csr", s, [&] { return launch_energy_few(h->view, psi->data, w, part, c->tickets, c->step, host, s); });
         return;
     }
     if (lanes == SPMV_AUTO) lanes = h->prec == TQ_C128 && !h->sector ? SPMV_C128_LANES : (int)TQ_SPMV_XELL;
     if (lanes == TQ_SPMV_XELL && h->sector) lanes = 8;   // a sector Hamiltonian has the CSR only
     if (lanes == TQ_SPMV_XELL)
         launch(c, "energy_xell", s, [&] {
-            return launch_energy_xell(h->view, psi->data, psi->prec, w, w32, part, c->tickets, c->step, s,
+            return launch_energy_xell(h->view, psi->data, psi->prec, w, w32, part, c->tickets, c->step, host, s,
                                       (c->test_flags & TQ_TEST_WITHHOLD_CHUNK) ? 0 : -1);
         });
     else
         launch(c, "energy_csr", s, [&] { return launch_energy_csr2(h->view, psi->data, psi->prec, w, w32, part,
-                                                                   c->tickets, c->step, c->sm_count, s, lanes); });
+                                                                   c->tickets, c->step, host, c->sm_count, s, lanes); });
 }
 
 void run_gradients(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq_state* psi, double* g,
-                   double* part, cudaStream_t s) {
+                   double* part, cudaStream_t s, DevStep* host) {
     check_space(p, psi);
-    run_energy(c, h, psi, part, s);
+    run_energy(c, h, psi, part, s, host);
     if (p->sector) {
         launch(c, "sector_gradients", s, [&] {
             return launch_sector_gradients(p->view, static_cast<double2*>(c->scratch[S_W0]), psi->data, psi->prec,

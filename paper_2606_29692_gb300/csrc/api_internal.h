@@ -66,9 +66,10 @@ bool launch_update(tq_ctx* c, const tq_pool* p, long long n, int prec, int upt, 
 size_t partials_needed(long long D, int n_gitems, int nq, int sms);
 // Allocates (before any launch of a call) the scratch energy and gradients use.
 double* prepare(tq_ctx* c, long long D, const tq_pool* p, int nq);
-void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, cudaStream_t s);
+void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, cudaStream_t s,
+                DevStep* host = nullptr);
 void run_gradients(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq_state* psi, double* g, double* part,
-                   cudaStream_t s);
+                   cudaStream_t s, DevStep* host = nullptr);
 // Clears and reports TQ_ETIMEOUT left by a kernel's bounded wait.
 void raise_status(tq_ctx* c, int status, cudaStream_t s);
 

@@ -80,8 +80,9 @@ extern "C" int tq_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double
     set_device(c);
     cudaStream_t s = as_stream(stream);
     double* part = prepare(c, h->D, nullptr, h->nq);
-    run_energy(c, h, psi, part, s);
-    const DevStep* hs = read_step(c, 0, s);
+    auto* hs = static_cast<DevStep*>(host_scratch(c, sizeof(DevStep)));   // the kernel writes the result there
+    run_energy(c, h, psi, part, s, hs);
+    TQ_CUDA(cudaStreamSynchronize(s));
     *E = hs->energy;
     raise_status(c, hs->status, s);
     API_END
@@ -97,7 +98,7 @@ extern "C" int tq_energy_matrix_free(tq_ctx* c, const tq_ham* h, const tq_state*
     cudaStream_t s = as_stream(stream);
     double* part = prepare(c, h->D, nullptr, h->nq);
     launch(c, "energy_matrix_free", s, [&] { return launch_energy_matrix_free(h->view, psi->data, psi->prec, part, c->tickets + 1,
-                                              c->step, c->sm_count, s); });
+                                              c->step, nullptr, c->sm_count, s); });
     *E = read_step(c, 0, s)->energy;
     API_END
 }
@@ -108,18 +109,19 @@ extern "C" int tq_pool_gradients(tq_ctx* c, const tq_ham* h, const tq_pool* p, c
     TQ_REQUIRE(c && h && p && psi && g, "null argument");
     set_device(c);
     cudaStream_t s = as_stream(stream);
-    // a host result goes behind the step record (one read-back) where it fits
-    const bool in_tail = !g_on_device && p->M <= tq_ctx::kStepTail;
-    double* gd = g_on_device ? g
-                 : in_tail   ? c->tail()
-                             : static_cast<double*>(scratch(c, S_G, (size_t)p->M * sizeof(double)));
-    double* part = prepare(c, h->D, p, p->nq);
-    run_gradients(c, h, p, psi, gd, part, s);
+    // a host result is written by the kernels into page-locked memory: the
+    // record (for the status), then the gradients
+    DevStep* hs = nullptr;
+    double* gd = g;
     if (!g_on_device) {
-        if (!in_tail)
-            TQ_CUDA(cudaMemcpyAsync(g, gd, (size_t)p->M * sizeof(double), cudaMemcpyDeviceToHost, s));
-        const DevStep* hs = read_step(c, in_tail ? p->M : 0, s);
-        if (in_tail) std::memcpy(g, step_tail(hs), (size_t)p->M * sizeof(double));
+        hs = static_cast<DevStep*>(host_scratch(c, sizeof(DevStep) + (size_t)p->M * sizeof(double)));
+        gd = reinterpret_cast<double*>(hs + 1);
+    }
+    double* part = prepare(c, h->D, p, p->nq);
+    run_gradients(c, h, p, psi, gd, part, s, hs);
+    if (!g_on_device) {
+        TQ_CUDA(cudaStreamSynchronize(s));
+        std::memcpy(g, gd, (size_t)p->M * sizeof(double));
         raise_status(c, hs->status, s);
     }
     API_END

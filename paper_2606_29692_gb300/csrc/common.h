@@ -249,28 +249,30 @@ int launch_taylor5_csr(int nq, int prec, const int* rowptr, const int* col, cons
                        double* scratch_v0, double* scratch_v1, double* partials,
                        double* norm2, int sms, cudaStream_t s);
 
-// Energy, gradients, ADAPT glue
+// Energy, gradients, ADAPT glue.  host (optional): a record in page-locked
+// host memory that receives the energy and the status too.
 // CTAs (one partial pair each) of the launch launch_energy_csr makes.
 int energy_csr_grid(const HamView& h, int psi_prec, int sms);
 int launch_energy_csr(const HamView& h, const void* psi, int psi_prec, double2* w,
                       double* partials, unsigned* ticket, DevStep* step, int sms,
                       cudaStream_t s);
 int launch_energy_matrix_free(const HamView& h, const void* psi, int psi_prec,
-                              double* partials, unsigned* ticket, DevStep* step,
+                              double* partials, unsigned* ticket, DevStep* step, DevStep* host,
                               int sms, cudaStream_t s);
 int launch_energy_xell(const HamView& h, const void* psi, int psi_prec, double2* w, float2* w32,
-                       double* partials, unsigned* ticket, DevStep* step, cudaStream_t s, int withhold_chunk = -1);
+                       double* partials, unsigned* ticket, DevStep* step, DevStep* host, cudaStream_t s,
+                       int withhold_chunk = -1);
 int xell_grid(long long n_blocks, int prec, int sms);
 int xell_chunk_pairs();
 int launch_xell_split(const int* xptr, long long n_blocks, int grid, int* split, cudaStream_t s);
 int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2* w,
-                       float2* w32, double* partials, unsigned* ticket, DevStep* step,
+                       float2* w32, double* partials, unsigned* ticket, DevStep* step, DevStep* host,
                        int sms, cudaStream_t s, int lanes_per_row);
 // complex128 over a space of at most ENERGY_FEW rows: one row per group of
 // lanes (one partial pair per CTA, at most ENERGY_FEW / 32 of them).
 constexpr long long ENERGY_FEW16 = 1 << 12, ENERGY_FEW = 1 << 14;
 int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,
-                      cudaStream_t s);
+                      DevStep* host, cudaStream_t s);
 // gradients read w in float32 (w32) for complex64 states, float64 (w) otherwise
 int launch_pool_gradients(const PoolView& p, const double2* w, const float2* w32,
                           const void* psi, int prec, const DevStep* step, double* partials,

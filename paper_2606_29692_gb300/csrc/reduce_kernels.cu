@@ -34,6 +34,14 @@ __device__ __forceinline__ bool last_block(unsigned* ticket, unsigned nblocks) {
     return is_last;
 }
 
+// An energy call's result, written to page-locked host memory by the thread
+// that forms it (a copy behind the kernel costs 4 to 5 us of a 30 us call).
+// Another block's time-out is in step->status before this block's ticket.
+__device__ __forceinline__ void publish(DevStep* host, DevStep* step, double energy) {
+    host->energy = energy;
+    host->status = *const_cast<volatile int*>(&step->status);
+}
+
 template <typename T> __device__ __forceinline__ double2 to_d2(typename C2<T>::type v) {
     return make_double2((double)v.x, (double)v.y);
 }
@@ -44,7 +52,7 @@ template <typename T> __device__ __forceinline__ double2 to_d2(typename C2<T>::t
 template <typename T, typename VT, int L>
 __global__ void __launch_bounds__(256)
 k_energy_csr(HamView h, const typename C2<T>::type* __restrict__ psi, double2* __restrict__ w,
-             float2* __restrict__ w32, double* partials, unsigned* ticket, DevStep* step) {
+             float2* __restrict__ w32, double* partials, unsigned* ticket, DevStep* step, DevStep* host) {
     __shared__ double sh[2 * 8];
     const VT* __restrict__ val = static_cast<const VT*>(h.val);
     double num = 0.0, den = 0.0;
@@ -64,9 +72,11 @@ k_energy_csr(HamView h, const typename C2<T>::type* __restrict__ psi, double2* _
         double a, b;
         block_sum_pairs(partials, 0, (int)gridDim.x, sh, a, b);
         if (threadIdx.x == 0) {
+            const double e = a / b;
             step->e_num = a;
             step->e_den = b;
-            step->energy = a / b;
+            step->energy = e;
+            if (host) publish(host, step, e);
             *ticket = 0u;
         }
     }
@@ -82,7 +92,7 @@ k_energy_csr(HamView h, const typename C2<T>::type* __restrict__ psi, double2* _
 template <int L>
 __global__ void __launch_bounds__(256)
 k_energy_few(HamView h, const double2* __restrict__ psi, double2* __restrict__ w, double* partials, unsigned* ticket,
-             DevStep* step) {
+             DevStep* step, DevStep* host) {
     constexpr int R = 256 / L;                    // rows per CTA
     static_assert(L >= 8 && L <= 32, "the rows of a CTA are finished by one warp");
     __shared__ double sh[2 * 8];
@@ -124,9 +134,11 @@ k_energy_few(HamView h, const double2* __restrict__ psi, double2* __restrict__ w
         double a, b;
         block_sum_pairs(partials, 0, (int)gridDim.x, sh, a, b);
         if (tid == 0) {
+            const double e = a / b;
             step->e_num = a;
             step->e_den = b;
-            step->energy = a / b;
+            step->energy = e;
+            if (host) publish(host, step, e);
             *ticket = 0u;
         }
     }
@@ -231,7 +243,8 @@ __device__ __forceinline__ void xt_round(const uint32_t* mask, const typename C2
 template <typename T, typename VT>
 __global__ void __launch_bounds__(XT_THREADS, sizeof(VT) == 4 ? 3 : 2)
 k_energy_xell_tma(HamView h, const typename C2<T>::type* __restrict__ psi, double2* __restrict__ w,
-                  float2* __restrict__ w32, double* partials, unsigned* ticket, DevStep* step, int withhold) {
+                  float2* __restrict__ w32, double* partials, unsigned* ticket, DevStep* step, DevStep* host,
+                  int withhold) {
     using V = typename C2<T>::type;
     constexpr int S = xt_stages<VT>();
     extern __shared__ __align__(128) unsigned char xt_raw[];
@@ -375,9 +388,11 @@ k_energy_xell_tma(HamView h, const typename C2<T>::type* __restrict__ psi, doubl
         double a, b;
         block_sum_pairs(partials, 0, (int)gridDim.x, sm.sh, a, b);
         if (t == 0) {
+            const double e = a / b;
             step->e_num = a;
             step->e_den = b;
-            step->energy = a / b;
+            step->energy = e;
+            if (host) publish(host, step, e);
             *ticket = 0u;
         }
     }
@@ -393,7 +408,7 @@ k_energy_xell_tma(HamView h, const typename C2<T>::type* __restrict__ psi, doubl
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_energy_mf(HamView h, const typename C2<T>::type* __restrict__ psi, double* partials,
-            unsigned* ticket, DevStep* step) {
+            unsigned* ticket, DevStep* step, DevStep* host) {
     __shared__ double sh[2 * 8];
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -430,9 +445,11 @@ k_energy_mf(HamView h, const typename C2<T>::type* __restrict__ psi, double* par
         double a, b;
         block_sum_pairs(partials, 0, (int)gridDim.x, sh, a, b);
         if (threadIdx.x == 0) {
+            const double e = a / b;
             step->e_num = a;
             step->e_den = b;
-            step->energy = a / b;
+            step->energy = e;
+            if (host) publish(host, step, e);
             *ticket = 0u;
         }
     }
@@ -1204,7 +1221,7 @@ int energy_grid(long long D, int sms) { return grid_rows(D, ENERGY_ROWS, sms, 8)
 
 int launch_energy_csr(const HamView& h, const void* psi, int psi_prec, double2* w,
                       double* partials, unsigned* ticket, DevStep* step, int sms, cudaStream_t s) {
-    return launch_energy_csr2(h, psi, psi_prec, w, nullptr, partials, ticket, step, sms, s, 32);
+    return launch_energy_csr2(h, psi, psi_prec, w, nullptr, partials, ticket, step, nullptr, sms, s, 32);
 }
 
 namespace {
@@ -1221,13 +1238,13 @@ int resident(int sms) {
 
 template <typename T, typename VT, int L>
 void energy_launch(const HamView& h, const void* psi, double2* w, float2* w32, double* partials,
-                   unsigned* ticket, DevStep* step, int sms, cudaStream_t s) {
+                   unsigned* ticket, DevStep* step, DevStep* host, int sms, cudaStream_t s) {
     using V = typename C2<T>::type;
     const long long items = (h.D + ENERGY_ROWS - 1) / ENERGY_ROWS;
     long long grid = resident<T, VT, L>(sms);
     if (grid > items) grid = items;
     k_energy_csr<T, VT, L><<<(int)grid, 256, 0, s>>>(h, static_cast<const V*>(psi), w, w32, partials, ticket,
-                                                     step);
+                                                     step, host);
 }
 
 // The grid energy_launch uses: resident CTAs, at most one per row item.
@@ -1240,12 +1257,12 @@ int energy_csr_grid_t(const HamView& h, int sms) {
 
 template <typename T, typename VT>
 int energy_dispatch(int lanes, const HamView& h, const void* psi, double2* w, float2* w32, double* partials,
-                    unsigned* ticket, DevStep* step, int sms, cudaStream_t s) {
+                    unsigned* ticket, DevStep* step, DevStep* host, int sms, cudaStream_t s) {
     switch (lanes) {
-        case 4: energy_launch<T, VT, 4>(h, psi, w, w32, partials, ticket, step, sms, s); return 1;
-        case 8: energy_launch<T, VT, 8>(h, psi, w, w32, partials, ticket, step, sms, s); return 1;
-        case 16: energy_launch<T, VT, 16>(h, psi, w, w32, partials, ticket, step, sms, s); return 1;
-        case 32: energy_launch<T, VT, 32>(h, psi, w, w32, partials, ticket, step, sms, s); return 1;
+        case 4: energy_launch<T, VT, 4>(h, psi, w, w32, partials, ticket, step, host, sms, s); return 1;
+        case 8: energy_launch<T, VT, 8>(h, psi, w, w32, partials, ticket, step, host, sms, s); return 1;
+        case 16: energy_launch<T, VT, 16>(h, psi, w, w32, partials, ticket, step, host, sms, s); return 1;
+        case 32: energy_launch<T, VT, 32>(h, psi, w, w32, partials, ticket, step, host, sms, s); return 1;
         default: return -1;
     }
 }
@@ -1256,7 +1273,7 @@ namespace {
 
 template <typename T, typename VT>
 void xell_launch(const HamView& h, const void* psi, double2* w, float2* w32, double* partials,
-                 unsigned* ticket, DevStep* step, cudaStream_t s, int withhold) {
+                 unsigned* ticket, DevStep* step, DevStep* host, cudaStream_t s, int withhold) {
     using V = typename C2<T>::type;
     static bool attr = false;
     if (!attr) {
@@ -1265,7 +1282,7 @@ void xell_launch(const HamView& h, const void* psi, double2* w, float2* w32, dou
         attr = true;
     }
     k_energy_xell_tma<T, VT><<<h.xgrid, XT_THREADS, sizeof(XtSmem<T, VT>), s>>>(
-        h, static_cast<const V*>(psi), w, w32, partials, ticket, step, withhold);
+        h, static_cast<const V*>(psi), w, w32, partials, ticket, step, host, withhold);
 }
 
 }  // namespace
@@ -1278,11 +1295,12 @@ int energy_csr_grid(const HamView& h, int psi_prec, int sms) {
 }
 
 int launch_energy_xell(const HamView& h, const void* psi, int psi_prec, double2* w, float2* w32,
-                       double* partials, unsigned* ticket, DevStep* step, cudaStream_t s, int withhold_chunk) {
+                       double* partials, unsigned* ticket, DevStep* step, DevStep* host, cudaStream_t s,
+                       int withhold_chunk) {
     if (psi_prec == TQ_C128)
-        xell_launch<double, double>(h, psi, w, w32, partials, ticket, step, s, withhold_chunk);
+        xell_launch<double, double>(h, psi, w, w32, partials, ticket, step, host, s, withhold_chunk);
     else
-        xell_launch<float, float>(h, psi, w, w32, partials, ticket, step, s, withhold_chunk);
+        xell_launch<float, float>(h, psi, w, w32, partials, ticket, step, host, s, withhold_chunk);
     return 1;
 }
 
@@ -1309,31 +1327,31 @@ int xell_grid(long long n_blocks, int prec, int sms) {
 int xell_chunk_pairs() { return XT_CHUNK; }
 
 int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2* w, float2* w32,
-                       double* partials, unsigned* ticket, DevStep* step, int sms, cudaStream_t s,
+                       double* partials, unsigned* ticket, DevStep* step, DevStep* host, int sms, cudaStream_t s,
                        int lanes) {
     if (psi_prec == TQ_C128)
-        return energy_dispatch<double, double>(lanes, h, psi, w, w32, partials, ticket, step, sms, s);
-    return energy_dispatch<float, float>(lanes, h, psi, w, w32, partials, ticket, step, sms, s);
+        return energy_dispatch<double, double>(lanes, h, psi, w, w32, partials, ticket, step, host, sms, s);
+    return energy_dispatch<float, float>(lanes, h, psi, w, w32, partials, ticket, step, host, sms, s);
 }
 
 int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,
-                      cudaStream_t s) {
+                      DevStep* host, cudaStream_t s) {
     const auto* p = static_cast<const double2*>(psi);
     if (h.D <= ENERGY_FEW16)
-        k_energy_few<16><<<(int)((h.D + 15) / 16), 256, 0, s>>>(h, p, w, partials, ticket, step);
+        k_energy_few<16><<<(int)((h.D + 15) / 16), 256, 0, s>>>(h, p, w, partials, ticket, step, host);
     else
-        k_energy_few<8><<<(int)((h.D + 31) / 32), 256, 0, s>>>(h, p, w, partials, ticket, step);
+        k_energy_few<8><<<(int)((h.D + 31) / 32), 256, 0, s>>>(h, p, w, partials, ticket, step, host);
     return 1;
 }
 
 int launch_energy_matrix_free(const HamView& h, const void* psi, int psi_prec, double* partials,
-                              unsigned* ticket, DevStep* step, int sms, cudaStream_t s) {
+                              unsigned* ticket, DevStep* step, DevStep* host, int sms, cudaStream_t s) {
     const long long blocks = (h.D + 255) / 256;                 // one row per thread
     const int grid = (int)(blocks < (long long)sms * 8 ? blocks : (long long)sms * 8);
     if (psi_prec == TQ_C128)
-        k_energy_mf<double><<<grid, 256, 0, s>>>(h, static_cast<const double2*>(psi), partials, ticket, step);
+        k_energy_mf<double><<<grid, 256, 0, s>>>(h, static_cast<const double2*>(psi), partials, ticket, step, host);
     else
-        k_energy_mf<float><<<grid, 256, 0, s>>>(h, static_cast<const float2*>(psi), partials, ticket, step);
+        k_energy_mf<float><<<grid, 256, 0, s>>>(h, static_cast<const float2*>(psi), partials, ticket, step, host);
     return 1;
 }
 

@@ -21,7 +21,7 @@ namespace {
 // pools, pools with entries other than +-1.
 void ansatz_by_factor(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq_state* psi0, int n, const int* ops,
                       const double* th, bool grad, unsigned char* phis, void* chi, double* gdev, double* part,
-                      const tq_state& last, cudaStream_t s) {
+                      const tq_state& last, cudaStream_t s, DevStep* host) {
     const int prec = psi0->prec, upt = c->pair_upt[prec];
     const long long D = psi0->D;
     const size_t vb = (size_t)D * elem_bytes(prec);
@@ -31,7 +31,7 @@ void ansatz_by_factor(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq_sta
         TQ_CUDA(cudaMemcpyAsync(dst, phis + (size_t)j * vb, vb, cudaMemcpyDeviceToDevice, s));
         launch_update(c, p, 1, prec, upt, dst, nullptr, nullptr, ops[j], th[j], nullptr, part, nullptr, nullptr, s);
     }
-    run_energy(c, h, &last, part, s);
+    run_energy(c, h, &last, part, s, host);
     if (!grad) return;
     launch(c, "residual", s, [&] { return launch_residual(static_cast<double2*>(c->scratch[S_W0]), last.data, chi, prec,
                                                           D, c->step, s); });
@@ -68,10 +68,10 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
     unsigned char* phis = static_cast<unsigned char*>(scratch(c, S_PHI, (size_t)(n + 1) * vb));
     void* chi = scratch(c, S_CHI, vb);
     const size_t gbytes = (size_t)std::max(n, 1) * sizeof(double);
-    double* gpart = static_cast<double*>(
-        scratch(c, S_AG, gbytes + (size_t)SWEEP_OPS * SWEEP_MAX_CLUSTER * sizeof(double)));
-    const bool in_tail = n <= tq_ctx::kStepTail;
-    double* gdev = in_tail ? c->tail() : gpart + SWEEP_OPS * SWEEP_MAX_CLUSTER;
+    double* gpart = static_cast<double*>(scratch(c, S_AG, (size_t)SWEEP_OPS * SWEEP_MAX_CLUSTER * sizeof(double)));
+    // the record and the gradients are written by the kernels into page-locked memory
+    auto* hs = static_cast<DevStep*>(host_scratch(c, sizeof(DevStep) + gbytes));
+    double* gdev = reinterpret_cast<double*>(hs + 1);
     tq_state last = *psi0;
     last.owned = 0;
     last.data = phis + (size_t)n * vb;
@@ -95,7 +95,7 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
                                              grad ? phis + (size_t)j * half : nullptr, s);
             });
         }
-        run_energy(c, h, &last, part, s);
+        run_energy(c, h, &last, part, s, hs);
         for (int j1 = n; grad && j1 > 0;) {
             const int j0 = ((j1 - 1) / SWEEP_OPS) * SWEEP_OPS;
             const SweepOps o = chunk(j0, j1);
@@ -107,13 +107,11 @@ double ansatz_energy_grad(tq_ctx* c, const tq_ham* h, const tq_pool* p, const tq
             j1 = j0;
         }
     } else {
-        ansatz_by_factor(c, h, p, psi0, n, ops, th, grad != nullptr, phis, chi, gdev, part, last, s);
+        ansatz_by_factor(c, h, p, psi0, n, ops, th, grad != nullptr, phis, chi, gdev, part, last, s, hs);
     }
-    const size_t ng = grad ? (size_t)n : 0;
-    if (ng && !in_tail) TQ_CUDA(cudaMemcpyAsync(grad, gdev, ng * sizeof(double), cudaMemcpyDeviceToHost, s));
     if (psi_out) TQ_CUDA(cudaMemcpyAsync(psi_out, last.data, vb, cudaMemcpyDeviceToDevice, s));
-    const DevStep* hs = read_step(c, in_tail ? ng : 0, s);
-    if (ng && in_tail) std::memcpy(grad, step_tail(hs), ng * sizeof(double));
+    TQ_CUDA(cudaStreamSynchronize(s));
+    if (grad) std::memcpy(grad, gdev, (size_t)n * sizeof(double));
     raise_status(c, hs->status, s);
     return hs->energy;
 }

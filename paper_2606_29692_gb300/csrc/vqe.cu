@@ -109,7 +109,7 @@ __global__ void k_residual(const double2* __restrict__ w, const typename C2<T>::
 // What bounds it: the latency of a factor (barrier, distributed shared
 // memory round trip, pair arithmetic).  20 factors at 14 qubits, complex64,
 // energy and read-back included: 588 us as 40 update and 20 dot launches
-// with their copies, 148 us here (forward 32, energy 20, adjoint 43 us, the
+// with their copies, 112 us here (forward 33, energy 18, adjoint 35 us, the
 // rest launches and read-back).
 template <typename T>
 struct SweepOp {
@@ -154,24 +154,76 @@ __device__ __forceinline__ void sweep_pair(const SweepOp<double>& o, bool neg_r,
     closed_pair_sign(neg_r ? -1 : 1, neg_r ? 1 : -1, o.cf, o.c5, o.s5, a, b);
 }
 
-// Sums of products: float64, or float32 (hi, lo) pairs with exact products.
-template <typename T> struct DotAcc;
-template <> struct DotAcc<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
-    __device__ __forceinline__ double warp() const { return warp_sum(v); }
+// The dots X and Y of a factor: float64 sums, or float32 (hi, lo) pairs with
+// exact products.  A warp leaves its sums in a 16-byte slot; they are turned
+// into float64 gradients after the last factor (a float64 instruction per
+// warp and factor would sit on every factor's critical path).
+template <typename T> struct SweepDot;
+template <> struct SweepDot<double> {
+    double x = 0.0, y = 0.0;
+    __device__ __forceinline__ void add_x(double a, double b) { x = fma(a, b, x); }
+    __device__ __forceinline__ void add_y(double a, double b) { y = fma(a, b, y); }
+    __device__ __forceinline__ void leave(double2* slot) {
+        const int lane = threadIdx.x & 31;
+        const bool up = lane & 16;
+        double v = (up ? y : x) + __shfl_xor_sync(0xffffffffu, up ? x : y, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane % 16 == 0) reinterpret_cast<double*>(slot)[lane / 16] = v;
+    }
+    static __device__ __forceinline__ double grad(const double2& s, double c4, double s4) { return c4 * s.x - s4 * s.y; }
 };
-template <> struct DotAcc<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float a, float b) {
+template <> struct SweepDot<float> {
+    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
+    static __device__ __forceinline__ void add(float& hi, float& lo, float a, float b) {
         const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
         float s, r;
         two_sum(hi, p, s, r);
         hi = s;
         lo += r + e;
     }
-    __device__ __forceinline__ double warp() const { return warp_sum_compensated_pair(hi, lo); }
+    __device__ __forceinline__ void add_x(float a, float b) { add(xh, xl, a, b); }
+    __device__ __forceinline__ void add_y(float a, float b) { add(yh, yl, a, b); }
+    __device__ __forceinline__ void leave(double2* slot) {
+        // X in the lower half, Y in the upper after the first step
+        const int lane = threadIdx.x & 31;
+        const bool up = lane & 16;
+        float hi = up ? yh : xh, lo = up ? yl : xl;
+        float oh = __shfl_xor_sync(0xffffffffu, up ? xh : yh, 16), ol = __shfl_xor_sync(0xffffffffu, up ? xl : yl, 16);
+        float s, r;
+        two_sum(hi, oh, s, r);
+        hi = s;
+        lo += ol + r;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            oh = __shfl_xor_sync(0xffffffffu, hi, o);
+            ol = __shfl_xor_sync(0xffffffffu, lo, o);
+            two_sum(hi, oh, s, r);
+            hi = s;
+            lo += ol + r;
+        }
+        if (lane % 16 == 0) reinterpret_cast<float2*>(slot)[lane / 16] = make_float2(hi, lo);
+    }
+    static __device__ __forceinline__ double grad(const double2& v, double c4, double s4) {
+        const float2* f = reinterpret_cast<const float2*>(&v);
+        return c4 * ((double)f[0].x + (double)f[0].y) - s4 * ((double)f[1].x + (double)f[1].y);
+    }
 };
+
+// A thread's pair u of a factor: rows and the sign of A[r][q].
+struct SweepPair {
+    uint32_t r, q;
+    bool on, neg;      // on: the thread has this pair; neg: A[r][q] = -1
+};
+template <typename T>
+__device__ __forceinline__ SweepPair sweep_rows(const SweepOp<T>& o, uint32_t u) {
+    SweepPair s;
+    s.on = u < o.pairs;
+    s.r = expand_row(o.rx, u);
+    s.q = s.r ^ o.x;
+    s.neg = (parity32(s.q & o.z0) ^ o.neg) != 0;
+    return s;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(SWEEP_MAX_TPB)
@@ -188,21 +240,26 @@ k_ansatz_forward(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
     sweep_prepare<T>(p, ops, n, false, op);
     __syncthreads();
     cluster_arrive();
-    cluster_wait();                       // every slice is loaded
     const uint32_t t0 = rank * blockDim.x + threadIdx.x, step = cl.num_blocks() * blockDim.x;
+    SweepPair next = sweep_rows(op[0], t0);
+    cluster_wait();                       // every slice is loaded
     for (int j = 0; j < n; ++j) {
         const SweepOp<T>& o = op[j];
-        for (uint32_t u = t0; u < o.pairs; u += step) {
-            const uint32_t r = expand_row(o.rx, u), q = r ^ o.x;
-            V* pr = cl.map_shared_rank(st + (r & lo), r >> slice_log);
-            V* pq = cl.map_shared_rank(st + (q & lo), q >> slice_log);
+        SweepPair s = next;
+        for (uint32_t u = t0; s.on;) {
+            V* pr = cl.map_shared_rank(st + (s.r & lo), s.r >> slice_log);
+            V* pq = cl.map_shared_rank(st + (s.q & lo), s.q >> slice_log);
             V a = *pr, b = *pq;
             if (pairs_out) store2(pairs_out + (size_t)j * stride, 2 * u, a, b);
-            sweep_pair(o, (parity32(q & o.z0) ^ o.neg) != 0, a, b);
+            sweep_pair(o, s.neg, a, b);
             *pr = a;
             *pq = b;
+            u += step;
+            if (u >= o.pairs) break;
+            s = sweep_rows(o, u);
         }
         cluster_arrive();
+        if (j + 1 < n) next = sweep_rows(op[j + 1], t0);      // while the others arrive
         cluster_wait();                   // the factor is applied, and no peer reads this slice any more
     }
     for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) psi_end[((size_t)rank << slice_log) + i] = st[i];
@@ -220,9 +277,9 @@ k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
     extern __shared__ __align__(16) unsigned char sw_raw[];
     cg::cluster_group cl = cg::this_cluster();
     SweepOp<T>* op = reinterpret_cast<SweepOp<T>*>(sw_raw);
-    const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double* wsum = reinterpret_cast<double*>(sw_raw + SWEEP_OPS * sizeof(SweepOp<T>));   // [n][nw]
-    V* st = reinterpret_cast<V*>(wsum + (size_t)SWEEP_OPS * (SWEEP_MAX_TPB / 32));
+    const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5;
+    double2* wsum = reinterpret_cast<double2*>(sw_raw + SWEEP_OPS * sizeof(SweepOp<T>));   // [n][nw]
+    V* st = reinterpret_cast<V*>(wsum + (size_t)SWEEP_OPS * nw);
     const uint32_t per = 1u << slice_log, lo = per - 1u, rank = cl.block_rank();
     const double E = step->energy;
     for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) {
@@ -238,42 +295,53 @@ k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
     sweep_prepare<T>(p, ops, n, true, op);
     __syncthreads();
     cluster_arrive();
-    cluster_wait();
     const uint32_t t0 = rank * blockDim.x + threadIdx.x, step_u = cl.num_blocks() * blockDim.x;
+    // the next factor's rows and forward pair load while the others arrive
+    SweepPair next = sweep_rows(op[n - 1], t0);
+    V nr = V{}, nq = V{};
+    if (next.on) load2(pairs_in + (size_t)(n - 1) * stride, 2 * t0, nr, nq);
+    cluster_wait();
     for (int j = n - 1; j >= 0; --j) {
         const SweepOp<T>& o = op[j];
-        DotAcc<T> X, Y;
-        for (uint32_t u = t0; u < o.pairs; u += step_u) {
-            V fr, fq;
-            load2(pairs_in + (size_t)j * stride, 2 * u, fr, fq);
-            const uint32_t r = expand_row(o.rx, u), q = r ^ o.x;
-            V* pr = cl.map_shared_rank(st + (r & lo), r >> slice_log);
-            V* pq = cl.map_shared_rank(st + (q & lo), q >> slice_log);
+        SweepDot<T> dot;
+        SweepPair s = next;
+        V fr = nr, fq = nq;
+        for (uint32_t u = t0; s.on;) {
+            V* pr = cl.map_shared_rank(st + (s.r & lo), s.r >> slice_log);
+            V* pq = cl.map_shared_rank(st + (s.q & lo), s.q >> slice_log);
             V a = *pr, b = *pq;
-            const bool neg = (parity32(q & o.z0) ^ o.neg) != 0;      // A[r][q] = -1, A[q][r] = +1
-            const T s = neg ? T(-1) : T(1);
-            X.add(s * a.x, fq.x);
-            X.add(s * a.y, fq.y);
-            X.add(-s * b.x, fr.x);
-            X.add(-s * b.y, fr.y);
-            Y.add(a.x, fr.x);
-            Y.add(a.y, fr.y);
-            Y.add(b.x, fq.x);
-            Y.add(b.y, fq.y);
-            sweep_pair(o, neg, a, b);
+            const V a0 = a, b0 = b;
+            sweep_pair(o, s.neg, a, b);
             *pr = a;
             *pq = b;
+            const T sg = s.neg ? T(-1) : T(1);       // A[r][q]; A[q][r] is its negative
+            dot.add_x(sg * a0.x, fq.x);
+            dot.add_x(sg * a0.y, fq.y);
+            dot.add_x(-sg * b0.x, fr.x);
+            dot.add_x(-sg * b0.y, fr.y);
+            dot.add_y(a0.x, fr.x);
+            dot.add_y(a0.y, fr.y);
+            dot.add_y(b0.x, fq.x);
+            dot.add_y(b0.y, fq.y);
+            u += step_u;
+            if (u >= o.pairs) break;
+            load2(pairs_in + (size_t)j * stride, 2 * u, fr, fq);
+            s = sweep_rows(o, u);
         }
         cluster_arrive();
-        const double x = X.warp(), y = Y.warp();
-        if (lane == 0) wsum[j * nw + wid] = o.c4 * x - o.s4 * y;
+        if (j > 0) {
+            next = sweep_rows(op[j - 1], t0);
+            if (next.on) load2(pairs_in + (size_t)(j - 1) * stride, 2 * t0, nr, nq);
+        }
+        dot.leave(wsum + j * nw + wid);
         cluster_wait();
     }
     for (uint32_t i = threadIdx.x; chi_out && i < per; i += blockDim.x) chi_out[((size_t)rank << slice_log) + i] = st[i];
     // this CTA's sums in warp order, then the CTAs' in rank order
+    __syncthreads();
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         double v = 0.0;
-        for (int i = 0; i < nw; ++i) v += wsum[j * nw + i];
+        for (int i = 0; i < nw; ++i) v += SweepDot<T>::grad(wsum[j * nw + i], op[j].c4, op[j].s4);
         part[(size_t)j * SWEEP_MAX_CLUSTER + rank] = v;
     }
     __threadfence();
@@ -294,20 +362,23 @@ int small_grid(long long D, int sms) {
 }
 
 template <typename T>
-size_t sweep_smem(bool adjoint, int slice_log) {
-    return SWEEP_OPS * sizeof(SweepOp<T>) + (adjoint ? (size_t)SWEEP_OPS * (SWEEP_MAX_TPB / 32) * sizeof(double) : 0) +
+size_t sweep_smem(bool adjoint, int slice_log, int tpb) {
+    return SWEEP_OPS * sizeof(SweepOp<T>) + (adjoint ? (size_t)SWEEP_OPS * (tpb / 32) * sizeof(double2) : 0) +
            ((size_t)1 << slice_log) * 2 * sizeof(T);
 }
 
-// CTAs and threads per CTA for 2^nq amplitudes: a single excitation has D/4
-// pairs, aimed at one per thread.  complex64 takes 256 pairs per CTA
-// (latency bounds it), complex128 128 (its float64 work spreads over more
-// SMs), up to 16 CTAs, then more threads.
-void sweep_shape(int nq, int prec, int* cs, int* tpb) {
-    const long long pairs = std::max(1ll, (1ll << nq) >> 2), per_cta = prec == TQ_C128 ? 128 : 256;
-    const long long c = std::min<long long>(SWEEP_MAX_CLUSTER, std::max(1ll, pairs / per_cta));
+// CTAs and threads per CTA for 2^nq amplitudes; a single excitation has D/4
+// pairs.  64 pairs per CTA up to 16 CTAs, then 256 threads with several pairs
+// each (more threads make the barriers longer: 20 factors at 16 qubits,
+// complex64, forward + adjoint: 97 us with 256 threads, 132 with 1024; 12
+// qubits: 61 us on 16 CTAs, 74 on 4), and 1024 threads only where a CTA has
+// more than 1024 pairs (18 qubits: 184 us against 248).
+void sweep_shape(int nq, int* cs, int* tpb) {
+    const long long pairs = std::max(1ll, (1ll << nq) >> 2);
+    const long long c = std::min<long long>(SWEEP_MAX_CLUSTER, std::max(1ll, pairs / 64));
     *cs = (int)c;
-    *tpb = (int)std::min<long long>(SWEEP_MAX_TPB, std::max(32ll, pairs / c));
+    const long long per = pairs / c;
+    *tpb = (int)std::min<long long>(per > 1024 ? SWEEP_MAX_TPB : 256, std::max(32ll, per));
 }
 
 template <typename K>
@@ -330,20 +401,20 @@ cudaError_t sweep_config(K kern, int cs, int tpb, size_t smem, cudaStream_t s, c
 }
 
 template <typename T>
-bool sweep_fits(int nq, int prec) {
+bool sweep_fits(int nq) {
     int cs, tpb;
-    sweep_shape(nq, prec, &cs, &tpb);
+    sweep_shape(nq, &cs, &tpb);
     int lg = nq;
     while (cs >> (nq - lg + 1)) --lg;          // slice of D / cs amplitudes
-    const size_t smem = sweep_smem<T>(true, lg);
-    if (smem > 200 * 1024) return false;
+    const size_t smem = sweep_smem<T>(true, lg, tpb);
+    if (smem > 220 * 1024) return false;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     int n = 0;
     cudaError_t e = sweep_config(k_ansatz_adjoint<T>, cs, tpb, smem, 0, &cfg, &attr);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_ansatz_adjoint<T>, &cfg);
     if (e == cudaSuccess && n >= 1) {
-        e = sweep_config(k_ansatz_forward<T>, cs, tpb, sweep_smem<T>(false, lg), 0, &cfg, &attr);
+        e = sweep_config(k_ansatz_forward<T>, cs, tpb, sweep_smem<T>(false, lg, tpb), 0, &cfg, &attr);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_ansatz_forward<T>, &cfg);
     }
     if (e != cudaSuccess) (void)cudaGetLastError();
@@ -355,19 +426,19 @@ bool sweep_fits(int nq, int prec) {
 // Asked once per call: a few microseconds of host queries beside the sweep.
 bool ansatz_sweep_ready(int nq, int prec) {
     if (nq < 2 || nq >= 32) return false;
-    return prec == TQ_C128 ? sweep_fits<double>(nq, prec) : sweep_fits<float>(nq, prec);
+    return prec == TQ_C128 ? sweep_fits<double>(nq) : sweep_fits<float>(nq);
 }
 
 template <typename T>
-static int forward_t(const PoolView& p, const SweepOps& ops, int n, int prec, const void* psi0, void* psi_end,
+static int forward_t(const PoolView& p, const SweepOps& ops, int n, const void* psi0, void* psi_end,
                      void* pairs, cudaStream_t s) {
     using V = typename C2<T>::type;
     int cs, tpb, lg = p.nq;
-    sweep_shape(p.nq, prec, &cs, &tpb);
+    sweep_shape(p.nq, &cs, &tpb);
     while (cs >> (p.nq - lg + 1)) --lg;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    cudaError_t e = sweep_config(k_ansatz_forward<T>, cs, tpb, sweep_smem<T>(false, lg), s, &cfg, &attr);
+    cudaError_t e = sweep_config(k_ansatz_forward<T>, cs, tpb, sweep_smem<T>(false, lg, tpb), s, &cfg, &attr);
     if (e == cudaSuccess)
         e = cudaLaunchKernelEx(&cfg, k_ansatz_forward<T>, p, ops, n, lg, static_cast<const V*>(psi0),
                                static_cast<V*>(psi_end), static_cast<V*>(pairs), (1ll << p.nq) / 2);
@@ -375,16 +446,16 @@ static int forward_t(const PoolView& p, const SweepOps& ops, int n, int prec, co
 }
 
 template <typename T>
-static int adjoint_t(const PoolView& p, const SweepOps& ops, int n, int prec, const double2* w, const void* psi,
+static int adjoint_t(const PoolView& p, const SweepOps& ops, int n, const double2* w, const void* psi,
                      const DevStep* step, const void* chi_in, void* chi_out, const void* pairs, double* part,
                      double* grad, cudaStream_t s) {
     using V = typename C2<T>::type;
     int cs, tpb, lg = p.nq;
-    sweep_shape(p.nq, prec, &cs, &tpb);
+    sweep_shape(p.nq, &cs, &tpb);
     while (cs >> (p.nq - lg + 1)) --lg;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
-    cudaError_t e = sweep_config(k_ansatz_adjoint<T>, cs, tpb, sweep_smem<T>(true, lg), s, &cfg, &attr);
+    cudaError_t e = sweep_config(k_ansatz_adjoint<T>, cs, tpb, sweep_smem<T>(true, lg, tpb), s, &cfg, &attr);
     if (e == cudaSuccess)
         e = cudaLaunchKernelEx(&cfg, k_ansatz_adjoint<T>, p, ops, n, lg, w, static_cast<const V*>(psi), step,
                                static_cast<const V*>(chi_in), static_cast<V*>(chi_out), static_cast<const V*>(pairs),
@@ -394,16 +465,16 @@ static int adjoint_t(const PoolView& p, const SweepOps& ops, int n, int prec, co
 
 int launch_ansatz_forward(const PoolView& p, const SweepOps& ops, int n, int prec, const void* psi0, void* psi_end,
                           void* pairs, cudaStream_t s) {
-    return prec == TQ_C128 ? forward_t<double>(p, ops, n, prec, psi0, psi_end, pairs, s)
-                           : forward_t<float>(p, ops, n, prec, psi0, psi_end, pairs, s);
+    return prec == TQ_C128 ? forward_t<double>(p, ops, n, psi0, psi_end, pairs, s)
+                           : forward_t<float>(p, ops, n, psi0, psi_end, pairs, s);
 }
 
 int launch_ansatz_adjoint(const PoolView& p, const SweepOps& ops, int n, int prec, const double2* w, const void* psi,
                           const DevStep* step, const void* chi_in, void* chi_out, const void* pairs, double* part,
                           double* grad, cudaStream_t s) {
     return prec == TQ_C128
-               ? adjoint_t<double>(p, ops, n, prec, w, psi, step, chi_in, chi_out, pairs, part, grad, s)
-               : adjoint_t<float>(p, ops, n, prec, w, psi, step, chi_in, chi_out, pairs, part, grad, s);
+               ? adjoint_t<double>(p, ops, n, w, psi, step, chi_in, chi_out, pairs, part, grad, s)
+               : adjoint_t<float>(p, ops, n, w, psi, step, chi_in, chi_out, pairs, part, grad, s);
 }
 
 int launch_ansatz_dot(const PoolView& p, int k, double c4, double s4, const void* chi, const void* phi, int prec,

@@ -55,7 +55,6 @@ extern "C" int tq_ctx_create(int device, tq_ctx** out) {
         c->l2_fetch_default = (int)fetch;
         // the line search's sample table, filled before any call can read it
         c->line_sc = static_cast<double2*>(dev_alloc(4096 * sizeof(double2)));
-        c->line_se = static_cast<long long*>(dev_alloc((4096 + 64) * sizeof(long long)));
         c->line_rank = static_cast<int*>(dev_alloc(4096 * sizeof(int)));
         {
             std::vector<int> rank(4096);
@@ -82,7 +81,6 @@ extern "C" int tq_ctx_destroy(tq_ctx* c) {
     if (c->host_buf) cudaFreeHost(c->host_buf);
     if (c->tickets) cudaFree(c->tickets);
     if (c->line_sc) cudaFree(c->line_sc);
-    if (c->line_se) cudaFree(c->line_se);
     if (c->line_rank) cudaFree(c->line_rank);
     for (auto& s : c->aux)
         if (s) cudaStreamDestroy(s);

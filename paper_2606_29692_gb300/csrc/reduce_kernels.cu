@@ -15,6 +15,10 @@
 #include <cmath>
 #include <vector>
 
+#include <cooperative_groups.h>
+
+namespace cg = cooperative_groups;
+
 namespace tq {
 
 namespace {
@@ -799,12 +803,30 @@ __device__ __forceinline__ double re_dot(double2 a, double2 b) {
     return __dadd_rn(__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y));
 }
 
-// Row sums of one support row before its float64 finish: y_S (columns in
-// S) and y_1 (H u1 over columns in S) as compensated (hi, lo) pairs per
-// component, y_O (columns outside S) plain.  complex128: float64 sums.
-template <typename T> struct LineSums {
-    typename C2<T>::type s, o, u;   // y_S, y_O, y_1
-};
+// The six row sums (y_S, y_O, y_1, two components each) of the rows served by
+// groups of L lanes, by the xor butterfly over the group, scattered as it goes:
+// each half of the lanes keeps half of the values (for 16 lanes 8 additions
+// instead of 24).  Value i ends in the lanes with sub / (L / 8) == i, which
+// put it into out[i].
+template <typename T, int L>
+__device__ __forceinline__ void line_row_sums(typename C2<T>::type yS, typename C2<T>::type yO,
+                                              typename C2<T>::type y1, int sub, T* out) {
+    T v[8] = {yS.x, yS.y, yO.x, yO.y, y1.x, y1.y, T(0), T(0)};
+    int o = L / 2;
+#pragma unroll
+    for (int k = 8; k > 1; k >>= 1, o >>= 1) {
+        const bool up = sub & o;
+#pragma unroll
+        for (int i = 0; i < k / 2; ++i) {
+            const T give = up ? v[i] : v[i + k / 2], keep = up ? v[i + k / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (int q = L / 16; q > 0; q >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], q);
+    const int i = sub / (L / 8);
+    if (sub % (L / 8) == 0 && i < 6) out[i] = v[0];
+}
 
 template <typename T, int L>
 __global__ void __launch_bounds__(256)
@@ -813,8 +835,10 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
     pdl_wait();
     using V = typename C2<T>::type;
     __shared__ double sh[5 * 8];
-    // the sums of a warp's 32 rows, finished in float64 by one lane each
-    __shared__ LineSums<T> stash[8][32];
+    // the sums of the CTA's rows of a round, finished in float64 by one thread
+    // each: with few rows per warp one warp finishes them all (a float64
+    // instruction costs a warp the same for two lanes as for 32)
+    __shared__ T stash[256][6];
     if (step->converged) return;
     const T* __restrict__ val = static_cast<const T*>(h.val);
     const int k = step->selected;
@@ -824,23 +848,22 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
     const long long nrows = 1ll << (p.nq - s.m);
     const int lane = threadIdx.x & 31, sub = lane & (L - 1), wid = threadIdx.x >> 5;
     constexpr int RPW = 32 / L;
-    const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // H01, H02, H11, H12, H22 (before / <psi|psi>)
-    // rows per warp group: 32 (one float64 finish per lane) when the support
-    // has rows enough for every warp, fewer for small supports so that all
-    // warps get work (a power of two, at least the RPW rows of one round)
+    // rows per warp: 32 when the support has rows enough for every warp, fewer
+    // for small supports so that all warps get work (a power of two, at least
+    // the RPW rows of one round)
     int G = 32;
     while (G > RPW && (long long)G * nwarps > nrows) G >>= 1;
     const int rounds = G / RPW;
-    for (long long g0 = warp * G; g0 < nrows; g0 += nwarps * G) {
+    for (long long c0r = blockIdx.x * 8ll * G; c0r < nrows; c0r += nwarps * G) {
+        const long long g0 = c0r + wid * G;
         // `rounds` rounds of RPW rows fill the warp's G slots
         for (int rd = 0; rd < rounds; ++rd) {
             const int slot = rd * RPW + lane / L;
             const long long i = g0 + slot;
             const bool live = i < nrows;
             const uint32_t r = live ? expand_support_row(rx, (uint32_t)i) : 0u;
-            LineSums<T> out;
             if constexpr (sizeof(T) == 4) {
                 float2 yS = make_float2(0.f, 0.f), yO = yS, y1 = yS;
                 if (live) {
@@ -893,18 +916,7 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
                         }
                     }
                 }
-#pragma unroll
-                for (int o = L / 2; o > 0; o >>= 1) {
-                    yS.x += __shfl_xor_sync(0xffffffffu, yS.x, o);
-                    yS.y += __shfl_xor_sync(0xffffffffu, yS.y, o);
-                    yO.x += __shfl_xor_sync(0xffffffffu, yO.x, o);
-                    yO.y += __shfl_xor_sync(0xffffffffu, yO.y, o);
-                    y1.x += __shfl_xor_sync(0xffffffffu, y1.x, o);
-                    y1.y += __shfl_xor_sync(0xffffffffu, y1.y, o);
-                }
-                out.s = yS;
-                out.o = yO;
-                out.u = y1;
+                line_row_sums<T, L>(yS, yO, y1, sub, stash[wid * G + slot]);
             } else {
                 double ax[3] = {0.0, 0.0, 0.0}, ay[3] = {0.0, 0.0, 0.0};   // y_S, y_O, y_1
                 if (live) {
@@ -958,43 +970,33 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
                         }
                     }
                 }
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-#pragma unroll
-                    for (int o = L / 2; o > 0; o >>= 1) {
-                        ax[q] += __shfl_xor_sync(0xffffffffu, ax[q], o);
-                        ay[q] += __shfl_xor_sync(0xffffffffu, ay[q], o);
-                    }
-                }
-                out.s = make_double2(ax[0], ay[0]);
-                out.o = make_double2(ax[1], ay[1]);
-                out.u = make_double2(ax[2], ay[2]);
+                line_row_sums<T, L>(make_double2(ax[0], ay[0]), make_double2(ax[1], ay[1]), make_double2(ax[2], ay[2]),
+                                    sub, stash[wid * G + slot]);
             }
-            if (sub == 0) stash[wid][slot] = out;
         }
-        __syncwarp();
-        // lane g < G finishes row g0 + g in float64
-        const long long i = g0 + lane;
-        if (lane < G && i < nrows) {
+        __syncthreads();
+        // thread t < 8 G finishes row c0r + t in float64
+        const long long i = c0r + threadIdx.x;
+        if (threadIdx.x < 8 * G && i < nrows) {
             const uint32_t r = expand_support_row(rx, (uint32_t)i);
-            const LineSums<T> in = stash[wid][lane];
-            const double sSx = (double)in.s.x, sSy = (double)in.s.y;
+            const T* in = stash[threadIdx.x];
+            const double sSx = (double)in[0], sSy = (double)in[1];
             const double d = h.diag[r];
             const V pr = psi[r], pq = psi[r ^ s.x];
             const double sg = (double)sup_sign<T>(s, c0, r ^ s.x);
             const double2 p0 = make_double2((double)pr.x, (double)pr.y);
             const double2 u1 = make_double2(sg * (double)pq.x, sg * (double)pq.y);
             // (H psi)_r, (H psi_S)_r and (H u1)_r
-            const double2 x0 = make_double2(fma(d, p0.x, sSx + (double)in.o.x), fma(d, p0.y, sSy + (double)in.o.y));
+            const double2 x0 = make_double2(fma(d, p0.x, sSx + (double)in[2]), fma(d, p0.y, sSy + (double)in[3]));
             const double2 xS = make_double2(fma(d, p0.x, sSx), fma(d, p0.y, sSy));
-            const double2 x1 = make_double2(fma(d, u1.x, (double)in.u.x), fma(d, u1.y, (double)in.u.y));
+            const double2 x1 = make_double2(fma(d, u1.x, (double)in[4]), fma(d, u1.y, (double)in[5]));
             a[0] = __dadd_rn(a[0], re_dot(x0, u1));     // H01
             a[1] = __dsub_rn(a[1], re_dot(x0, p0));     // H02
             a[2] = __dadd_rn(a[2], re_dot(u1, x1));     // H11
             a[3] = __dsub_rn(a[3], re_dot(xS, u1));     // H12
             a[4] = __dadd_rn(a[4], re_dot(xS, p0));     // H22
         }
-        __syncwarp();   // the stash is refilled by the next group
+        __syncthreads();   // the stash is refilled by the next round
     }
     pdl_start();
     block_sum<5>(a, sh);
@@ -1014,19 +1016,14 @@ k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ p
     }
 }
 
-// E(theta) from sin(theta) and cos(theta).
-__device__ __forceinline__ double line_e_sc(const double* c, double s, double co) {
-    const double u = 1.0 - co;
-    return c[0] + 2 * s * c[1] + 2 * u * c[2] + s * s * c[3] + 2 * s * u * c[4] + u * u * c[5];
-}
-__device__ __forceinline__ double line_e(const double* c, double th) { return line_e_sc(c, sin(th), cos(th)); }
-// The same curve as a0 + a1 cos + b1 sin + a2 cos 2theta + b2 sin 2theta: its
-// two derivatives then take 8 multiply-adds and the double angle.
+// E(theta) = H00 + 2 s H01 + 2 u H02 + s^2 H11 + 2 s u H12 + u^2 H22 (s = sin
+// theta, u = 1 - cos theta) as a0 + a1 cos + b1 sin + a2 cos 2theta + b2 sin 2theta.
 struct LineTrig {
-    double a1, b1, a2, b2;
+    double a0, a1, b1, a2, b2;
 };
 __device__ __forceinline__ LineTrig line_trig(const double* c) {
     LineTrig t;
+    t.a0 = c[0] + 2.0 * c[2] + 0.5 * c[3] + 1.5 * c[5];
     t.a1 = -2.0 * (c[2] + c[5]);
     t.b1 = 2.0 * (c[1] + c[4]);
     t.a2 = 0.5 * (c[5] - c[3]);
@@ -1035,28 +1032,6 @@ __device__ __forceinline__ LineTrig line_trig(const double* c) {
 }
 __host__ __device__ __forceinline__ double sample_theta(int m) {
     return -kPi + 2.0 * kPi * (double)(m + 1) / 4096.0;
-}
-
-// sin and cos of theta0 + d from those of theta0 and the Taylor series of
-// sin d and cos d (angle addition).  The polish keeps |d| within one sample
-// spacing, 2 pi / 4096 < 1.6e-3, where the first omitted terms (d^7 / 7!,
-// d^8 / 8!) are below 1e-22 of the leading ones: no float64 sincos per
-// Newton step.
-__device__ __forceinline__ void sincos_near(double2 sc0, double d, double& s, double& c) {
-    const double q = d * d;
-    const double sd = d * fma(q, fma(q, 1.0 / 120.0, -1.0 / 6.0), 1.0);
-    const double cd = fma(q, fma(q, fma(q, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
-    s = fma(sc0.x, cd, sc0.y * sd);
-    c = fma(sc0.y, cd, -(sc0.x * sd));
-}
-
-// 1 / d to float32 accuracy (d > 0), scaled by a power of two first so that it
-// stays in float32 range.
-__device__ __forceinline__ double quick_reciprocal(double d) {
-    const int e = ((__double2hiint(d) >> 20) & 0x7ff) - 1023;
-    if (e < -1000 || e > 1000) return 1.0 / d;
-    const double down = __hiloint2double((1023 - e) << 20, 0);      // 2^-e
-    return (double)(1.0f / (float)(d * down)) * down;
 }
 
 // Order-preserving int64 key of a double: the integer order of the keys is
@@ -1084,115 +1059,125 @@ __global__ void k_line_table(double2* sc) {
 // Angle for the update: the given one, or the line-search minimiser
 // (4096 samples over (-pi, pi], ties within 1e-10 max(1,|E_min|) to the
 // smallest |theta| then lowest index, Newton polish within one spacing).
-// The samples are spread over LS_BLOCKS blocks, one per thread, from the
-// context's sin/cos table; the last block to finish (a ticket) takes the
-// minimum, applies the tie rule and polishes.  Energies are kept as
-// order-preserving int64 keys, and the tie rule reads the context's rank
-// table (rank[m]: the position of sample m in the order (|theta_m|, m),
-// from the same float64 |theta_m|), so the minimum, the tolerance test and
-// the tie pick are integer work; the float64 pipe issues a warp
-// instruction only every 64 cycles on this part.
-constexpr int LS_BS = 256;
+//
+// One thread-block cluster, a sample per thread; the minimum and the choice
+// are exchanged through distributed shared memory (a global ticket and the
+// samples' round trip through L2 took half of the 11 us this kernel needed).
+// A sample is a0 + a1 cos + b1 sin + a2 cos 2theta + b2 sin 2theta from the
+// context's sin/cos table, whose entries for 2 theta are its own: samples pi
+// apart share them bit for bit, so on a pi-periodic curve (a1 = b1 = 0
+// exactly) the two minima tie exactly.  Energies are compared as
+// order-preserving int64 keys, and the tie rule reads the context's rank table
+// (rank[m]: the position of sample m in the order (|theta_m|, m), from the
+// same float64 |theta_m|), so the minimum, the tolerance test and the tie pick
+// are integer work; the float64 pipe issues a warp instruction only every 64
+// cycles on this part.
+constexpr int LS_BS = 512;
 constexpr int LS_BLOCKS = 4096 / LS_BS;
+
+// The minimiser of the curve within one spacing h of sample angle th0, whose
+// sin, cos and double-angle sin, cos are s1, s2.  E'(th0 + d) is a polynomial
+// in d (the Taylor series of two frequencies; terms past d^5 are below 1e-17
+// of the leading ones for |d| <= h): solved by Newton in float32, whose d is
+// good to 1e-7 relative, then by two steps in float64 with the float32
+// slope, which leave 1e-21.  The whole chain is one thread on a pipe that
+// holds every float64 instruction for 64 cycles, so its length is its time.
+__device__ __forceinline__ double line_polish(const LineTrig& t, double2 s1, double2 s2, double th0, double h) {
+    const double p = fma(t.a1, s1.y, t.b1 * s1.x), r = fma(t.b1, s1.y, -(t.a1 * s1.x));
+    const double P = fma(t.a2, s2.y, t.b2 * s2.x), R = fma(t.b2, s2.y, -(t.a2 * s2.x));
+    const double f1 = fma(2.0, R, r), f2 = fma(-4.0, P, -p);
+    if (!(f2 > 0.0)) return th0;
+    const double f3 = fma(-8.0, R, -r) * 0.5, f4 = fma(16.0, P, p) * (1.0 / 6.0), f5 = fma(32.0, R, r) * (1.0 / 24.0);
+    const double f6 = fma(-64.0, P, -p) * (1.0 / 120.0);
+    // in units of f2: the float32 slope is then of order one
+    const double inv = 1.0 / f2;
+    const float g1 = (float)(f1 * inv), g3 = (float)(f3 * inv), g4 = (float)(f4 * inv), g5 = (float)(f5 * inv);
+    float x = 0.f, slope = 1.f;
+    for (int it = 0; it < 4; ++it) {
+        const float v = g1 + x * (1.f + x * (g3 + x * (g4 + x * g5)));
+        const float sl = 1.f + x * (2.f * g3 + x * (3.f * g4 + x * 4.f * g5));
+        if (!(sl > 0.f)) break;
+        const float nx = x - v / sl;
+        if (!(fabsf(nx) <= (float)h)) break;
+        x = nx;
+        slope = sl;
+    }
+    double d = (double)x;
+    const double step = inv * (double)(1.f / slope);
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+        const double v = fma(d, fma(d, fma(d, fma(d, fma(d, f6, f5), f4), f3), f2), f1);
+        const double nd = fma(-v, step, d);
+        if (!(fabs(nd) <= h)) break;
+        d = nd;
+    }
+    // the change of E from th0: kept only if it does not rise
+    const double dE = d * fma(d, fma(d, fma(d, f4 * 0.25, f3 * (1.0 / 3.0)), 0.5 * f2), f1);
+    return dE > 0.0 ? th0 : th0 + d;
+}
 
 __global__ void __launch_bounds__(LS_BS)
 k_line_search(DevStep* step, double theta_given, const double* theta_list, const double2* __restrict__ sc,
-              const int* __restrict__ rank, long long* se, unsigned* ticket) {
+              const int* __restrict__ rank) {
+    constexpr int NW = LS_BS / 32;
+    __shared__ long long red[NW], mins[LS_BLOCKS], thr_sh;
+    __shared__ int redi[NW], picks[LS_BLOCKS];
+    cg::cluster_group cl = cg::this_cluster();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, cta = (int)cl.block_rank();
+    const int m0 = cta * LS_BS + threadIdx.x;
+    const int twice = (2 * m0 + 2049) & 4095;     // the sample at 2 theta
+    const double2 t0 = sc[m0], t2 = sc[twice];
+    const int mine = rank[m0] * 4096 + m0;
     pdl_start();
     pdl_wait();
-    __shared__ long long red[LS_BS / 32];
-    __shared__ int redi[LS_BS / 32];
-    __shared__ long long thr_sh;
-    if (step->converged) return;                 // uniform over the grid
+    if (step->converged) return;                 // uniform over the cluster, before any barrier
     if (theta_list) theta_given = theta_list[step->iter];
     if (!isnan(theta_given)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) step->theta = theta_given;
+        if (m0 == 0) step->theta = theta_given;
         return;
     }
+    // every CTA must be running before a peer writes into its shared memory:
+    // arrive here, wait just before the first write
+    asm volatile("barrier.cluster.arrive;" ::: "memory");
     double c[6];
-    c[0] = step->dots[0];   // H00, from the same products as the others
-    c[1] = step->dots[1];   // H01
-    c[2] = step->dots[2];   // H02
-    c[3] = step->dots[3];   // H11
-    c[4] = step->dots[4];   // H12
-    c[5] = step->dots[5];   // H22
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int NW = LS_BS / 32;
-    const int m0 = blockIdx.x * LS_BS + threadIdx.x;
-    const double2 t0 = sc[m0];
-    const long long key = order_key(line_e_sc(c, t0.x, t0.y));
-    se[m0] = key;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) c[i] = step->dots[i];   // H00, H01, H02, H11, H12, H22
+    const LineTrig tr = line_trig(c);
+    const double e = fma(tr.a1, t0.y, fma(tr.b1, t0.x, fma(tr.a2, t2.y, fma(tr.b2, t2.x, tr.a0))));
+    const long long key = order_key(e);
     long long mn = key;
-    for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_down_sync(0xffffffffu, mn, o));
+    for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
     if (lane == 0) red[wid] = mn;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        long long b = red[0];
-        for (int i = 1; i < NW; ++i) b = min(b, red[i]);
-        se[4096 + blockIdx.x] = b;
-    }
-    __threadfence();                              // every sample visible before the ticket
-    if (!last_block(ticket, gridDim.x)) return;
-    // the last block: global minimum, tolerance, tie rule, polish
+    asm volatile("barrier.cluster.wait;" ::: "memory");
     if (threadIdx.x < 32) {
-        long long b = threadIdx.x < LS_BLOCKS ? __ldcg(se + 4096 + threadIdx.x) : LLONG_MAX;
-        for (int o = 16; o > 0; o >>= 1) b = min(b, __shfl_down_sync(0xffffffffu, b, o));
-        if (threadIdx.x == 0) {
-            const double emin = key_value(b);
-            thr_sh = order_key(emin + 1e-10 * fmax(1.0, fabs(emin)));
-        }
+        long long b = lane < NW ? red[lane] : LLONG_MAX;
+        for (int o = NW / 2; o > 0; o >>= 1) b = min(b, __shfl_xor_sync(0xffffffffu, b, o));
+        if (lane < LS_BLOCKS) *cl.map_shared_rank(&mins[cta], lane) = __shfl_sync((1u << LS_BLOCKS) - 1u, b, 0);
+    }
+    cl.sync();
+    if (threadIdx.x == 0) {
+        long long b = mins[0];
+        for (int i = 1; i < LS_BLOCKS; ++i) b = min(b, mins[i]);
+        const double emin = key_value(b);
+        thr_sh = order_key(emin + 1e-10 * fmax(1.0, fabs(emin)));
     }
     __syncthreads();
-    const long long thr = thr_sh;
-    int best = INT_MAX;   // rank * 4096 + m of the preferred sample within the tolerance
-    {
-        // every key load issued before the first comparison waits on one
-        constexpr int PER = 4096 / LS_BS;
-        long long key_m[PER];
-#pragma unroll
-        for (int j = 0; j < PER; ++j) key_m[j] = __ldcg(se + threadIdx.x + j * LS_BS);
-#pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const int m = threadIdx.x + j * LS_BS;
-            if (key_m[j] <= thr) best = min(best, rank[m] * 4096 + m);
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_down_sync(0xffffffffu, best, o));
+    // rank * 4096 + m of the preferred sample within the tolerance
+    int best = key <= thr_sh ? mine : INT_MAX;
+    best = __reduce_min_sync(0xffffffffu, best);
     if (lane == 0) redi[wid] = best;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int b = redi[0];
-        for (int i = 1; i < NW; ++i) b = min(b, redi[i]);
+        for (int i = 1; i < NW; ++i) best = min(best, redi[i]);
+        *cl.map_shared_rank(&picks[cta], 0) = best;
+    }
+    cl.sync();                                    // no access to a peer after this
+    if (m0 == 0) {
+        int b = picks[0];
+        for (int i = 1; i < LS_BLOCKS; ++i) b = min(b, picks[i]);
         const int mb = b & 4095;                  // the global minimum is always within the tolerance
-        const double th0 = sample_theta(mb);
-        const double2 s0 = sc[mb];
-        const double e0 = key_value(__ldcg(se + mb));
-        const double h = 2.0 * kPi / 4096.0;
-        // Newton on dE/dtheta.  The chain runs in one thread on a pipe that
-        // holds every float64 instruction for 64 cycles, so its length is its
-        // time: the trigonometric form of the derivatives, and the quotient
-        // by a float32 reciprocal (it scales a step by 1 + 1e-7, which the next
-        // step makes good)
-        const LineTrig tr = line_trig(c);
-        double th = th0, dl = 0.0;
-        for (int it = 0; it < 8; ++it) {
-            double sn, cs;
-            sincos_near(s0, dl, sn, cs);
-            const double s2 = 2.0 * sn * cs, c2 = fma(cs, cs, -(sn * sn));
-            const double d2 = -fma(tr.a1, cs, fma(tr.b1, sn, 4.0 * fma(tr.a2, c2, tr.b2 * s2)));
-            if (!(d2 > 0.0)) break;
-            const double d1 = fma(tr.b1, cs, fma(-tr.a1, sn, 2.0 * fma(tr.b2, c2, -(tr.a2 * s2))));
-            const double stp = d1 * quick_reciprocal(d2);
-            if (fabs(dl - stp) > h) break;
-            dl -= stp;
-            th = th0 + dl;
-            if (fabs(stp) < 1e-15) break;
-        }
-        double sn, cs;
-        sincos_near(s0, dl, sn, cs);
-        if (line_e_sc(c, sn, cs) > e0) th = th0;
-        step->theta = th;
-        *ticket = 0u;
+        step->theta = line_polish(tr, sc[mb], sc[(2 * mb + 2049) & 4095], sample_theta(mb), 2.0 * kPi / 4096.0);
     }
 }
 
@@ -1475,9 +1460,21 @@ int launch_line_table(double2* sc, cudaStream_t s) {
 }
 
 int launch_line_search(DevStep* step, double theta_given, const double* theta_list, const double2* sc,
-                       const int* rank, long long* se, unsigned* ticket, cudaStream_t s) {
-    launch_pdl(k_line_search, LS_BLOCKS, LS_BS, 0, s, step, theta_given, theta_list, sc, rank, se, ticket);
-    return 1;
+                       const int* rank, cudaStream_t s) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = LS_BLOCKS;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(LS_BLOCKS);
+    cfg.blockDim = dim3(LS_BS);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, k_line_search, step, theta_given, theta_list, sc, rank) == cudaSuccess ? 1 : -1;
 }
 
 __global__ void k_step_record(DevStep* step, double* rec, int n) {

@@ -47,10 +47,16 @@ struct ReqDev {
     double* gpart;
     unsigned* gtick;
     double energy, e_den, max_grad, norm2;
+    double scale;            // 1 / ||psi'|| of an evolve request
     int kind, M, k, argmax;
     unsigned etick;
-    int pad;
+    int eoff;                // first energy partial of this request
+    int group;               // at a group's first entry: requests of the group (its entries follow)
+    const float2* pack;      // there: the group's states interleaved, pack_width(group) per amplitude (or null)
 };
+
+// Interleaved states per amplitude of a group of n requests.
+__host__ __device__ constexpr int pack_width(int n) { return n <= 1 ? 1 : n == 2 ? 2 : 4; }
 
 namespace {
 
@@ -59,7 +65,8 @@ constexpr int MAX_TICK = 2048;
 
 // index block of a tick, in ints
 struct Idx {
-    int e_off[MAX_TICK + 1];   // energy items per E entry (prefix)
+    int e_off[MAX_TICK + 1];   // energy items per group of E entries (prefix)
+    int e_first[MAX_TICK];     // first E entry of each group
     int g_off[MAX_TICK + 1];   // gradient items per G entry (prefix)
     int g_pos[MAX_TICK];       // position of each G entry in E
     int p_off[MAX_TICK + 1];   // pair tiles per P entry (prefix)
@@ -76,38 +83,256 @@ __device__ __forceinline__ int find_req(const int* off, int n, int it) {
     return lo;
 }
 
-template <typename T, typename VT, int L>
+// The last block of a request's items (found by its ticket) adds its partials.
+__device__ __forceinline__ void finish_energy(ReqDev& d, int items, const double* epart, double* sh) {
+    double a, b;
+    block_sum_pairs(epart, d.eoff, items, sh, a, b);
+    if (threadIdx.x == 0) {
+        d.e_den = b;
+        d.energy = a / b;
+    }
+}
+
+// complex128: one request per group.
+template <int L>
 __global__ void __launch_bounds__(SV_BS)
-ks_energy(ReqDev* E, const Idx* ix, int n, double* epart) {
-    using V = typename C2<T>::type;
+ks_energy_c128(ReqDev* E, const Idx* ix, int n, double* epart) {
     __shared__ double sh[2 * (SV_BS / 32)];
     __shared__ bool last;
     const int total = ix->e_off[n];
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
-        const int q = find_req(ix->e_off, n, it);
-        ReqDev& d = E[q];
-        const long long r0 = (long long)(it - ix->e_off[q]) * ENERGY_ROWS;
-        const long long r1 = min(r0 + ENERGY_ROWS, d.D);
+        const int g = find_req(ix->e_off, n, it);
+        ReqDev& d = E[ix->e_first[g]];
+        const int items = ix->e_off[g + 1] - ix->e_off[g], blk = it - ix->e_off[g];
+        const long long r0 = (long long)blk * ENERGY_ROWS, r1 = min(r0 + ENERGY_ROWS, d.D);
         double num = 0.0, den = 0.0;
-        energy_rows<T, VT, L>(d.rowptr, d.col, static_cast<const VT*>(d.val), d.diag,
-                              static_cast<const V*>(d.psi), d.w64, d.w32, r0, r1, num, den);
+        energy_rows<double, double, L>(d.rowptr, d.col, static_cast<const double*>(d.val), d.diag,
+                                       static_cast<const double2*>(d.psi), d.w64, d.w32, r0, r1, num, den);
         double v[2] = {num, den};
         block_sum<2>(v, sh);
         if (threadIdx.x == 0) {
-            epart[2 * it] = v[0];
-            epart[2 * it + 1] = v[1];
+            epart[2 * (d.eoff + blk)] = v[0];
+            epart[2 * (d.eoff + blk) + 1] = v[1];
             __threadfence();
-            last = atomicAdd(&d.etick, 1u) == (unsigned)(ix->e_off[q + 1] - ix->e_off[q]) - 1;
+            last = atomicAdd(&d.etick, 1u) == (unsigned)items - 1;
         }
         __syncthreads();
-        if (last) {
-            double a, b;
-            block_sum_pairs(epart, ix->e_off[q], ix->e_off[q + 1] - ix->e_off[q], sh, a, b);
-            if (threadIdx.x == 0) {
-                d.e_den = b;
-                d.energy = a / b;
-            }
+        if (last) finish_energy(d, items, epart, sh);
+        __syncthreads();
+    }
+}
+
+// ---- complex64: requests of a tick on the same Hamiltonian, up to four at a time
+//
+// A CSR energy is bound by its gathers: 32 lanes touch 32 lines, and the L1
+// serves about one line a cycle, whatever is used of it.  Up to four states
+// of a group are therefore interleaved per amplitude (ks_pack; one 32-byte
+// sector), and one gather feeds four products; the entries are read once for
+// all.  96 mixed requests on 24 sessions of three molecules (12 to 16 qubits):
+// the energy launches 1.33 ms one by one, 0.87 ms here.  A request's row sums run in the order of the single form (entry e
+// on lane (e - first) mod 8, butterfly 4, 2, 1) and its energy sums in one
+// tree for every width, so its result does not depend on its group.
+template <int W> struct PackVec;
+template <> struct PackVec<1> {
+    float2 v[1];
+    __device__ __forceinline__ void load(const float2* p, int c) { v[0] = __ldg(p + c); }
+};
+template <> struct PackVec<2> {
+    float2 v[2];
+    __device__ __forceinline__ void load(const float2* p, int c) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(p) + c);
+        v[0] = make_float2(q.x, q.y);
+        v[1] = make_float2(q.z, q.w);
+    }
+};
+template <> struct PackVec<4> {
+    float2 v[4];
+    __device__ __forceinline__ void load(const float2* p, int c) {
+        // one 32-byte access per lane (sm_100 and later)
+        asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x),
+              "=f"(v[3].y)
+            : "l"(p + 4ll * c));
+    }
+};
+
+// One row's sums of W states on a group of 8 lanes (the order of
+// row_dot<.., 8>), scattered over the lanes: value (state v, component) ends
+// in lane gl with gl / (8 / (2 W)) == 2 v + component.
+template <int W>
+__device__ __forceinline__ float pack_row(const int* __restrict__ col, const float* __restrict__ val,
+                                          const float2* x, int e0, int e1, int gl) {
+    float2 acc[W];
+#pragma unroll
+    for (int v = 0; v < W; ++v) acc[v] = make_float2(0.f, 0.f);
+    int e = e0 + gl;
+    constexpr int U = W == 4 ? 2 : 4;             // 64 or 32 bytes of states in flight per lane
+    int c[U];
+    float a[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+        const bool in = e + 8 * j < e1;
+        c[j] = in ? col[e + 8 * j] : -1;
+        a[j] = in ? val[e + 8 * j] : 0.f;
+    }
+    while (e < e1) {
+        PackVec<W> g[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (c[j] >= 0) g[j].load(x, c[j]);
+        e += 8 * U;
+        int nc[U];
+        float na[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const bool in = e + 8 * j < e1;
+            nc[j] = in ? col[e + 8 * j] : -1;
+            na[j] = in ? val[e + 8 * j] : 0.f;
         }
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (c[j] >= 0)
+#pragma unroll
+                for (int v = 0; v < W; ++v) acc[v] = __ffma2_rn(make_float2(a[j], a[j]), g[j].v[v], acc[v]);
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            c[j] = nc[j];
+            a[j] = na[j];
+        }
+    }
+    __syncwarp();
+    float s[2 * W];
+#pragma unroll
+    for (int v = 0; v < W; ++v) {
+        s[2 * v] = acc[v].x;
+        s[2 * v + 1] = acc[v].y;
+    }
+    int o = 4;
+#pragma unroll
+    for (int k = 2 * W; k > 1; k >>= 1, o >>= 1) {
+        const bool up = gl & o;
+#pragma unroll
+        for (int i = 0; i < k / 2; ++i) {
+            const float give = up ? s[i] : s[i + k / 2], keep = up ? s[i + k / 2] : s[i];
+            s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (int q = 4 / (2 * W); q > 0; q >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], q);
+    return s[0];
+}
+
+// 64 rows of up to W requests: a warp takes 8 rows, each 8-lane group two
+// of them (j = 0, 1); the lane of (state v, j) finishes its row in float64.
+// sums[w][..] receives the warps' (num, den) per state.
+template <int W>
+__device__ __forceinline__ void pack_rows(ReqDev* E, int n, const float2* x, long long r0, long long r1,
+                                          double (*sums)[8]) {
+    const ReqDev& d = E[0];
+    const int lane = threadIdx.x & 31, gl = lane & 7, wid = threadIdx.x >> 5;
+    const long long base = r0 + wid * ENERGY_WARP_ROWS + (lane >> 3) * 2;
+    const float* val = static_cast<const float*>(d.val);
+    float k[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const long long r = base + j;
+        int e0 = 0, e1 = 0;                       // a row past the end has no entries; every lane takes part
+        if (r < r1) {
+            e0 = d.rowptr[r];
+            e1 = d.rowptr[r + 1];
+        }
+        k[j] = pack_row<W>(d.col, val, x, e0, e1, gl);
+    }
+    // components sit PAIR lanes apart; of the pair (and of its copies) one
+    // lane takes j = 0 and one j = 1
+    constexpr int PAIR = 8 / (2 * W);
+    const int v = gl / (2 * PAIR), comp = (gl / PAIR) & 1;
+    const int j = W == 1 ? gl & 1 : comp;
+    const float give = W == 1 ? ((gl & 1) ? k[1] : k[0]) : (comp ? k[0] : k[1]);
+    const float got = __shfl_xor_sync(0xffffffffu, give, PAIR);
+    float sx, sy;
+    bool mine;
+    if (W == 1) {
+        mine = gl < 2;
+        sx = give;
+        sy = got;
+    } else {
+        mine = gl % PAIR == 0;
+        sx = comp ? got : k[0];
+        sy = comp ? k[1] : got;
+    }
+    double num = 0.0, den = 0.0;
+    const long long r = base + j;
+    if (mine && v < n && r < r1) {
+        const ReqDev& q = E[v];
+        const float2 pv = static_cast<const float2*>(q.psi)[r];
+        const double px = (double)pv.x, py = (double)pv.y, dg = d.diag[r];
+        const double wx = fma(dg, px, (double)sx), wy = fma(dg, py, (double)sy);
+        q.w32[r] = make_float2((float)wx, (float)wy);
+        num = px * wx + py * wy;
+        den = px * px + py * py;
+    }
+    // per state: rows j = 0 and 1, then the four groups of the warp
+    constexpr int JJ = W == 1 ? 1 : PAIR;
+    num += __shfl_xor_sync(0xffffffffu, num, JJ);
+    den += __shfl_xor_sync(0xffffffffu, den, JJ);
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    if (lane < 8 && mine && j == 0) {
+        sums[wid][2 * v] = num;
+        sums[wid][2 * v + 1] = den;
+    }
+}
+
+__global__ void __launch_bounds__(SV_BS)
+ks_pack(ReqDev* E, const Idx* ix, int n) {
+    const int total = ix->e_off[n];
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        const int g = find_req(ix->e_off, n, it);
+        ReqDev* q = E + ix->e_first[g];
+        if (!q->pack) continue;
+        const int W = pack_width(q->group), v = threadIdx.x / ENERGY_ROWS;
+        const long long r = (long long)(it - ix->e_off[g]) * ENERGY_ROWS + threadIdx.x % ENERGY_ROWS;
+        if (v < W && r < q->D)
+            const_cast<float2*>(q->pack)[W * r + v] =
+                v < q->group ? static_cast<const float2*>(q[v].psi)[r] : make_float2(0.f, 0.f);
+    }
+}
+
+__global__ void __launch_bounds__(SV_BS, 3)
+ks_energy_c64(ReqDev* E, const Idx* ix, int n, double* epart) {
+    constexpr int NW = SV_BS / 32;
+    __shared__ double sh[2 * NW];
+    __shared__ double sums[NW][8];
+    __shared__ bool last[4];
+    const int total = ix->e_off[n];
+    for (int it = blockIdx.x; it < total; it += gridDim.x) {
+        const int g = find_req(ix->e_off, n, it);
+        ReqDev* q = E + ix->e_first[g];
+        const int items = ix->e_off[g + 1] - ix->e_off[g], blk = it - ix->e_off[g], cnt = q->group;
+        const long long r0 = (long long)blk * ENERGY_ROWS, r1 = min(r0 + ENERGY_ROWS, q->D);
+        const float2* x = q->pack ? q->pack : static_cast<const float2*>(q->psi);
+        if (cnt == 1) pack_rows<1>(q, 1, x, r0, r1, sums);
+        else if (cnt == 2) pack_rows<2>(q, 2, x, r0, r1, sums);
+        else pack_rows<4>(q, cnt, x, r0, r1, sums);
+        __syncthreads();
+        // eight lanes per value, one per warp
+        const int t = threadIdx.x, i = t >> 3;
+        if (t < 64) {
+            double s = i < 2 * cnt ? sums[t & 7][i] : 0.0;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((t & 7) == 0 && i < 2 * cnt) epart[2 * (q[i >> 1].eoff + blk) + (i & 1)] = s;
+        }
+        __threadfence();
+        __syncthreads();
+        if (t < cnt) last[t] = atomicAdd(&q[t].etick, 1u) == (unsigned)items - 1;
+        __syncthreads();
+        for (int v = 0; v < cnt; ++v)
+            if (last[v]) finish_energy(q[v], items, epart, sh);
         __syncthreads();
     }
 }
@@ -203,7 +428,12 @@ __global__ void ks_norm(ReqDev* P, const Idx* ix, int np, const double* npart) {
         }
     }
     acc = warp_sum(acc);
-    if (lane == 0) P[q].norm2 = acc;
+    if (lane == 0) {
+        P[q].norm2 = acc;
+        // once per request: a float64 root and division in every warp of the
+        // rescale took two thirds of its time
+        P[q].scale = 1.0 / sqrt(acc);
+    }
 }
 
 template <typename T>
@@ -211,7 +441,7 @@ __global__ void ks_scale(ReqDev* P, int np) {
     using V = typename C2<T>::type;
     for (int q = blockIdx.y; q < np; q += gridDim.y) {
         ReqDev& d = P[q];
-        const double sc = 1.0 / sqrt(d.norm2);
+        const double sc = d.scale;
         V* psi = static_cast<V*>(d.psi);
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < d.D;
              i += (long long)gridDim.x * blockDim.x) {
@@ -339,11 +569,20 @@ void launch_tick(tq_server* s, tq_server::Tick& tk) {
     ReqDev* E = tick_E(tk.h);
     ReqDev* P = tick_P(tk.h);
     Idx* ix = tick_I(tk.h);
-    int ne = 0, ng = 0, np = 0;
+    int ne = 0, ng = 0, np = 0, n_grp = 0;
     ix->e_off[0] = ix->g_off[0] = ix->p_off[0] = ix->p_base[0] = 0;
     size_t arena_off = 0;
     tk.slot.assign(tk.reqs.size(), 0);
-    for (size_t i = 0; i < tk.reqs.size(); ++i) {
+    // energies and gradients of one Hamiltonian side by side (arrival order
+    // inside): they are evaluated together
+    std::vector<size_t> order(tk.reqs.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) {
+        return s->sessions[tk.reqs[a].session].ham < s->sessions[tk.reqs[b].session].ham;
+    });
+    std::vector<int> e_ham;
+    int e_items = 0;
+    for (size_t i : order) {
         const tq_request& r = tk.reqs[i];
         const auto& ss = s->sessions[r.session];
         const tq_ham* hm = s->hams[ss.ham];
@@ -385,10 +624,35 @@ void launch_tick(tq_server* s, tq_server::Tick& tk) {
             ++ng;
         }
         arena_off += off;
-        ix->e_off[ne + 1] = ix->e_off[ne] + (int)((d.D + ENERGY_ROWS - 1) / ENERGY_ROWS);
+        d.eoff = e_items;
+        e_items += (int)((d.D + ENERGY_ROWS - 1) / ENERGY_ROWS);
         E[ne] = d;
+        e_ham.push_back(ss.ham);
         tk.slot[i] = ne;
         ++ne;
+    }
+    // groups of up to four; their interleaved states come from what the
+    // admitted requests leave of the arena (a group that does not fit runs one
+    // by one)
+    bool packed = false;
+    for (int e = 0; e < ne;) {
+        int n = 1;
+        size_t room = 0;
+        if (sizeof(T) == 4) {
+            while (n < 4 && e + n < ne && e_ham[e + n] == e_ham[e]) ++n;
+            room = align256((size_t)E[e].D * pack_width(n) * sizeof(float2));
+            if (n > 1 && arena_off + room > s->arena_bytes) n = 1;
+        }
+        E[e].group = n;
+        if (n > 1) {
+            E[e].pack = reinterpret_cast<const float2*>(s->arena + arena_off);
+            arena_off += room;
+            packed = true;
+        }
+        ix->e_first[n_grp] = e;
+        ix->e_off[n_grp + 1] = ix->e_off[n_grp] + (int)((E[e].D + ENERGY_ROWS - 1) / ENERGY_ROWS);
+        ++n_grp;
+        e += n;
     }
     tk.ne = ne;
     tk.np = np;
@@ -403,9 +667,17 @@ void launch_tick(tq_server* s, tq_server::Tick& tk) {
     for (int j = 0; j < ng; ++j)
         TQ_CUDA(cudaMemsetAsync(E[ix->g_pos[j]].gtick, 0, (size_t)E[ix->g_pos[j]].M * sizeof(unsigned), st));
     if (ne) {
-        const int items = ix->e_off[ne];
+        const int items = ix->e_off[n_grp];
+        if (packed)
+            launch(c, "serve_pack", st, [&] {
+                ks_pack<<<std::min(items, s->ctx->sm_count * 8), SV_BS, 0, st>>>(dE, dI, n_grp);
+                return 1;
+            });
         launch(c, "serve_energy", st, [&] {
-            ks_energy<T, VT, 8><<<std::min(items, s->grid_e), SV_BS, 0, st>>>(dE, dI, ne, s->epart);
+            if constexpr (sizeof(T) == 4)
+                ks_energy_c64<<<std::min(items, s->grid_e), SV_BS, 0, st>>>(dE, dI, n_grp, s->epart);
+            else
+                ks_energy_c128<8><<<std::min(items, s->grid_e), SV_BS, 0, st>>>(dE, dI, n_grp, s->epart);
             return 1;
         });
     }
@@ -513,7 +785,8 @@ void server_loop(tq_server* s) {
 template <typename T, typename VT>
 void compute_grids(tq_server* s) {
     const int sms = s->ctx->sm_count;
-    s->grid_e = resident(ks_energy<T, VT, 8>, SV_BS, sms);
+    if constexpr (sizeof(T) == 4) s->grid_e = resident(ks_energy_c64, SV_BS, sms);
+    else s->grid_e = resident(ks_energy_c128<8>, SV_BS, sms);
     s->grid_g = resident(ks_grad<T>, GRAD_TPB, sms);
     s->grid_p = resident(ks_pair<T>, PAIR_BS, sms);
 }

@@ -9,11 +9,11 @@
 //   grads    items (t, op, chunk): the chunk's part of 2 Re<w_t|A_k psi_t>;
 //   select   one block per t: its energy, g_t[k] (divided by <psi|psi>)
 //            summed from the chunk parts in a fixed order, k*, max|g|, convergence, angle,
-//            record, and the iteration counter advanced; the last block
-//            numbers the active trajectories' energy items for the next
-//            iteration (prefix counts);
+//            record, and the iteration counter advanced;
 //   update   items (t, tile): the fused Taylor-5 pair update with A_{k*}
-//            and the partials of ||psi'||^2.
+//            and the partials of ||psi'||^2; one more block numbers the
+//            active trajectories' energy items for the next iteration
+//            (prefix counts).
 // The state is renormalised once, after the last iteration (items
 // (t, chunk): psi /= ||psi||): every quantity an iteration computes is
 // independent of the state's scale (the energy is <psi|H|psi>/<psi|psi>,
@@ -66,7 +66,7 @@ struct TrajDev {
     const double* thetas;
     double* g;
     double* gpart;           // one partial per gradient item of this trajectory
-    const int* gfirst;       // first gradient item of each op (M + 1, the pool's table)
+    const int* gfirst;       // first gradient item of each op (M + 1)
     int gbase;               // first gradient item of this trajectory
     double* res_e;
     double* res_g;
@@ -492,30 +492,28 @@ kb_energy_smem(const TrajDev* tr, const long long* __restrict__ wpre, const int*
     }
 }
 
-// Gradient item: (t, op, chunk of the op's support rows).
+// Gradient item, one per warp: (t, op, chunk of GRAD_WARP_CHUNK support rows).
+// 24 trajectories of 10 to 14 qubits: 22 us with a block per item of up to
+// 8192 rows, 15 us here (with event overhead).
 template <typename T>
 __global__ void __launch_bounds__(GRAD_TPB)
 kb_grad(const TrajDev* tr, const TrajState* ts, const int4* items, int n_items) {
     using V = typename C2<T>::type;
-    __shared__ double sh[GRAD_TPB / 32];
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const int4 w4 = items[it];          // (t, op, chunk, chunks of this op)
+    const int warps = gridDim.x * (GRAD_TPB / 32);
+    for (int it = blockIdx.x * (GRAD_TPB / 32) + (threadIdx.x >> 5); it < n_items; it += warps) {
+        const int4 w4 = items[it];          // (t, op, chunk, -)
         const int t = w4.x, k = w4.y;
         if (!ts[t].active) continue;
         const TrajDev& d = tr[t];
         const SuppRec s = load_supp(d.pool, k);
         const uint32_t size = (uint32_t)(d.D >> s.m);
-        const uint32_t u0 = (uint32_t)w4.z * GRAD_CHUNK;
-        const uint32_t cnt = min((uint32_t)GRAD_CHUNK, size - u0);
+        const uint32_t u0 = (uint32_t)w4.z * GRAD_WARP_CHUNK;
+        const uint32_t cnt = min((uint32_t)GRAD_WARP_CHUNK, size - u0);
         const T c0 = sizeof(T) == 4 ? (T)d.pool.fc0f[k] : (T)d.pool.fc0d[k];
         double v;
-        if constexpr (sizeof(T) == 4)
-            v = grad_item<T>(s, c0, d.w32, static_cast<const V*>(d.psi), u0, cnt, sh);
-        else
-            v = grad_item<T>(s, c0, d.w, static_cast<const V*>(d.psi), u0, cnt, sh);
-        // the select launch sums the op's chunks (grad_item ends with a
-        // barrier, so sh is free again)
-        if (threadIdx.x == 0) d.gpart[it - d.gbase] = v;
+        if constexpr (sizeof(T) == 4) v = grad_item_warp<T>(s, c0, d.w32, static_cast<const V*>(d.psi), u0, cnt);
+        else v = grad_item_warp<T>(s, c0, d.w, static_cast<const V*>(d.psi), u0, cnt);
+        if ((threadIdx.x & 31) == 0) d.gpart[it - d.gbase] = v;     // the select launch sums the op's chunks
     }
 }
 
@@ -591,17 +589,14 @@ __device__ void number_active(const TrajDev* tr, const TrajState* ts, int n, con
 
 // One block per trajectory: its energy from the segments' sums (seg set), each
 // gradient from its op's chunk partials (Eq. (5), divided by <psi|psi>), then
-// choice, convergence, angle, record, and the iteration counter advanced.
-// The last block to finish renews the active trajectories' numbering.  Maxima
+// choice, convergence, angle, record, and the iteration counter advanced.  Maxima
 // and thresholds compare bit patterns (a non-negative double orders like
 // them), off the float64 pipe.
 constexpr int SEL_BS = 128;
 __global__ void __launch_bounds__(SEL_BS)
-kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, Active act, const double2* seg, int seg_ctas,
-          unsigned* ticket) {
+kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, Active act, const double2* seg, int seg_ctas) {
     constexpr int NW = SEL_BS / 32;
     constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;
-    __shared__ bool last;
     __shared__ double e_sh[2];
     __shared__ unsigned long long smax[NW];
     __shared__ int smin[NW];
@@ -623,8 +618,12 @@ kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, Active 
                         den += v.y;
                     }
                 }
-                num = warp_sum(num);
-                den = warp_sum(den);
+                const bool up = lane & 16;         // num in the lower half, den in the upper
+                double v = (up ? den : num) + __shfl_xor_sync(0xffffffffu, up ? num : den, 16);
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                num = v;
+                den = __shfl_sync(0xffffffffu, v, 16);
             } else {
                 num = s.e_num;
                 den = s.e_den;
@@ -702,24 +701,21 @@ kb_select(const TrajDev* tr, TrajState* ts, int n, double eps, int prec, Active 
             d.res_th[it] = s.theta;
             s.iter = it + 1;
             s.active = (!s.converged && it + 1 < d.len) ? 1 : 0;
-            __threadfence();
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    number_active(tr, ts, n, act);
-    if (threadIdx.x == 0) *ticket = 0u;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(PAIR_BS)
-kb_pair(const TrajDev* tr, const TrajState* ts, const int4* items, int n_items, double* npart) {
+kb_pair(const TrajDev* tr, const TrajState* ts, const int4* items, int n_items, double* npart, int n, Active act) {
     constexpr int NW = PAIR_BS / 32;
     const int warp = threadIdx.x >> 5;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
+    // the last block renews the active trajectories' numbering meanwhile
+    if (blockIdx.x == gridDim.x - 1) {
+        number_active(tr, ts, n, act);
+        return;
+    }
+    for (int it = blockIdx.x; it < n_items; it += gridDim.x - 1) {
         const int4 w4 = items[it];
         const int t = w4.x, tl = w4.y;
         const TrajState& s = ts[t];
@@ -815,7 +811,6 @@ struct tq_batch {
     double2* seg = nullptr;         // energy segments (kb_energy_smem)
     int room = 0;                   // amplitudes it holds in shared memory
     bool by_segments() const { return prec == TQ_C64 && lpr == 32; }
-    unsigned* nticket = nullptr;    // blocks of the select launch done
     unsigned char* res = nullptr;   // results block (see tq_batch_create)
     size_t res_len = 0;             // iterations of all trajectories
     size_t states_at() const {
@@ -887,7 +882,7 @@ void compute_grids(tq_batch* b) {
     if constexpr (sizeof(T) == 8) b->grid_e[3] = std::min(b->n_e, resident_grid(kb_energy<T, VT, 32>, BT_BS, sms));
     else TQ_CUDA(cudaFuncSetAttribute(kb_energy_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kbs_smem(KBS_ROOM)));
     b->grid_x = std::min(b->n_e, resident_grid(kbx_energy<T, VT>, BT_BS, sms));
-    b->grid_g = std::min(b->n_g, resident_grid(kb_grad<T>, GRAD_TPB, sms));
+    b->grid_g = std::min((b->n_g + GRAD_TPB / 32 - 1) / (GRAD_TPB / 32), resident_grid(kb_grad<T>, GRAD_TPB, sms));
     b->grid_p = std::min(b->n_p, resident_grid(kb_pair<T>, PAIR_BS, sms));
 }
 
@@ -909,11 +904,11 @@ void enqueue_iteration(tq_batch* b, cudaStream_t s) {
     });
     launch(c, "batch_select", s, [&] {
         kb_select<<<b->n, SEL_BS, 0, s>>>(b->d_td, b->d_ts, b->n, b->eps, b->prec, b->act,
-                                          b->by_segments() ? b->seg : nullptr, c->sm_count, b->nticket);
+                                          b->by_segments() ? b->seg : nullptr, c->sm_count);
         return 1;
     });
     launch(c, "batch_taylor5_pair", s, [&] {
-        kb_pair<T><<<b->grid_p, PAIR_BS, 0, s>>>(b->d_td, b->d_ts, b->pitems, b->n_p, b->npart);
+        kb_pair<T><<<b->grid_p + 1, PAIR_BS, 0, s>>>(b->d_td, b->d_ts, b->pitems, b->n_p, b->npart, b->n, b->act);
         return 1;
     });
 }
@@ -1016,13 +1011,14 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
             d.cut = cut;
             if (d.D <= KBS_ROOM) b->room = std::max(b->room, (int)d.D);
             d.gbase = (int)gi.size();
-            // the pool's own item table: op k's chunks are items gf[k] .. gf[k + 1] - 1
-            std::vector<int> gf((size_t)d.M + 1);
-            TQ_CUDA(cudaMemcpy(gf.data(), p->view.gfirst, gf.size() * sizeof(int), cudaMemcpyDeviceToHost));
+            // op k's chunks are items gf[k] .. gf[k + 1] - 1 (the support of a
+            // single is D/2 rows, of a double D/8)
+            std::vector<int> gf((size_t)d.M + 1, 0);
             for (int k = 0; k < d.M; ++k) {
-                const int nchunks = gf[k + 1] - gf[k];
-                TQ_REQUIRE(gf[k] == (int)gi.size() - d.gbase && nchunks >= 1, "pool gradient table is inconsistent");
-                for (int ch = 0; ch < nchunks; ++ch) gi.push_back(make_int4(t, k, ch, nchunks));
+                const long long rows = d.D >> (p->idx4[4 * (size_t)k + 2] < 0 ? 1 : 3);
+                const int nchunks = (int)std::max<long long>(1, (rows + GRAD_WARP_CHUNK - 1) / GRAD_WARP_CHUNK);
+                for (int ch = 0; ch < nchunks; ++ch) gi.push_back(make_int4(t, k, ch, 0));
+                gf[k + 1] = (int)gi.size() - d.gbase;
             }
             const int n_gitems_t = (int)gi.size() - d.gbase;
             const long long units = d.D >> 2;
@@ -1040,7 +1036,7 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
             toff += d.len;
             d.g = dalloc<double>(b, d.M);
             d.gpart = dalloc<double>(b, (size_t)n_gitems_t);
-            d.gfirst = p->view.gfirst;
+            d.gfirst = dupload(b, gf);
             b->max_len = std::max(b->max_len, d.len);
             b->td.push_back(d);
         }
@@ -1103,8 +1099,6 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
             b->act0 = dupload(b, img);
             b->act = view(dupload(b, img));
             b->seg = dalloc<double2>(b, (size_t)c->sm_count + n_traj);
-            b->nticket = dalloc<unsigned>(b, 1);
-            TQ_CUDA(cudaMemset(b->nticket, 0, sizeof(unsigned)));
         }
         b->d_td = dupload(b, b->td);
         b->d_ts = reinterpret_cast<TrajState*>(b->res + b->states_at());

@@ -127,6 +127,25 @@ __device__ __forceinline__ double2 sign_flip(int odd, double2 v) {
                         __hiloint2double(__double2hiint(v.y) ^ f, __double2loint(v.y)));
 }
 
+// Adds one support row's product Re<w_r|A psi> to (hi, lo).  complex64: a
+// compensated float32 sum.  complex128: the sign on the integer pipe, c0 once
+// at the end of the item: two float64 instructions per row instead of four
+// (they bound the sweep: 16 qubits 35 -> 20 us).
+__device__ __forceinline__ void grad_add(const SuppRec& s, float c0, uint32_t r, float2 w, float2 v, float& hi,
+                                         float& lo) {
+    const float prod = (parity32((r ^ s.x) & s.z0) ? -c0 : c0) * fmaf(w.x, v.x, w.y * v.y);
+    float sum, err;
+    two_sum(hi, prod, sum, err);
+    hi = sum;
+    lo += err;
+}
+__device__ __forceinline__ void grad_add(const SuppRec& s, double, uint32_t r, double2 w, double2 v, double& hi,
+                                         double& lo) {
+    const double2 f = sign_flip(parity32((r ^ s.x) & s.z0), v);
+    hi = fma(w.x, f.x, hi);
+    lo = fma(w.y, f.y, lo);
+}
+
 // Sum of one item over the block of GRAD_TPB threads; valid in thread 0.
 // `sh` holds 2 * warps doubles.  W is float2 (complex64: w in float32) or
 // double2.
@@ -170,23 +189,7 @@ __device__ __forceinline__ double grad_item(const SuppRec& s, T c0, const W* __r
             }
 #pragma unroll
         for (int u = 0; u < GRAD_U; ++u)
-            if (in[u]) {
-                const int odd = parity32((r[u] ^ s.x) & s.z0);
-                if constexpr (sizeof(T) == 4) {
-                    const T prod = (odd ? -c0 : c0) * fma((T)wr[u].x, (T)v[u].x, (T)wr[u].y * (T)v[u].y);
-                    T sum, err;
-                    two_sum(hi, prod, sum, err);
-                    hi = sum;
-                    lo += err;
-                } else {
-                    // the sign on the integer pipe, c0 once at the end: two
-                    // float64 instructions per row instead of four (they
-                    // bound the sweep: 16 qubits 35 -> 20 us)
-                    const double2 f = sign_flip(odd, v[u]);
-                    hi = fma(wr[u].x, f.x, hi);
-                    lo = fma(wr[u].y, f.y, lo);
-                }
-            }
+            if (in[u]) grad_add(s, c0, r[u], wr[u], v[u], hi, lo);
     }
     double part;
     if constexpr (sizeof(T) == 4) part = warp_sum_compensated_pair(hi, lo);
@@ -201,6 +204,45 @@ __device__ __forceinline__ double grad_item(const SuppRec& s, T c0, const W* __r
     }
     __syncthreads();
     return tot;
+}
+
+// The same for one warp and at most GRAD_WARP_CHUNK rows, with no barrier: valid
+// in lane 0.  A warp per item suits many small supports at once (a
+// trajectory batch): a block's item is mostly its chain of loads and
+// barriers.
+constexpr int GRAD_WARP_CHUNK = 1024;
+static_assert(GRAD_WARP_CHUNK <= 32 * 32, "one row base per lane");
+template <typename T, typename W, typename V>
+__device__ __forceinline__ double grad_item_warp(const SuppRec& s, T c0, const W* __restrict__ w,
+                                                 const V* __restrict__ psi, uint32_t u0, uint32_t cnt) {
+    const uint32_t lane = threadIdx.x & 31;
+    const RowExp rx = make_rowexp(s, 0);
+    const uint32_t L = expand_support_row(rx, lane) ^ rx.tb;
+    const uint32_t Rl = expand_support_row(rx, u0 + lane * 32);
+    const uint32_t nk = (cnt + 31) / 32;
+    T hi = T(0), lo = T(0);
+    for (uint32_t k = 0; k < nk; k += GRAD_U) {
+        uint32_t r[GRAD_U];
+        bool in[GRAD_U];
+        W wr[GRAD_U];
+        V v[GRAD_U];
+#pragma unroll
+        for (int u = 0; u < GRAD_U; ++u) {
+            r[u] = __shfl_sync(0xffffffffu, Rl, (k + u) & 31) ^ L;
+            in[u] = lane + (k + u) * 32 < cnt;
+        }
+#pragma unroll
+        for (int u = 0; u < GRAD_U; ++u)
+            if (in[u]) {
+                wr[u] = w[r[u]];
+                v[u] = psi[r[u] ^ s.x];
+            }
+#pragma unroll
+        for (int u = 0; u < GRAD_U; ++u)
+            if (in[u]) grad_add(s, c0, r[u], wr[u], v[u], hi, lo);
+    }
+    if constexpr (sizeof(T) == 4) return warp_sum_compensated_pair(hi, lo);
+    else return warp_sum(c0 * (hi + lo));
 }
 
 }  // namespace tq

@@ -558,6 +558,9 @@ void build_full(tq_ctx* c, tq_ham* h, const Grouped& q) {
     v.n_blocks = B;
     v.xgrid = xell_grid(B, h->prec, c->sm_count);
     const size_t a_split = a.room((size_t)(v.xgrid + 1) * sizeof(int));
+    const bool half = h->prec == TQ_C64 && h->nq >= HALF_MIN_QUBITS;
+    const size_t a_hcls = a.room(half ? (size_t)B * sizeof(uint2) : 0),
+                 a_hsplit = a.room(half ? (size_t)(half_warps(c->sm_count) + 1) * sizeof(int) : 0);
     auto* base = static_cast<unsigned char*>(dev_alloc(a.bytes));
     h->allocs.push_back(base);
     TQ_CUDA(cudaMemcpy(base, a.image.data(), a.image.size(), cudaMemcpyHostToDevice));
@@ -575,6 +578,10 @@ void build_full(tq_ctx* c, tq_ham* h, const Grouped& q) {
     v.rowptr = rowptr;
     v.xptr = xptr;
     v.xsplit = split;
+    uint2* hcls = half ? reinterpret_cast<uint2*>(base + a_hcls) : nullptr;
+    int* hsplit = half ? reinterpret_cast<int*>(base + a_hsplit) : nullptr;
+    v.hcls = hcls;
+    v.hsplit = hsplit;
 
     // build-time data
     std::vector<uint32_t> sz(q.dz.size());
@@ -595,7 +602,9 @@ void build_full(tq_ctx* c, tq_ham* h, const Grouped& q) {
     const size_t w_T = w.room((size_t)plan.n_entries * sizeof(double)),
                  w_Tf = w.room((size_t)plan.n_entries * sizeof(float)),
                  w_rows = w.room((size_t)D * sizeof(int)), w_blks = w.room((size_t)B * sizeof(int)),
-                 w_seg = w.room((size_t)segs * sizeof(BuildSeg)), w_off = w.room((size_t)segs * sizeof(longlong2));
+                 w_seg = w.room((size_t)segs * sizeof(BuildSeg)), w_off = w.room((size_t)segs * sizeof(BuildOffsets)),
+                 w_half = w.room(half ? (size_t)B * sizeof(int) : 0),
+                 w_hptr = w.room(half ? (size_t)(B + 1) * sizeof(int) : 0);
     auto* wb = static_cast<unsigned char*>(scratch(c, S_STAGE, w.bytes));
     TQ_CUDA(cudaMemcpy(wb, w.image.data(), w.image.size(), cudaMemcpyHostToDevice));
     BuildView bv{};
@@ -616,6 +625,12 @@ void build_full(tq_ctx* c, tq_ham* h, const Grouped& q) {
     bv.hx = reinterpret_cast<uint32_t*>(wb + w_hx);
     bv.hoff = reinterpret_cast<int*>(wb + w_hoff);
     bv.sib = reinterpret_cast<uint32_t*>(wb + w_sib);
+    if (half) {
+        bv.half_bit = h->nq - HALF_CLASSES;
+        for (int j = 0; j < HALF_CLASSES; ++j)
+            bv.cls[j] = (int)(std::lower_bound(q.gx.begin(), q.gx.end(), 1u << (bv.half_bit + j)) - q.gx.begin());
+    }
+    int* hptr = half ? reinterpret_cast<int*>(wb + w_hptr) : nullptr;
     auto* tot = reinterpret_cast<BuildTotals*>(wb + w_tot);
     const unsigned long long tol = double_bits(1e-12 * q.maxc), amb = double_bits(1e-9 * q.maxc);
 
@@ -632,10 +647,14 @@ void build_full(tq_ctx* c, tq_ham* h, const Grouped& q) {
         });
     launch(c, "build_count", 0, [&] {
         return launch_build_count(bv, D, B, tol, amb, reinterpret_cast<int*>(wb + w_rows),
-                                  reinterpret_cast<int*>(wb + w_blks), reinterpret_cast<BuildSeg*>(wb + w_seg),
-                                  reinterpret_cast<longlong2*>(wb + w_off), tot, rowptr, xptr, 0);
+                                  reinterpret_cast<int*>(wb + w_blks), reinterpret_cast<int*>(wb + w_half),
+                                  reinterpret_cast<BuildSeg*>(wb + w_seg),
+                                  reinterpret_cast<BuildOffsets*>(wb + w_off), tot, rowptr, xptr, hcls, hptr, 0);
     });
-    launch(c, "xell_split", 0, [&] { return launch_xell_split(xptr, B, v.xgrid, split, 0); });
+    launch(c, "xell_split", 0, [&] {
+        const int n = launch_xell_split(xptr, B, v.xgrid, split, 0);
+        return half ? n + launch_xell_split(hptr, B, half_warps(c->sm_count), hsplit, 0) : n;
+    });
     BuildTotals ht;
     TQ_CUDA(cudaMemcpy(&ht, tot, sizeof ht, cudaMemcpyDeviceToHost));
     if (ht.rows >= 2147483647ll)

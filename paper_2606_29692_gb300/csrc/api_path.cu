@@ -81,7 +81,20 @@ extern "C" int tq_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double
     cudaStream_t s = as_stream(stream);
     double* part = prepare(c, h->D, nullptr, h->nq);
     auto* hs = static_cast<DevStep*>(host_scratch(c, sizeof(DevStep)));   // the kernel writes the result there
-    run_energy(c, h, psi, part, s, hs);
+    check_space(h, psi);
+    TQ_REQUIRE(h->prec == psi->prec, "state and Hamiltonian precisions differ");
+    // H psi is not asked for: under the XOR-ELL schedule (or none) the half
+    // pass, where the build laid out its tables (complex64 from
+    // HALF_MIN_QUBITS on: below, launch and read-back outweigh the pass).  It
+    // reads amplitudes by pairs of rows (16-byte aligned states only) and has
+    // no wait that a test could let run out.
+    if ((c->spmv_lanes == SPMV_AUTO || c->spmv_lanes == TQ_SPMV_XELL) && h->view.hcls && !c->test_flags &&
+        reinterpret_cast<uintptr_t>(psi->data) % 16 == 0)
+        launch(c, "energy_xell", s, [&] {
+            return launch_energy_half(h->view, psi->data, part, c->tickets, c->step, hs, c->sm_count, s);
+        });
+    else
+        run_energy(c, h, psi, part, s, hs);
     TQ_CUDA(cudaStreamSynchronize(s));
     *E = hs->energy;
     raise_status(c, hs->status, s);

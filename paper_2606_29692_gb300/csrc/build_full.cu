@@ -307,13 +307,13 @@ __device__ __forceinline__ void add_rows(uint32_t (&w)[4], uint32_t k) {
 // at most G entries, and G is below 2^14 for 26 qubits.
 __global__ void __launch_bounds__(BW * 32)
 k_build_count(BuildView v, long long D, long long B, unsigned long long tol, unsigned long long amb, int* rowcnt,
-              int* blkcnt, BuildSeg* seg, unsigned long long* n_amb) {
+              int* blkcnt, uint2* hcls, int* halfcnt, BuildSeg* seg, unsigned long long* n_amb) {
     extern __shared__ unsigned char sk_raw[];
-    __shared__ int s_rows[BW], s_pairs[BW], s_max[BW];
+    __shared__ int s_rows[BW], s_pairs[BW], s_half[BW], s_max[BW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned char* wkeep = sk_raw + (size_t)wid * 2 * v.W;      // kept and ambiguous rows of the wide groups
     unsigned char* wamb = wkeep + v.W;
-    int rows = 0, pairs = 0, mx = 0, namb = 0;
+    int rows = 0, pairs = 0, half = 0, mx = 0, namb = 0;
     for (int j = 0; j < BLOCKS_PER_WARP; ++j) {
         const long long R = ((long long)blockIdx.x * BW + wid) * BLOCKS_PER_WARP + j;
         if (R >= B) break;                                       // warp-uniform
@@ -333,7 +333,7 @@ k_build_count(BuildView v, long long D, long long B, unsigned long long tol, uns
         }
         __syncwarp();
         uint32_t cnt[4] = {0u, 0u, 0u, 0u};
-        int any = 0;
+        uint32_t any[3] = {0u, 0u, 0u};        // pairs, by class of the mask's top bit (two 16-bit counts a word)
         for (int g = lane; g < v.G; g += 32) {
             const BuildGroup r = load_group(v.rec, g);
             uint32_t k, q = 0;
@@ -348,12 +348,22 @@ k_build_count(BuildView v, long long D, long long B, unsigned long long tol, uns
             }
             k &= vm;
             namb += __popc(q & vm);
-            any += k != 0;
+            if (k) {
+                int c = 0;
+                if (v.half_bit)
+#pragma unroll
+                    for (int j = 0; j < HALF_CLASSES; ++j) c += g >= v.cls[j];
+                const uint32_t one = 1u << (16 * (c & 1));
+                any[0] += c < 2 ? one : 0u;
+                any[1] += (c >> 1) == 1 ? one : 0u;
+                any[2] += c > 3 ? one : 0u;
+            }
             add_rows(cnt, k);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) cnt[q] = __reduce_add_sync(0xffffffffu, cnt[q]);
-        any = __reduce_add_sync(0xffffffffu, any);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) any[q] = __reduce_add_sync(0xffffffffu, any[q]);
         if (lane < 8 && (vm >> lane) & 1u) {
             const uint32_t word = lane < 2 ? cnt[0] : lane < 4 ? cnt[1] : lane < 6 ? cnt[2] : cnt[3];
             const int n = (int)((word >> (16 * (lane & 1))) & 0xffffu);
@@ -362,8 +372,21 @@ k_build_count(BuildView v, long long D, long long B, unsigned long long tol, uns
             rows += n;
         }
         if (lane == 0) {
-            blkcnt[R] = any;
-            pairs += any;
+            static_assert(HALF_CLASSES == 4, "four 16-bit offsets per block");
+            const uint32_t o1 = any[0] & 0xffffu, o2 = o1 + (any[0] >> 16), o3 = o2 + (any[1] & 0xffffu),
+                           o4 = o3 + (any[1] >> 16), o5 = o4 + any[2];
+            blkcnt[R] = (int)o5;
+            pairs += (int)o5;
+            if (v.half_bit) {
+                // the half pass takes a class where the row's bit is 0
+                const uint32_t top = (uint32_t)(R >> (v.half_bit - 3));
+                const int n = (int)(o1 + ((top & 1u) ? 0u : o2 - o1) + ((top & 2u) ? 0u : o3 - o2) +
+                                    ((top & 4u) ? 0u : o4 - o3) + ((top & 8u) ? 0u : o5 - o4));
+                hcls[R] = make_uint2(o1 | (o2 << 16), o3 | (o4 << 16));
+                // the split's measure: a block's own work is that of about 48 pairs
+                halfcnt[R] = n + 48;
+                half += n + 48;
+            }
         }
         __syncwarp();
     }
@@ -373,15 +396,17 @@ k_build_count(BuildView v, long long D, long long B, unsigned long long tol, uns
     if (lane == 0) {
         s_rows[wid] = rows;
         s_pairs[wid] = pairs;
+        s_half[wid] = half;
         s_max[wid] = mx;
         if (namb) atomicAdd(n_amb, (unsigned long long)namb);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        BuildSeg o{0, 0, 0};
+        BuildSeg o{0, 0, 0, 0};
         for (int i = 0; i < BW; ++i) {
             o.rows += s_rows[i];
             o.pairs += s_pairs[i];
+            o.half += s_half[i];
             o.max_row = max(o.max_row, s_max[i]);
         }
         seg[blockIdx.x] = o;
@@ -389,41 +414,40 @@ k_build_count(BuildView v, long long D, long long B, unsigned long long tol, uns
 }
 
 // Exclusive offsets of the segments (one CTA, coalesced rounds of 1024).
-__global__ void __launch_bounds__(1024) k_build_scan(const BuildSeg* __restrict__ seg, int n, longlong2* off,
+__global__ void __launch_bounds__(1024) k_build_scan(const BuildSeg* __restrict__ seg, int n, BuildOffsets* off,
                                                      BuildTotals* out) {
-    __shared__ long long sr[32], sp[32];
+    __shared__ long long sw[3][32];
     __shared__ int sm[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    long long base_r = 0, base_p = 0;
+    long long base[3] = {0, 0, 0};
     int mx = 0;
     for (int i0 = 0; i0 < n; i0 += 1024) {
         const int i = i0 + threadIdx.x;
-        const BuildSeg s = i < n ? seg[i] : BuildSeg{0, 0, 0};
-        long long r = s.rows, p = s.pairs;
+        const BuildSeg s = i < n ? seg[i] : BuildSeg{0, 0, 0, 0};
+        const long long own[3] = {s.rows, s.pairs, s.half};
+        long long inc[3] = {own[0], own[1], own[2]};
         mx = max(mx, s.max_row);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long a = __shfl_up_sync(0xffffffffu, r, o), b = __shfl_up_sync(0xffffffffu, p, o);
-            if (lane >= o) {
-                r += a;
-                p += b;
+        for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const long long a = __shfl_up_sync(0xffffffffu, inc[q], o);
+                if (lane >= o) inc[q] += a;
             }
-        }
-        if (lane == 31) {
-            sr[wid] = r;
-            sp[wid] = p;
-        }
+        if (lane == 31)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) sw[q][wid] = inc[q];
         __syncthreads();
-        long long br = base_r, bp = base_p;
-        for (int w = 0; w < 32; ++w) {
-            if (w < wid) {
-                br += sr[w];
-                bp += sp[w];
+        long long at[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            at[q] = base[q] + inc[q] - own[q];
+            for (int w = 0; w < 32; ++w) {
+                if (w < wid) at[q] += sw[q][w];
+                base[q] += sw[q][w];
             }
-            base_r += sr[w];
-            base_p += sp[w];
         }
-        if (i < n) off[i] = make_longlong2(br + r - s.rows, bp + p - s.pairs);
+        if (i < n) off[i] = {at[0], at[1], at[2]};
         __syncthreads();
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
@@ -432,8 +456,9 @@ __global__ void __launch_bounds__(1024) k_build_scan(const BuildSeg* __restrict_
     if (threadIdx.x == 0) {
         int m = 0;
         for (int w = 0; w < 32; ++w) m = max(m, sm[w]);
-        out->rows = base_r;
-        out->pairs = base_p;
+        out->rows = base[0];
+        out->pairs = base[1];
+        out->half = base[2];
         out->max_row = m;
     }
 }
@@ -441,35 +466,43 @@ __global__ void __launch_bounds__(1024) k_build_scan(const BuildSeg* __restrict_
 // rowptr and xptr of one segment per CTA from its offsets (nothing when a
 // total does not fit int32: the host refuses the build then).
 __global__ void __launch_bounds__(SEG_BLOCKS * 8)
-k_build_offsets(const int* __restrict__ rowcnt, const int* __restrict__ blkcnt, const longlong2* __restrict__ off,
-                const BuildTotals* __restrict__ tot, long long D, long long B, int* rowptr, int* xptr) {
+k_build_offsets(const int* __restrict__ rowcnt, const int* __restrict__ blkcnt, const int* __restrict__ halfcnt,
+                const BuildOffsets* __restrict__ off, const BuildTotals* __restrict__ tot, long long D, long long B,
+                int* rowptr, int* xptr, int* hptr) {
     constexpr int NW = SEG_BLOCKS * 8 / 32;
     static_assert(SEG_BLOCKS <= 32, "the pair counts of a segment are scanned by one warp");
     __shared__ int sr[NW];
     if (tot->rows >= INT_MAX || tot->pairs >= INT_MAX) return;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const long long r = (long long)blockIdx.x * SEG_BLOCKS * 8 + t, b = (long long)blockIdx.x * SEG_BLOCKS + t;
-    const longlong2 o = off[blockIdx.x];
+    const BuildOffsets o = off[blockIdx.x];
     const int c = r < D ? rowcnt[r] : 0;
     const int x = t < SEG_BLOCKS && b < B ? blkcnt[b] : 0;
-    int ci = c, xi = x;
+    const int y = hptr && t < SEG_BLOCKS && b < B ? halfcnt[b] : 0;
+    int ci = c, xi = x, yi = y;
 #pragma unroll
     for (int k = 1; k < 32; k <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, ci, k), y = __shfl_up_sync(0xffffffffu, xi, k);
+        const int a0 = __shfl_up_sync(0xffffffffu, ci, k), a1 = __shfl_up_sync(0xffffffffu, xi, k),
+                  a2 = __shfl_up_sync(0xffffffffu, yi, k);
         if (lane >= k) {
-            ci += a;
-            xi += y;
+            ci += a0;
+            xi += a1;
+            yi += a2;
         }
     }
     if (lane == 31) sr[wid] = ci;
     __syncthreads();
     int before = 0;
     for (int w = 0; w < wid; ++w) before += sr[w];
-    if (r < D) rowptr[r] = (int)o.x + before + ci - c;
-    if (t < SEG_BLOCKS && b < B) xptr[b] = (int)o.y + xi - x;
+    if (r < D) rowptr[r] = (int)o.rows + before + ci - c;
+    if (t < SEG_BLOCKS && b < B) {
+        xptr[b] = (int)o.pairs + xi - x;
+        if (hptr) hptr[b] = (int)min(o.half + yi - y, 0x7fffffffll);   // balance only: may saturate
+    }
     if (blockIdx.x == 0 && t == 0) {
         rowptr[D] = (int)tot->rows;
         xptr[B] = (int)tot->pairs;
+        if (hptr) hptr[B] = (int)min(tot->half, 0x7fffffffll);
     }
 }
 
@@ -688,12 +721,13 @@ int launch_build_diag(long long D, const int* dbin, const uint32_t* dz, const do
 }
 
 int launch_build_count(const BuildView& v, long long D, long long B, unsigned long long tol, unsigned long long amb,
-                       int* rowcnt, int* blkcnt, BuildSeg* seg, longlong2* off, BuildTotals* tot, int* rowptr,
-                       int* xptr, cudaStream_t s) {
+                       int* rowcnt, int* blkcnt, int* halfcnt, BuildSeg* seg, BuildOffsets* off, BuildTotals* tot,
+                       int* rowptr, int* xptr, uint2* hcls, int* hptr, cudaStream_t s) {
     const int n = build_segments(B);
-    k_build_count<<<n, BW * 32, (size_t)BW * 2 * v.W, s>>>(v, D, B, tol, amb, rowcnt, blkcnt, seg, &tot->amb);
+    k_build_count<<<n, BW * 32, (size_t)BW * 2 * v.W, s>>>(v, D, B, tol, amb, rowcnt, blkcnt, hcls, halfcnt, seg,
+                                                           &tot->amb);
     k_build_scan<<<1, 1024, 0, s>>>(seg, n, off, tot);
-    k_build_offsets<<<n, SEG_BLOCKS * 8, 0, s>>>(rowcnt, blkcnt, off, tot, D, B, rowptr, xptr);
+    k_build_offsets<<<n, SEG_BLOCKS * 8, 0, s>>>(rowcnt, blkcnt, halfcnt, off, tot, D, B, rowptr, xptr, hptr);
     return 3;
 }
 

@@ -25,11 +25,14 @@ struct BuildRun {
 };
 
 struct BuildSeg {
-    int rows, pairs, max_row;
+    int rows, pairs, half, max_row;
+};
+struct BuildOffsets {
+    long long rows, pairs, half;
 };
 
 struct BuildTotals {
-    long long rows, pairs;
+    long long rows, pairs, half;
     unsigned long long amb;
     int max_row, pad;
 };
@@ -66,6 +69,8 @@ struct BuildView {
     const uint32_t* hx;
     const int* hoff;
     const uint32_t* sib;
+    int half_bit;            // lowest of the HALF_CLASSES top index bits, or 0: no half pass
+    int cls[HALF_CLASSES];   // first group whose mask has a bit at or above half_bit + j
 };
 
 int build_segments(long long B);
@@ -76,9 +81,10 @@ int launch_build_tables(const BuildView& v, int n_runs, const uint32_t* comb, co
                         cudaStream_t s);
 int launch_build_diag(long long D, const int* dbin, const uint32_t* dz, const double* dc, double* diag, int sms,
                       cudaStream_t s);
+// hcls, hptr: the half pass's tables (null when v.half_bit is 0).
 int launch_build_count(const BuildView& v, long long D, long long B, unsigned long long tol, unsigned long long amb,
-                       int* rowcnt, int* blkcnt, BuildSeg* seg, longlong2* off, BuildTotals* tot, int* rowptr,
-                       int* xptr, cudaStream_t s);
+                       int* rowcnt, int* blkcnt, int* halfcnt, BuildSeg* seg, BuildOffsets* off, BuildTotals* tot,
+                       int* rowptr, int* xptr, uint2* hcls, int* hptr, cudaStream_t s);
 int launch_build_fill(const BuildView& v, long long D, long long B, long long nnz, unsigned long long tol, int prec,
                       const int* rowptr, int* col, void* val, const int* xptr, uint32_t* xmask, void* xval, int sms,
                       cudaStream_t s);

@@ -143,6 +143,9 @@ constexpr int XELL_ROWS = 8;   // rows per XOR-ELL block
 constexpr int SPMV_AUTO = -1;
 constexpr int SPMV_C128_LANES = 4;
 
+constexpr int HALF_CLASSES = 4;        // top index bits told apart by the half pass
+constexpr int HALF_MIN_QUBITS = 16;
+
 // Hamiltonian: float64 diagonal + off-diagonal CSR + the same off-diagonal
 // entries in XOR-ELL form + X-mask-grouped terms.
 struct HamView {
@@ -164,6 +167,10 @@ struct HamView {
                             // (both arrays padded to whole copy chunks)
     int xgrid;              // CTAs of the staged XOR-ELL energy launch
     const int* xsplit;      // [xgrid + 1] first row block of each CTA
+    // half pass (energies without H psi, complex64, HALF_MIN_QUBITS and more):
+    // pairs by class of the mask's top index bit
+    const uint2* hcls;      // [n_blocks] first pair of classes 1 .. 4 in the block (16 bits each), or null
+    const int* hsplit;      // [half_warps + 1] first row block of each warp, balanced by the pairs the pass reads
     int G;                  // off-diagonal X-mask groups
     const uint32_t* gx;     // [G] group masks
     const int* goff;        // [G + 1] term offsets
@@ -268,6 +275,10 @@ int launch_xell_split(const int* xptr, long long n_blocks, int grid, int* split,
 int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2* w,
                        float2* w32, double* partials, unsigned* ticket, DevStep* step, DevStep* host,
                        int sms, cudaStream_t s, int lanes_per_row);
+// The energy alone (no H psi), complex64, Hamiltonians with h.hcls.
+int half_warps(int sms);
+int launch_energy_half(const HamView& h, const void* psi, double* partials, unsigned* ticket, DevStep* step,
+                       DevStep* host, int sms, cudaStream_t s);
 // complex128 over a space of at most ENERGY_FEW rows: one row per group of
 // lanes (one partial pair per CTA, at most ENERGY_FEW / 32 of them).
 constexpr long long ENERGY_FEW16 = 1 << 12, ENERGY_FEW = 1 << 14;

@@ -402,6 +402,226 @@ k_energy_xell_tma(HamView h, const typename C2<T>::type* __restrict__ psi, doubl
     }
 }
 
+// The energy alone from about 0.6 of the XOR-ELL pairs (complex64).  H is real
+// and symmetric, so the coupling of rows r and r ^ x enters the energy twice
+// with the same value: of a pair whose mask's top bit is one of the four
+// highest index bits, only the row block with that bit clear is read, and
+// counts twice (the masks below are read in full; all of them would halve the
+// work, but these four classes hold four fifths of the pairs and their
+// choice is constant over long runs of blocks).  A block's pairs ascend by
+// mask, so a class is one run of the block's pairs (h.hcls).  No H psi is
+// formed: the callers that need it run the full pass.
+//
+// One warp per block, the blocks split over all warps by pairs (h.hsplit).
+// Lane 4 sub + u takes pairs sub, sub + 8, .. of a run and rows 2u, 2u + 1:
+// their two columns lie in one aligned 16 bytes, so a warp gathers eight
+// pairs with one load.  The next round's masks and values are loaded (past
+// the first-level cache, which the amplitudes keep) while this round's
+// amplitudes arrive.  Row sums meet once per block; the rows are finished in
+// float64 for 32 blocks together, outside the loop over rounds (inside it the
+// compiler runs the float64 instructions in every round: 530 us).
+//
+// What bounds it: latency of the loads in flight (a round waits for the pair
+// stream from memory, 0.62 GB at 18 qubits, and for the gathers through the
+// L2).  18 qubits: 222 us for the full pass, 164 us here; rounds of 16, 24
+// and 32 pairs at 4, 4 and 3 CTAs per SM: 206, 165 (with spills) and 173 us,
+// a second round ahead gives nothing.  The full pass's ring over the same
+// pairs was 235 us: each block costs every warp of a CTA about 300
+// instructions there, as many as the pairs themselves.
+constexpr int HALF_THREADS = 256;
+constexpr int HALF_CTAS = 2;                 // per SM
+constexpr int HALF_K = 8;                    // steps of eight pairs per round
+
+// A run of a block's pairs: pairs s .. e - 1, rows R * 8 ..; flags: counts
+// half, last run of its block.
+struct alignas(16) HalfRun {
+    int s, e, R, flags;
+};
+constexpr int HALF_LOW = 1, HALF_LAST = 2, HALF_STOP = 4;
+
+// One round's masks and values, its block, and the flags of the run that ends
+// with it.
+template <int K>
+struct HalfRound {
+    uint32_t x[K];
+    float2 av[K];
+    int R, flags;
+};
+
+// The runs of block R (at most three: the low class, and neighbouring classes
+// together) to `out`; returns their number.
+__device__ __forceinline__ int half_runs(uint32_t R, int bit, int p0, int p1, uint2 cls, HalfRun* out) {
+    static_assert(HALF_CLASSES == 4, "at most two runs of four classes");
+    const int o[HALF_CLASSES + 2] = {0, (int)(cls.x & 0xffffu), (int)(cls.x >> 16), (int)(cls.y & 0xffffu),
+                                     (int)(cls.y >> 16), p1 - p0};
+    const uint32_t top = R >> (bit - 3);
+    int n = 0;
+    if (o[1] > 0) out[n++] = {p0, p0 + o[1], (int)R, HALF_LOW};
+    int s = 0, e = 0;                        // open run
+#pragma unroll
+    for (int c = 1; c <= HALF_CLASSES; ++c) {
+        if (!((top >> (c - 1)) & 1u)) {
+            if (e != o[c]) {
+                if (e > s) out[n++] = {p0 + s, p0 + e, (int)R, 0};
+                s = o[c];
+            }
+            e = o[c + 1];
+        }
+    }
+    if (e > s) out[n++] = {p0 + s, p0 + e, (int)R, 0};
+    if (n) out[n - 1].flags |= HALF_LAST;
+    return n;
+}
+
+// Mask and value of pair q (zero from e on), past the first-level cache.
+__device__ __forceinline__ void load_pair(const uint32_t* mask, const float2* val, int q, int e, uint32_t& x,
+                                          float2& a) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.lt.s32 p, %5, %6;\n"
+        "mov.b32 %0, 0;\n"
+        "mov.b32 %1, 0f00000000;\n"
+        "mov.b32 %2, 0f00000000;\n"
+        "@p ld.global.nc.L1::no_allocate.b32 %0, [%3];\n"
+        "@p ld.global.nc.L1::no_allocate.v2.f32 {%1, %2}, [%4];\n"
+        "}\n"
+        : "=&r"(x), "=&f"(a.x), "=&f"(a.y)
+        : "l"(mask), "l"(val), "r"(q), "r"(e));
+}
+
+__global__ void __launch_bounds__(HALF_THREADS, HALF_CTAS)
+k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsigned* ticket, DevStep* step,
+              DevStep* host) {
+    constexpr int K = HALF_K;
+    __shared__ HalfRun s_run[HALF_THREADS / 32][3 * 32 + 1];
+    __shared__ float2 s_row[HALF_THREADS / 32][32 * XELL_ROWS];
+    __shared__ double sh[2 * (HALF_THREADS / 32)];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, u = lane & 3, sub = lane >> 2;
+    const int bit = h.nq - HALF_CLASSES;
+    const uint32_t dmask = (uint32_t)(h.D - 1);
+    const float2* __restrict__ val = static_cast<const float2*>(h.xval);
+    const int w = blockIdx.x * (HALF_THREADS / 32) + wid;
+    const int b0 = h.hsplit[w], b1 = h.hsplit[w + 1];
+    HalfRun* run = s_run[wid];
+    float2* row = s_row[wid];
+    double num = 0.0, den = 0.0;
+    for (int G0 = b0; G0 < b1; G0 += 32) {
+        // the runs of 32 blocks, one block per lane
+        HalfRun own[3];
+        int n = 0;
+        const int own_block = G0 + lane;
+        if (own_block < b1)
+            n = half_runs((uint32_t)own_block, bit, h.xptr[own_block], h.xptr[own_block + 1], h.hcls[own_block], own);
+        int at = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += a;
+        }
+        const int nr = __shfl_sync(0xffffffffu, at, 31);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k < n) run[at - n + k] = own[k];
+        if (lane == 0) run[nr] = {0, 0, 0, HALF_STOP};
+        for (int j = lane; j < 32 * XELL_ROWS; j += 32) row[j] = make_float2(0.f, 0.f);    // blocks without pairs
+        __syncwarp();
+        // one round's pairs are on their way while the last one's are summed
+        int i = 0;
+        HalfRun g = run[0];
+        int p = g.s;
+        auto fill = [&](HalfRound<K>& r) {
+            r.R = g.R;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int q = p + 8 * k + sub;
+                load_pair(h.xmask + q, val + (size_t)q * (XELL_ROWS / 2) + u, q, g.e, r.x[k], r.av[k]);
+            }
+            p += 8 * K;
+            r.flags = 0;
+            if (p >= g.e) {                                  // warp-uniform
+                r.flags = g.flags;
+                if (i < nr) {
+                    g = run[++i];
+                    p = g.s;
+                }
+            }
+        };
+        float2 A = make_float2(0.f, 0.f), Bv = make_float2(0.f, 0.f);
+        auto sum = [&](HalfRound<K>& r) {
+            const int R = r.R, flags = r.flags;
+            const uint32_t ru = (uint32_t)R * XELL_ROWS + 2 * u;
+            float4 v[K];
+            float2 c[K];
+            uint32_t odd[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const uint32_t a = (ru ^ r.x[k]) & dmask;
+                v[k] = __ldg(reinterpret_cast<const float4*>(psi + (a & ~1u)));
+                c[k] = r.av[k];
+                odd[k] = a & 1u;
+            }
+            fill(r);
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const float2 v0 = odd[k] ? make_float2(v[k].z, v[k].w) : make_float2(v[k].x, v[k].y);
+                const float2 v1 = odd[k] ? make_float2(v[k].x, v[k].y) : make_float2(v[k].z, v[k].w);
+                A = __ffma2_rn(make_float2(c[k].x, c[k].x), v0, A);
+                Bv = __ffma2_rn(make_float2(c[k].y, c[k].y), v1, Bv);
+            }
+            if (flags & HALF_LOW) {                          // read from both sides: half of each (exact)
+                A = make_float2(0.5f * A.x, 0.5f * A.y);
+                Bv = make_float2(0.5f * Bv.x, 0.5f * Bv.y);
+            }
+            if (flags & HALF_LAST) {
+                // each lane ends with one component of one row
+                const bool hi = lane & 4, im = lane & 8;
+                float2 m = hi ? Bv : A;
+                const float2 o = hi ? A : Bv;
+                m.x += __shfl_xor_sync(0xffffffffu, o.x, 4);
+                m.y += __shfl_xor_sync(0xffffffffu, o.y, 4);
+                float f = (im ? m.y : m.x) + __shfl_xor_sync(0xffffffffu, im ? m.x : m.y, 8);
+                f += __shfl_xor_sync(0xffffffffu, f, 16);
+                if (lane < 16) reinterpret_cast<float*>(row)[((R - G0) * XELL_ROWS + 2 * u + (hi ? 1 : 0)) * 2 + (im ? 1 : 0)] = f;
+                A = Bv = make_float2(0.f, 0.f);
+            }
+        };
+        HalfRound<K> r;
+        fill(r);
+        while (!(r.flags & HALF_STOP)) sum(r);
+        // the rows in float64, four blocks at a time
+        __syncwarp();
+        const int rows = min(32, b1 - G0) * XELL_ROWS;
+        for (int j = lane; j < rows; j += 32) {
+            const long long r = (long long)G0 * XELL_ROWS + j;
+            const float2 p = psi[r], m = row[j];
+            const double px = (double)p.x, py = (double)p.y, n2 = fma(px, px, py * py);
+            const double o = fma(px, (double)m.x, py * (double)m.y);
+            num += fma(h.diag[r], n2, 2.0 * o);
+            den += n2;
+        }
+    }
+    double v[2] = {num, den};
+    block_sum<2>(v, sh);
+    if (threadIdx.x == 0) {
+        partials[2 * blockIdx.x] = v[0];
+        partials[2 * blockIdx.x + 1] = v[1];
+    }
+    if (last_block(ticket, gridDim.x)) {
+        double a, b;
+        block_sum_pairs(partials, 0, (int)gridDim.x, sh, a, b);
+        if (threadIdx.x == 0) {
+            const double e = a / b;
+            step->e_num = a;
+            step->e_den = b;
+            step->energy = e;
+            if (host) publish(host, step, e);
+            *ticket = 0u;
+        }
+    }
+}
+
 // Same energy from the X-mask-grouped terms (no CSR), one row per lane:
 // the warp walks the groups together, so every lane reads the same term
 // (a broadcast) and the 32 gathers psi[r ^ x] of its consecutive rows fall
@@ -1317,6 +1537,15 @@ int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2*
     if (psi_prec == TQ_C128)
         return energy_dispatch<double, double>(lanes, h, psi, w, w32, partials, ticket, step, host, sms, s);
     return energy_dispatch<float, float>(lanes, h, psi, w, w32, partials, ticket, step, host, sms, s);
+}
+
+int half_grid(int sms) { return sms * HALF_CTAS; }
+int half_warps(int sms) { return half_grid(sms) * (HALF_THREADS / 32); }
+
+int launch_energy_half(const HamView& h, const void* psi, double* partials, unsigned* ticket, DevStep* step,
+                       DevStep* host, int sms, cudaStream_t s) {
+    k_energy_half<<<half_grid(sms), HALF_THREADS, 0, s>>>(h, static_cast<const float2*>(psi), partials, ticket, step, host);
+    return 1;
 }
 
 int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,

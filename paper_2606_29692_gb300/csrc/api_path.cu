@@ -86,10 +86,9 @@ extern "C" int tq_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double
     // H psi is not asked for: under the XOR-ELL schedule (or none) the half
     // pass, where the build laid out its tables (complex64 from
     // HALF_MIN_QUBITS on: below, launch and read-back outweigh the pass).  It
-    // reads amplitudes by pairs of rows (16-byte aligned states only) and has
-    // no wait that a test could let run out.
-    if ((c->spmv_lanes == SPMV_AUTO || c->spmv_lanes == TQ_SPMV_XELL) && h->view.hcls && !c->test_flags &&
-        reinterpret_cast<uintptr_t>(psi->data) % 16 == 0)
+    // reads amplitudes by pairs of rows (every state is 16-byte aligned) and
+    // has no wait that a test could let run out.
+    if ((c->spmv_lanes == SPMV_AUTO || c->spmv_lanes == TQ_SPMV_XELL) && h->view.hcls && !c->test_flags)
         launch(c, "energy_xell", s, [&] {
             return launch_energy_half(h->view, psi->data, part, c->tickets, c->step, hs, c->sm_count, s);
         });

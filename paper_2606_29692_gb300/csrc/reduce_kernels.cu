@@ -415,9 +415,9 @@ k_energy_xell_tma(HamView h, const typename C2<T>::type* __restrict__ psi, doubl
 // One warp per block, the blocks split over all warps by pairs (h.hsplit).
 // Lane 4 sub + u takes pairs sub, sub + 8, .. of a run and rows 2u, 2u + 1:
 // their two columns lie in one aligned 16 bytes, so a warp gathers eight
-// pairs with one load.  The next round's masks and values are loaded (past
-// the first-level cache, which the amplitudes keep) while this round's
-// amplitudes arrive.  Row sums meet once per block; the rows are finished in
+// pairs with one load.  The next masks and values are loaded (past the
+// first-level cache, which the amplitudes keep) while the current amplitudes
+// arrive.  Row sums meet once per block; the rows are finished in
 // float64 for 32 blocks together, outside the loop over rounds (inside it the
 // compiler runs the float64 instructions in every round: 530 us).
 //

@@ -615,10 +615,12 @@ int dispatch_support(int ppt, const PoolView& p, int n_states, void* psi, const 
 // Tiles per state.  One tile lets the CTA finish the state's norm itself (no
 // second launch) and take states from the shared counter, which evens out
 // singles and doubles; more tiles spread few or large states over the GPU.
-// Up to 14 qubits one tile wins from 64 states on in complex64 (14 qubits,
-// four pairs per thread pipelined: 64 states 10 us against 12 with tiles,
-// 2048 states 28 against 30-31, 8192 states 99), from 512 on in complex128
-// (14 qubits, 512 states 40 against 42-44 us; 64 states 25 against 15).
+// In complex64 one tile wins from 64 states on up to 12 qubits (both launches
+// are short: 8.2-9.0 us a call against 10.7), and beyond once there are 4
+// states per SM (14 qubits, four pairs per thread pipelined: 200 states 14.3
+// us with one tile, 11.0 with four; 380 states 14.0 and 14.5; 2048 states 28
+// against 30-31, 8192 states 99); in complex128 from 512 on up to 14 qubits
+// (512 states 40 against 42-44 us; 64 states 25 against 15).
 // Beyond, eight tiles (16 qubits, 2048 complex64 states: 154 us with one
 // tile, 138 with 4, 135 with 8; 1024 complex128 states 310, 194, 189; 18
 // qubits, 256 complex128 states 166 with 8, 203 with 32).  Batches below
@@ -627,7 +629,7 @@ int dispatch_support(int ppt, const PoolView& p, int n_states, void* psi, const 
 int support_tiles(int nq, int prec, int n_states, int sms) {
     const long long dpairs = nq >= 4 ? 1ll << (nq - 4) : 1;
     long long t = nq > 14 ? 8 : 1;
-    if (nq <= 14 && n_states >= (prec == TQ_C128 ? 512 : 64)) return 1;
+    if (prec == TQ_C128 ? nq <= 14 && n_states >= 512 : nq <= 12 && n_states >= 64) return 1;
     const long long want = (4ll * sms + n_states - 1) / std::max(n_states, 1);
     const long long cap = std::max(1ll, dpairs / 32);
     while (t < want && t * 2 <= cap) t *= 2;

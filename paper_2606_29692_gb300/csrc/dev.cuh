@@ -12,9 +12,11 @@ namespace tq {
 // Programmatic launch.  A kernel launched with launch_pdl may start while its
 // predecessor in the stream still runs; pdl_wait returns when that one has
 // completed and its writes are visible, and every CTA calls it before it
-// touches anything an earlier launch writes (and before it may return).  Such
-// data is not read through __ldg or an unconditional read-only pointer at a
-// kernel's top: the compiler may move those loads over the wait.
+// touches anything an overlapping launch writes (and before it may return).
+// Such data is not read through __ldg or a const __restrict__ pointer: both
+// promise that nothing writes it while the kernel runs, so the compiler may
+// move those loads over the wait.  What a launch before an unoverlapped one
+// wrote is final when the kernel starts and may be read either way.
 // pdl_start lets the next launch start in turn.  Only the short kernels of the
 // ADAPT step's chain are launched so (20 steps at 12 qubits, complex128: 1.345 to 1.32 ms):
 // dependents that wait beside a long pass slow it (launched so everywhere,

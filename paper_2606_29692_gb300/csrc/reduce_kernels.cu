@@ -1052,6 +1052,8 @@ template <typename T, int L>
 __global__ void __launch_bounds__(256)
 k_line_support(HamView h, PoolView p, const typename C2<T>::type* __restrict__ psi, DevStep* step,
                double* partials, unsigned* ticket) {
+    // psi is older than the gradient pass two launches ahead, which overlaps
+    // nothing before it: read-only for this kernel
     pdl_wait();
     using V = typename C2<T>::type;
     __shared__ double sh[5 * 8];

@@ -385,13 +385,12 @@ template <> struct NormPair<float> {
 
 template <typename T>
 __global__ void __launch_bounds__(LARGE_NORM_BS)
-k_large_norm(PoolView p, int k_imm, const DevStep* gate, const typename C2<T>::type* __restrict__ psi,
-             double2* __restrict__ part) {
+k_large_norm(PoolView p, int k_imm, const DevStep* gate, const typename C2<T>::type* psi, double2* part) {
     constexpr int NW = LARGE_NORM_BS / 32;
     static_assert(NW <= 32, "one lane per warp in the last tree");
     __shared__ __align__(16) double2 red[NW];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_start();
     if (gate && gate->converged) return;
     const int k = gate ? gate->selected : k_imm;
     const OpRec<T> op = make_rec<T>(p, k);
@@ -435,11 +434,14 @@ k_large_norm(PoolView p, int k_imm, const DevStep* gate, const typename C2<T>::t
 template <typename T>
 __global__ void __launch_bounds__(LARGE_BS)
 k_large_update(PoolView p, int k_imm, double th_imm, const DevStep* gate, typename C2<T>::type* psi,
-               const double2* __restrict__ part, int n_part, double* norm2_out) {
+               const double2* part, int n_part, double* norm2_out) {
     using V = typename C2<T>::type;
     __shared__ double scale_sh;
-    if (!n_part) asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (gate && gate->converged) return;
+    if (!n_part) pdl_wait();
+    if (gate && gate->converged) {
+        pdl_wait();        // no launch completes before the one it overlaps
+        return;
+    }
     const int k = gate ? gate->selected : k_imm;
     const double theta = gate ? gate->theta : th_imm;
     const OpRec<T> op = make_rec<T>(p, k);
@@ -464,7 +466,7 @@ k_large_update(PoolView p, int k_imm, double th_imm, const DevStep* gate, typena
         if (ok[j]) unit_update<T>(op, hb, cf, c5, s5, w[j], unused);
     T sc = T(1);
     if (n_part) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        pdl_wait();
         if (threadIdx.x < 32) {
             NormPair<T> t;
             for (int i = threadIdx.x; i < n_part; i += 32) t.add_slot(part + i);

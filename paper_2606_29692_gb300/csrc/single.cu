@@ -292,36 +292,43 @@ k_taylor5_single_closed(PoolView p, int k_imm, double th_imm, const DevStep* gat
 
 // ---------------------------------------- states beyond one cluster
 //
-// Two launches for a pool whose entries are +-1 (A^2 = -I on the support S,
-// so the new norm follows from the input state, as in
-// k_taylor5_single_closed):
-//   k_large_norm:   sum |psi|^2 and sum_S |psi|^2, one partial pair per CTA;
+// Two launches for a pool whose entries are +-1:
+//   k_large_norm:   one partial of ||psi'||^2 per CTA;
 //   k_large_update: the update and the rescale in one pass, after every CTA
 //                   has added the partials in CTA order.
 // The state is read twice and written once (update, norm reduction and
-// rescale as three launches read and write it twice).  Programmatic launch:
-// the norm kernel lets the update kernel start once its own wait is over,
-// so the update's amplitudes are loaded and its series summed while the norm
-// is still being reduced; it only stores after its wait.  Before that wait it
-// reads nothing the norm kernel writes, and what it does read was complete
-// before the norm kernel's wait ended.
+// rescale as three launches read and write it twice).  complex64: the norm
+// kernel runs the same update in registers and sums the squares of its
+// float32 results, so the norm is that of the amplitudes as rounded, and the
+// rescale factor is applied as a float32 pair, one rounding per amplitude
+// (with the norm from the input and a float32 factor | ||psi'|| - 1 | was
+// 2 to 3 times as large).  complex128: A^2 = -I on the support S, so the norm
+// follows from sum |psi|^2 and sum_S |psi|^2 and the coefficients, as in
+// k_taylor5_single_closed (an update costs the float64 pipe more than the
+// squares).
+// Programmatic launch: the norm kernel lets the update kernel start once its
+// own wait is over, so the update's amplitudes are loaded and its series
+// summed while the norm is still being reduced; it only stores after its
+// wait.  Before that wait it reads nothing the norm kernel writes, and what it
+// does read was complete before the norm kernel's wait ended.
 //
 // What bounds it: launch latency and the L2 (a 20-qubit complex64 state, 8 MB,
 // stays there); in complex128 the float64 pipe.  Renormalised, as three
-// launches and here: complex64 at 18, 20, 22, 24 qubits 24.6 / 9.1,
-// 43.1 / 8.8, 115 / 23.6, 430 / 96 us; complex128 24.6 / 20.8, 49.2 / 31.2,
-// 132 / 100, 521 / 361 us.
+// launches and here: complex64 at 18, 20, 22, 24 qubits 24.7 / 8.7,
+// 43.1 / 8.8, 115 / 21.3, 426 / 82.5 us; complex128 25.2 / 20.6, 48.4 / 33.4,
+// 132 / 105, 530 / 369 us.
 constexpr int LARGE_BS = 256;
 constexpr int LARGE_UPT = 2;         // units of 4 amplitudes per thread
 constexpr int LARGE_NORM_BS = 512;
 constexpr int LARGE_NORM_PER_SM = 2;
 
-// The two running sums (all rows, rows on S).  complex64 carries them as
-// float32 (hi, lo) pairs all the way to the last addition: every float64
-// warp instruction holds its SM quarter's pipe for 64 cycles, and float64
-// shuffle trees in every warp took 6 of the first version's 18 us.
-template <typename T> struct NormPair;
-template <> struct NormPair<double> {
+// The running sum of a norm.  complex128: |psi|^2 over all rows and over S.
+// complex64: |psi'|^2 as a float32 (hi, lo) pair (about 48 bits) all the way to
+// the last addition: every float64 warp instruction holds its SM quarter's
+// pipe for 64 cycles, and float64 shuffle trees in every warp took 6 of the
+// first version's 18 us.
+template <typename T> struct NormSum;
+template <> struct NormSum<double> {
     double a = 0.0, s = 0.0;
     __device__ __forceinline__ void add(double na, double ns) {
         a += na;
@@ -340,52 +347,87 @@ template <> struct NormPair<double> {
         a = slot->x;
         s = slot->y;
     }
-    __device__ __forceinline__ double all() const { return a; }
-    __device__ __forceinline__ double on() const { return s; }
+    // ||psi'||^2, growth: c5^2 + s5^2 - 1
+    __device__ __forceinline__ double norm2(double growth) const { return fma(growth, s, a); }
 };
-template <> struct NormPair<float> {
-    float ah = 0.f, al = 0.f, sh = 0.f, sl = 0.f;
-    __device__ __forceinline__ void acc(float& hi, float& lo, float h2, float l2) {
+template <> struct NormSum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float h2, float l2) {
         float sum, err;
         two_sum(hi, h2, sum, err);
         hi = sum;
         lo += l2 + err;
     }
-    __device__ __forceinline__ void add(float na, float ns) {
-        acc(ah, al, na, 0.f);
-        acc(sh, sl, ns, 0.f);
-    }
     __device__ __forceinline__ void add_slot(const double2* slot) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(slot));
-        acc(ah, al, v.x, v.y);
-        acc(sh, sl, v.z, v.w);
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(slot));
+        add(v.x, v.y);
     }
     __device__ __forceinline__ void warp() {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            const float h = __shfl_down_sync(0xffffffffu, ah, o), l = __shfl_down_sync(0xffffffffu, al, o);
-            const float h2 = __shfl_down_sync(0xffffffffu, sh, o), l2 = __shfl_down_sync(0xffffffffu, sl, o);
-            acc(ah, al, h, l);
-            acc(sh, sl, h2, l2);
+            const float h = __shfl_down_sync(0xffffffffu, hi, o), l = __shfl_down_sync(0xffffffffu, lo, o);
+            add(h, l);
         }
     }
-    __device__ __forceinline__ void store(double2* slot) const {
-        *reinterpret_cast<float4*>(slot) = make_float4(ah, al, sh, sl);
-    }
+    __device__ __forceinline__ void store(double2* slot) const { *reinterpret_cast<float2*>(slot) = make_float2(hi, lo); }
     __device__ __forceinline__ void load(const double2* slot) {
-        const float4 v = *reinterpret_cast<const float4*>(slot);
-        ah = v.x;
-        al = v.y;
-        sh = v.z;
-        sl = v.w;
+        const float2 v = *reinterpret_cast<const float2*>(slot);
+        hi = v.x;
+        lo = v.y;
     }
-    __device__ __forceinline__ double all() const { return (double)ah + (double)al; }
-    __device__ __forceinline__ double on() const { return (double)sh + (double)sl; }
+    __device__ __forceinline__ double norm2(double) const { return (double)hi + (double)lo; }
 };
+
+// A thread's share of the sums: complex64 units of 4 amplitudes, updated.
+__device__ __forceinline__ void large_norm_rows(const OpRec<float>& op, int nq, double theta, const float2* psi,
+                                                NormSum<float>& sum) {
+    float cf[6];
+    taylor_coefs_fast<float>(theta, cf);
+    const int hb = 31 - __clz(op.x);
+    const uint32_t units = (1u << nq) >> 2, step = gridDim.x * LARGE_NORM_BS;
+    for (uint32_t u0 = blockIdx.x * LARGE_NORM_BS + threadIdx.x; u0 < units; u0 += LARGE_UPT * step) {
+        PairUnit<float2> w[LARGE_UPT];
+#pragma unroll
+        for (int j = 0; j < LARGE_UPT; ++j)
+            if (u0 + j * step < units) unit_load(psi, op.x, hb, u0 + j * step, w[j]);
+        float t = 0.f;                           // 8 squares a unit, summed plainly
+#pragma unroll
+        for (int j = 0; j < LARGE_UPT; ++j)
+            if (u0 + j * step < units) unit_update<float>(op, hb, cf, 0.0, 0.0, w[j], t);
+        sum.add(t, 0.f);
+    }
+}
+
+// complex128: two consecutive rows a round, four rounds in flight.
+__device__ __forceinline__ void large_norm_rows(const OpRec<double>& op, int nq, double, const double2* psi,
+                                                NormSum<double>& sum) {
+    const uint32_t D = 1u << nq, step = gridDim.x * LARGE_NORM_BS * 2;
+    const int flip = (op.dcode >> 4) & 7;                    // parity codes of delta = 1
+    const int cx = (op.dcode >> 8) & 7;                      // and of x: col = r ^ x
+    for (uint32_t r0 = (blockIdx.x * LARGE_NORM_BS + threadIdx.x) * 2; r0 < D; r0 += 4 * step) {
+        double2 a[4], b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            a[j] = b[j] = make_double2(0.0, 0.0);
+            const uint32_t r = r0 + j * step;
+            if (r < D && r >= r0) load2(psi, r, a[j], b[j]);
+        }
+        double all = 0.0, on = 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int code = (base_code(op, r0 + j * step) & 7) ^ cx;
+            const double na = a[j].x * a[j].x + a[j].y * a[j].y, nb = b[j].x * b[j].x + b[j].y * b[j].y;
+            all += na + nb;
+            on += (code == op.t ? na : 0.0) + ((code ^ flip) == op.t ? nb : 0.0);
+        }
+        sum.add(all, on);
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(LARGE_NORM_BS)
-k_large_norm(PoolView p, int k_imm, const DevStep* gate, const typename C2<T>::type* psi, double2* part) {
+k_large_norm(PoolView p, int k_imm, double th_imm, const DevStep* gate, const typename C2<T>::type* psi,
+             double2* part) {
     constexpr int NW = LARGE_NORM_BS / 32;
     static_assert(NW <= 32, "one lane per warp in the last tree");
     __shared__ __align__(16) double2 red[NW];
@@ -394,39 +436,35 @@ k_large_norm(PoolView p, int k_imm, const DevStep* gate, const typename C2<T>::t
     if (gate && gate->converged) return;
     const int k = gate ? gate->selected : k_imm;
     const OpRec<T> op = make_rec<T>(p, k);
-    const uint32_t D = 1u << p.nq, step = gridDim.x * LARGE_NORM_BS * 2;
-    const int flip = (op.dcode >> 4) & 7;                    // parity codes of delta = 1
-    const int cx = (op.dcode >> 8) & 7;                      // and of x: col = r ^ x
-    NormPair<T> sum;
-    // four rounds of two consecutive rows in flight, summed plainly (8
-    // squares) before they join the running pair
-    for (uint32_t r0 = (blockIdx.x * LARGE_NORM_BS + threadIdx.x) * 2; r0 < D; r0 += 4 * step) {
-        typename C2<T>::type a[4], b[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            a[j] = b[j] = typename C2<T>::type{};
-            const uint32_t r = r0 + j * step;
-            if (r < D && r >= r0) load2(psi, r, a[j], b[j]);
-        }
-        T all = T(0), on = T(0);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int code = (base_code(op, r0 + j * step) & 7) ^ cx;
-            const T na = a[j].x * a[j].x + a[j].y * a[j].y, nb = b[j].x * b[j].x + b[j].y * b[j].y;
-            all += na + nb;
-            on += (code == op.t ? na : T(0)) + ((code ^ flip) == op.t ? nb : T(0));
-        }
-        sum.add(all, on);
-    }
+    NormSum<T> sum;
+    large_norm_rows(op, p.nq, gate ? gate->theta : th_imm, psi, sum);
     sum.warp();
     if ((threadIdx.x & 31) == 0) sum.store(&red[threadIdx.x >> 5]);
     __syncthreads();
     if (threadIdx.x < 32) {
-        NormPair<T> t;
+        NormSum<T> t;
         if (threadIdx.x < NW) t.load(&red[threadIdx.x]);
         t.warp();
         if (threadIdx.x == 0) t.store(part + blockIdx.x);
     }
+}
+
+// c5^2 + s5^2 - 1 of the coefficients as rounded, to about twice float64's
+// digits: the products' and the sum's errors are carried.
+__device__ __forceinline__ double closed_growth(double c5, double s5) {
+    const double c = __dmul_rn(c5, c5), s = __dmul_rn(s5, s5);
+    const double ec = fma(c5, c5, -c), es = fma(s5, s5, -s);
+    const double t = __dadd_rn(c, s), b = __dsub_rn(t, c);
+    const double et = __dadd_rn(__dsub_rn(c, __dsub_rn(t, b)), __dsub_rn(s, b));
+    return __dadd_rn(__dsub_rn(t, 1.0), __dadd_rn(et, __dadd_rn(ec, es)));
+}
+
+__device__ __forceinline__ void rescale(double2& v, double sc, double) {
+    v.x *= sc;
+    v.y *= sc;
+}
+__device__ __forceinline__ void rescale(float2& v, float hi, float lo) {
+    v = __ffma2_rn(v, make_float2(hi, hi), __fmul2_rn(v, make_float2(lo, lo)));
 }
 
 // Units of 4 amplitudes (PairUnit).  n_part: the norm kernel's CTAs, 0 when
@@ -436,7 +474,7 @@ __global__ void __launch_bounds__(LARGE_BS)
 k_large_update(PoolView p, int k_imm, double th_imm, const DevStep* gate, typename C2<T>::type* psi,
                const double2* part, int n_part, double* norm2_out) {
     using V = typename C2<T>::type;
-    __shared__ double scale_sh;
+    __shared__ T scale_sh[2];          // 1 / ||psi'||, and what its first part leaves of it
     if (!n_part) pdl_wait();
     if (gate && gate->converged) {
         pdl_wait();        // no launch completes before the one it overlaps
@@ -464,33 +502,31 @@ k_large_update(PoolView p, int k_imm, double th_imm, const DevStep* gate, typena
 #pragma unroll
     for (int j = 0; j < LARGE_UPT; ++j)
         if (ok[j]) unit_update<T>(op, hb, cf, c5, s5, w[j], unused);
-    T sc = T(1);
     if (n_part) {
+        double growth = 0.0;
+        if constexpr (sizeof(T) == 8) growth = threadIdx.x ? 0.0 : closed_growth(c5, s5);
         pdl_wait();
         if (threadIdx.x < 32) {
-            NormPair<T> t;
+            NormSum<T> t;
             for (int i = threadIdx.x; i < n_part; i += 32) t.add_slot(part + i);
             t.warp();
             if (threadIdx.x == 0) {
-                const double t2 = theta * theta, t6 = t2 * t2 * t2;   // c5^2 + s5^2 - 1 in closed form
-                const double n = fma(t6 * fma(t2, fma(t2, 1.0 / 14400.0, -1.0 / 960.0), 1.0 / 360.0), t.on(), t.all());
-                scale_sh = rsqrt(n);
+                const double n = t.norm2(growth), sc = 1.0 / sqrt(n);
+                scale_sh[0] = (T)sc;
+                scale_sh[1] = (T)(sc - (double)scale_sh[0]);
                 if (blockIdx.x == 0 && norm2_out) *norm2_out = n;
             }
         }
         __syncthreads();
-        sc = (T)scale_sh;
     }
 #pragma unroll
     for (int j = 0; j < LARGE_UPT; ++j) {
         if (!ok[j]) continue;
         if (n_part) {
-            V* v[4] = {&w[j].a0, &w[j].a1, &w[j].b0, &w[j].b1};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                v[i]->x *= sc;
-                v[i]->y *= sc;
-            }
+            rescale(w[j].a0, scale_sh[0], scale_sh[1]);
+            rescale(w[j].a1, scale_sh[0], scale_sh[1]);
+            rescale(w[j].b0, scale_sh[0], scale_sh[1]);
+            rescale(w[j].b1, scale_sh[0], scale_sh[1]);
         }
         unit_store(psi, x, hb, w[j]);
     }
@@ -701,7 +737,8 @@ int launch_large_t(const PoolView& p, int k, double theta, const DevStep* gate, 
                    double* norm2, int sms, cudaStream_t s) {
     using V = typename C2<T>::type;
     const long long units = (1ll << p.nq) >> 2;
-    const long long need = ((1ll << p.nq) + 2 * LARGE_NORM_BS - 1) / (2 * LARGE_NORM_BS);
+    const long long items = sizeof(T) == 4 ? units : 2 * units;      // units, or pairs of consecutive rows
+    const long long need = (items + LARGE_NORM_BS - 1) / LARGE_NORM_BS;
     const int n = renorm ? (int)std::min<long long>(need, large_parts(sms)) : 0;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -714,7 +751,7 @@ int launch_large_t(const PoolView& p, int k, double theta, const DevStep* gate, 
     if (n) {
         cfg.gridDim = dim3(n);
         cfg.blockDim = dim3(LARGE_NORM_BS);
-        e = cudaLaunchKernelEx(&cfg, k_large_norm<T>, p, k, gate, static_cast<const V*>(psi), part);
+        e = cudaLaunchKernelEx(&cfg, k_large_norm<T>, p, k, theta, gate, static_cast<const V*>(psi), part);
     }
     cfg.gridDim = dim3((unsigned)((units + LARGE_BS * LARGE_UPT - 1) / (LARGE_BS * LARGE_UPT)));
     cfg.blockDim = dim3(LARGE_BS);

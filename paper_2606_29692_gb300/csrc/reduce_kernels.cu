@@ -448,6 +448,39 @@ struct HalfRound {
     int R, flags;
 };
 
+// A float32 pair (about 48 bits) that TwoSum adds to.  A row's sum is one from
+// the rounds' sums on: a lane serves an eighth of a row's pairs, where the full
+// pass spreads a row over 64 slots, and every coupling counts twice.  With plain
+// float32 sums the energy's distance from float64 was 0.8 to 2.0 times the full
+// pass's, with pairs it is 0.6 to 1.1 times (root mean square over 40 states, 16
+// and 18 qubits, a few determinants to random); 18 qubits 175.4 us a call
+// with plain sums, 174.5 with pairs.
+struct PairSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float h, float l) {
+        float s, e;
+        two_sum(hi, h, s, e);
+        hi = s;
+        lo += l + e;
+    }
+    __device__ __forceinline__ void add_lane(const PairSum& give, int o) {
+        add(__shfl_xor_sync(0xffffffffu, give.hi, o), __shfl_xor_sync(0xffffffffu, give.lo, o));
+    }
+};
+struct RowSum {
+    PairSum x, y;
+    __device__ __forceinline__ void add(float2 v) {
+        x.add(v.x, 0.f);
+        y.add(v.y, 0.f);
+    }
+    __device__ __forceinline__ void halve() {
+        x.hi *= 0.5f;
+        x.lo *= 0.5f;
+        y.hi *= 0.5f;
+        y.lo *= 0.5f;
+    }
+};
+
 // The runs of block R (at most three: the low class, and neighbouring classes
 // together) to `out`; returns their number.
 __device__ __forceinline__ int half_runs(uint32_t R, int bit, int p0, int p1, uint2 cls, HalfRun* out) {
@@ -495,7 +528,7 @@ k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsig
               DevStep* host) {
     constexpr int K = HALF_K;
     __shared__ HalfRun s_run[HALF_THREADS / 32][3 * 32 + 1];
-    __shared__ float2 s_row[HALF_THREADS / 32][32 * XELL_ROWS];
+    __shared__ float2 s_row[HALF_THREADS / 32][32 * XELL_ROWS * 2];     // (hi, lo) per component
     __shared__ double sh[2 * (HALF_THREADS / 32)];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, u = lane & 3, sub = lane >> 2;
     const int bit = h.nq - HALF_CLASSES;
@@ -525,7 +558,7 @@ k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsig
         for (int k = 0; k < 3; ++k)
             if (k < n) run[at - n + k] = own[k];
         if (lane == 0) run[nr] = {0, 0, 0, HALF_STOP};
-        for (int j = lane; j < 32 * XELL_ROWS; j += 32) row[j] = make_float2(0.f, 0.f);    // blocks without pairs
+        for (int j = lane; j < 32 * XELL_ROWS * 2; j += 32) row[j] = make_float2(0.f, 0.f);    // blocks without pairs
         __syncwarp();
         // one round's pairs are on their way while the last one's are summed
         int i = 0;
@@ -548,7 +581,7 @@ k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsig
                 }
             }
         };
-        float2 A = make_float2(0.f, 0.f), Bv = make_float2(0.f, 0.f);
+        RowSum A, Bv;                                        // rows 2u and 2u + 1
         auto sum = [&](HalfRound<K>& r) {
             const int R = r.R, flags = r.flags;
             const uint32_t ru = (uint32_t)R * XELL_ROWS + 2 * u;
@@ -563,28 +596,32 @@ k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsig
                 odd[k] = a & 1u;
             }
             fill(r);
+            float2 a = make_float2(0.f, 0.f), b = a;         // the round's products, joined to the running sums below
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 const float2 v0 = odd[k] ? make_float2(v[k].z, v[k].w) : make_float2(v[k].x, v[k].y);
                 const float2 v1 = odd[k] ? make_float2(v[k].x, v[k].y) : make_float2(v[k].z, v[k].w);
-                A = __ffma2_rn(make_float2(c[k].x, c[k].x), v0, A);
-                Bv = __ffma2_rn(make_float2(c[k].y, c[k].y), v1, Bv);
+                a = __ffma2_rn(make_float2(c[k].x, c[k].x), v0, a);
+                b = __ffma2_rn(make_float2(c[k].y, c[k].y), v1, b);
             }
+            A.add(a);
+            Bv.add(b);
             if (flags & HALF_LOW) {                          // read from both sides: half of each (exact)
-                A = make_float2(0.5f * A.x, 0.5f * A.y);
-                Bv = make_float2(0.5f * Bv.x, 0.5f * Bv.y);
+                A.halve();
+                Bv.halve();
             }
             if (flags & HALF_LAST) {
                 // each lane ends with one component of one row
                 const bool hi = lane & 4, im = lane & 8;
-                float2 m = hi ? Bv : A;
-                const float2 o = hi ? A : Bv;
-                m.x += __shfl_xor_sync(0xffffffffu, o.x, 4);
-                m.y += __shfl_xor_sync(0xffffffffu, o.y, 4);
-                float f = (im ? m.y : m.x) + __shfl_xor_sync(0xffffffffu, im ? m.x : m.y, 8);
-                f += __shfl_xor_sync(0xffffffffu, f, 16);
-                if (lane < 16) reinterpret_cast<float*>(row)[((R - G0) * XELL_ROWS + 2 * u + (hi ? 1 : 0)) * 2 + (im ? 1 : 0)] = f;
-                A = Bv = make_float2(0.f, 0.f);
+                RowSum m = hi ? Bv : A;
+                const RowSum o = hi ? A : Bv;
+                m.x.add_lane(o.x, 4);
+                m.y.add_lane(o.y, 4);
+                PairSum f = im ? m.y : m.x;
+                f.add_lane(im ? m.x : m.y, 8);
+                f.add_lane(f, 16);
+                if (lane < 16) row[((R - G0) * XELL_ROWS + 2 * u + (hi ? 1 : 0)) * 2 + (im ? 1 : 0)] = make_float2(f.hi, f.lo);
+                A = Bv = RowSum{};
             }
         };
         HalfRound<K> r;
@@ -595,9 +632,9 @@ k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsig
         const int rows = min(32, b1 - G0) * XELL_ROWS;
         for (int j = lane; j < rows; j += 32) {
             const long long r = (long long)G0 * XELL_ROWS + j;
-            const float2 p = psi[r], m = row[j];
+            const float2 p = psi[r], mx = row[2 * j], my = row[2 * j + 1];
             const double px = (double)p.x, py = (double)p.y, n2 = fma(px, px, py * py);
-            const double o = fma(px, (double)m.x, py * (double)m.y);
+            const double o = fma(px, (double)mx.x + (double)mx.y, py * ((double)my.x + (double)my.y));
             num += fma(h.diag[r], n2, 2.0 * o);
             den += n2;
         }

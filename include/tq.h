@@ -124,17 +124,19 @@ int tq_ctx_get_l2_fetch(tq_ctx* ctx, int* bytes);
 
 /* Schedule of the energy SpMV (the H pass of tq_energy, tq_pool_gradients
  * and tq_adapt_step): 4, 8, 16 or 32 lanes sharing one row of the CSR,
- * or TQ_SPMV_XELL for the XOR-ELL layout.  Until one is set, complex64 uses
- * the XOR-ELL layout and complex128 the CSR at 4 lanes; a sector
- * Hamiltonian, which has only the CSR, uses 8 lanes for either.  Every Hamiltonian
- * holds both layouts of the same off-diagonal entries: the CSR, and blocks
+ * or TQ_SPMV_XELL for the XOR-ELL layout.  Until one is set, and after
+ * TQ_SPMV_AUTO, complex64 uses the XOR-ELL layout and complex128 the CSR, at 16
+ * lanes up to 2^12 rows, 8 up to 2^14 and 4 beyond; a sector Hamiltonian,
+ * which has only the CSR, uses 8 lanes for either.  Setting a schedule sets it
+ * for both precisions.  Every Hamiltonian holds both layouts of the same off-diagonal entries: the CSR, and blocks
  * of 8 rows where each X-mask present in the block stores its 8 values
  * H[8R+i][(8R+i)^x] (zero where the CSR has no entry), so one pair's 8
- * gathers read one aligned run of 8 amplitudes.  Under XOR-ELL, tq_energy on
- * complex64 from 16 qubits reads 0.6 of the pairs (H is symmetric).  The
- * autotuner times the H pass under every schedule on (ham, psi) and keeps
- * the fastest.  Synchronises the device. */
-enum { TQ_SPMV_XELL = 0 };
+ * gathers read one aligned run of 8 amplitudes.  tq_energy on complex64 from
+ * 16 qubits, which needs no H psi, reads 0.6 of the pairs (H is symmetric),
+ * unless a CSR schedule was set.  The autotuner times the pass with H psi under
+ * every schedule on (ham, psi) and keeps the fastest for ham's precision.
+ * Synchronises the device. */
+enum { TQ_SPMV_XELL = 0, TQ_SPMV_AUTO = -1 };
 /* Failure-path tests only (no counterpart in the paper).  With
  * TQ_TEST_WITHHOLD_CHUNK set, the XOR-ELL energy pass never copies its
  * first pair chunk into shared memory, so every consumer wait on it runs

@@ -18,6 +18,7 @@ from ._native import (TQ_BK, TQ_C64, TQ_C128, TQ_JW, AdaptResult, Completion, Re
 
 TQ_REQ_EVOLVE, TQ_REQ_ENERGY, TQ_REQ_GRADIENTS = 0, 1, 2
 TQ_SPMV_XELL = 0      # energy-SpMV schedule: the XOR-ELL layout (else CSR lanes per row)
+TQ_SPMV_AUTO = -1     # the default of each precision and size
 TQ_TEST_WITHHOLD_CHUNK = 1
 
 __all__ = [
@@ -26,7 +27,7 @@ __all__ = [
     "build_pool", "evolve_taylor5", "evolve_taylor5_csr", "energy", "energy_matrix_free",
     "pool_gradients", "adapt_step", "evolve_taylor5_batch", "evolve_taylor5_batch_host",
     "state_set_hf", "pool_csr", "ham_csr", "lib", "autotune_pair", "fp64_fma_rate", "energy_noalloc", "Batch", "autotune_spmv", "Server",
-    "TQ_REQ_EVOLVE", "TQ_REQ_ENERGY", "TQ_REQ_GRADIENTS", "TQ_SPMV_XELL", "ham_xell",
+    "TQ_REQ_EVOLVE", "TQ_REQ_ENERGY", "TQ_REQ_GRADIENTS", "TQ_SPMV_XELL", "TQ_SPMV_AUTO", "ham_xell",
     "sector_dim", "sector_basis", "build_hamiltonian_sector", "build_pool_sector", "pool_sector_table",
     "TQ_COMMUTE_FULL", "TQ_COMMUTE_QWC", "pool_families", "pool_families_host",
     "ansatz_energy_grad", "adapt_vqe", "read_fcidump", "write_fcidump", "state_save", "state_load", "replay",
@@ -204,8 +205,8 @@ class Context:
         call("tq_ctx_set_test_flags", self.handle, int(flags))
 
     def set_spmv_schedule(self, lanes_per_row):
-        """4, 8, 16 or 32 CSR lanes per row, or TQ_SPMV_XELL (until set: XELL for
-        complex64, 4 lanes for complex128)."""
+        """4, 8, 16 or 32 CSR lanes per row, TQ_SPMV_XELL, or TQ_SPMV_AUTO (until
+        set: XELL for complex64; for complex128 16, 8 or 4 lanes by size)."""
         call("tq_ctx_set_spmv_schedule", self.handle, int(lanes_per_row))
 
     def set_support_schedule(self, prec, pairs_per_thread):
@@ -617,7 +618,8 @@ def autotune_pair(ctx, pool, prec=TQ_C64, n_states=1024):
 
 
 def autotune_spmv(ctx, ham, state):
-    """Time every energy-SpMV schedule on (ham, state); set and return (schedule, ms).
+    """Time every energy-SpMV schedule on (ham, state); set it for ham's precision
+    and return (schedule, ms).
 
     The schedule is a CSR lanes-per-row count or TQ_SPMV_XELL."""
     l, ms = C.c_int(), C.c_double()

@@ -265,9 +265,12 @@ extern "C" int tq_ctx_set_spmv_schedule(tq_ctx* c, int lanes_per_row) {
     API_BEGIN
     TQ_REQUIRE(c != nullptr, "ctx is null");
     TQ_REQUIRE(lanes_per_row == TQ_SPMV_XELL || lanes_per_row == 4 || lanes_per_row == 8 ||
-                   lanes_per_row == 16 || lanes_per_row == 32,
-               "schedule must be 4, 8, 16 or 32 CSR lanes per row, or TQ_SPMV_XELL");
-    c->spmv_lanes = lanes_per_row;
+                   lanes_per_row == 16 || lanes_per_row == 32 || lanes_per_row == TQ_SPMV_AUTO,
+               "schedule must be 4, 8, 16 or 32 CSR lanes per row, TQ_SPMV_XELL or TQ_SPMV_AUTO");
+    for (int p : {TQ_C128, TQ_C64}) {
+        c->spmv_lanes[p] = lanes_per_row;
+        c->spmv_tuned[p] = false;
+    }
     API_END
 }
 
@@ -282,11 +285,12 @@ extern "C" int tq_autotune_spmv(tq_ctx* c, const tq_ham* h, const tq_state* psi,
     cudaEvent_t e0, e1;
     TQ_CUDA(cudaEventCreate(&e0));
     TQ_CUDA(cudaEventCreate(&e1));
-    int best = c->spmv_lanes;
+    int& lanes = c->spmv_lanes[h->prec];
+    int best = lanes;
     float best_t = 1e30f;
     for (int l : {4, 8, 16, 32, (int)TQ_SPMV_XELL}) {
         if (l == TQ_SPMV_XELL && h->sector) continue;   // a sector Hamiltonian has the CSR only
-        c->spmv_lanes = l;
+        lanes = l;
         run_energy(c, h, psi, part, 0);
         TQ_CUDA(cudaEventRecord(e0, 0));
         for (int r = 0; r < 3; ++r) run_energy(c, h, psi, part, 0);
@@ -302,7 +306,8 @@ extern "C" int tq_autotune_spmv(tq_ctx* c, const tq_ham* h, const tq_state* psi,
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c->spmv_lanes = best;
+    lanes = best;
+    c->spmv_tuned[h->prec] = true;
     if (best_lanes) *best_lanes = best;
     if (best_ms) *best_ms = best_t;
     API_END

@@ -173,19 +173,29 @@ size_t partials_needed(long long D, int n_gitems, int nq, int sms) {
     return n + 8;
 }
 
+// The schedule of the H pass over h: TQ_SPMV_XELL or CSR lanes per row.
+static int spmv_schedule(const tq_ctx* c, const tq_ham* h) {
+    const int lanes = c->spmv_lanes[h->prec];
+    if (h->sector) return lanes == TQ_SPMV_AUTO || lanes == TQ_SPMV_XELL ? 8 : lanes;   // the CSR only
+    if (lanes != TQ_SPMV_AUTO) return lanes;
+    if (h->prec == TQ_C64) return TQ_SPMV_XELL;
+    return h->D <= ENERGY_FEW16 ? 16 : h->D <= ENERGY_FEW ? 8 : SPMV_C128_LANES;
+}
+
 void run_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double* part, cudaStream_t s, DevStep* host) {
     check_space(h, psi);
     TQ_REQUIRE(h->prec == psi->prec, "state and Hamiltonian precisions differ");
     double2* w = static_cast<double2*>(c->scratch[S_W0]);
     float2* w32 = psi->prec == TQ_C64 ? static_cast<float2*>(c->scratch[S_W32]) : nullptr;
-    int lanes = c->spmv_lanes;
-    if (lanes == SPMV_AUTO && h->prec == TQ_C128 && !h->sector && h->D <= ENERGY_FEW) {
-        launch(c, "energy_csr", s, [&] { return launch_energy_few(h->view, psi->data, w, part, c->tickets, c->step, host, s); });
-        return;
-    }
-    if (lanes == SPMV_AUTO) lanes = h->prec == TQ_C128 && !h->sector ? SPMV_C128_LANES : (int)TQ_SPMV_XELL;
-    if (lanes == TQ_SPMV_XELL && h->sector) lanes = 8;   // a sector Hamiltonian has the CSR only
-    if (lanes == TQ_SPMV_XELL)
+    const int lanes = spmv_schedule(c, h);
+    // complex128 at the lanes launch_energy_few has: it beats the 64-row items
+    // at the same lanes (12 qubits 9.2 against 13.4 us), whoever asked for them
+    const long long few = lanes == 16 ? ENERGY_FEW16 : lanes == 8 ? ENERGY_FEW : 0;
+    if (h->prec == TQ_C128 && !h->sector && h->D <= few)
+        launch(c, "energy_csr", s, [&] {
+            return launch_energy_few(h->view, psi->data, w, part, c->tickets, c->step, host, s, lanes);
+        });
+    else if (lanes == TQ_SPMV_XELL)
         launch(c, "energy_xell", s, [&] {
             return launch_energy_xell(h->view, psi->data, psi->prec, w, w32, part, c->tickets, c->step, host, s,
                                       (c->test_flags & TQ_TEST_WITHHOLD_CHUNK) ? 0 : -1);

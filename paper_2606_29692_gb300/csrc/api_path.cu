@@ -83,12 +83,15 @@ extern "C" int tq_energy(tq_ctx* c, const tq_ham* h, const tq_state* psi, double
     auto* hs = static_cast<DevStep*>(host_scratch(c, sizeof(DevStep)));   // the kernel writes the result there
     check_space(h, psi);
     TQ_REQUIRE(h->prec == psi->prec, "state and Hamiltonian precisions differ");
-    // H psi is not asked for: under the XOR-ELL schedule (or none) the half
-    // pass, where the build laid out its tables (complex64 from
-    // HALF_MIN_QUBITS on: below, launch and read-back outweigh the pass).  It
-    // reads amplitudes by pairs of rows (every state is 16-byte aligned) and
-    // has no wait that a test could let run out.
-    if ((c->spmv_lanes == SPMV_AUTO || c->spmv_lanes == TQ_SPMV_XELL) && h->view.hcls && !c->test_flags)
+    // H psi is not asked for: the half pass, where the build laid out its
+    // tables (complex64 from HALF_MIN_QUBITS on: below, launch and read-back
+    // outweigh the pass), unless the caller asked for a CSR schedule.  A tuned
+    // schedule is that of the pass with H psi, which the half pass beats at
+    // every schedule (18 qubits 164 against 231 to 291 us).  It reads
+    // amplitudes by pairs of rows (every state is 16-byte aligned) and has no
+    // wait that a test could let run out.
+    const int asked = c->spmv_tuned[h->prec] ? (int)TQ_SPMV_AUTO : c->spmv_lanes[h->prec];
+    if ((asked == TQ_SPMV_AUTO || asked == TQ_SPMV_XELL) && h->view.hcls && !c->test_flags)
         launch(c, "energy_xell", s, [&] {
             return launch_energy_half(h->view, psi->data, part, c->tickets, c->step, hs, c->sm_count, s);
         });

@@ -132,15 +132,15 @@ struct PoolView {
 
 constexpr int XELL_ROWS = 8;   // rows per XOR-ELL block
 
-// The energy SpMV's schedule until the caller or an autotuner sets one: the
-// XOR-ELL layout for complex64, the CSR at 4 lanes per row for complex128.
+// The energy SpMV's schedule until the caller or an autotuner sets one
+// (spmv_schedule): the XOR-ELL layout for complex64; for complex128 the CSR, at
+// 4 lanes per row beyond ENERGY_FEW rows and below as launch_energy_few has it.
 // Complex128 products are bound by the float64 pipe, which works on a whole
 // warp instruction whatever its lanes hold: the XOR-ELL's zeros (half its
 // slots) cost as much as entries, and a wider row reduction adds float64
 // additions.  Traced, XOR-ELL against 4 lanes: 23 / 17 us at 12 qubits,
 // 59 / 27 at 14, 255 / 108 at 16, 1279 / 568 at 18 (8 lanes 581, 32 lanes
 // 728); complex64 at 16 and 18 qubits: 53 / 64 and 231 / 291.
-constexpr int SPMV_AUTO = -1;
 constexpr int SPMV_C128_LANES = 4;
 
 constexpr int HALF_CLASSES = 4;        // top index bits told apart by the half pass
@@ -279,11 +279,12 @@ int launch_energy_csr2(const HamView& h, const void* psi, int psi_prec, double2*
 int half_warps(int sms);
 int launch_energy_half(const HamView& h, const void* psi, double* partials, unsigned* ticket, DevStep* step,
                        DevStep* host, int sms, cudaStream_t s);
-// complex128 over a space of at most ENERGY_FEW rows: one row per group of
-// lanes (one partial pair per CTA, at most ENERGY_FEW / 32 of them).
+// complex128 over a full space of few rows: one row per group of lanes, 16 up
+// to ENERGY_FEW16 rows, 8 up to ENERGY_FEW (one partial pair per CTA, at most
+// ENERGY_FEW / 32 of them).
 constexpr long long ENERGY_FEW16 = 1 << 12, ENERGY_FEW = 1 << 14;
 int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,
-                      DevStep* host, cudaStream_t s);
+                      DevStep* host, cudaStream_t s, int lanes_per_row);
 // gradients read w in float32 (w32) for complex64 states, float64 (w) otherwise
 int launch_pool_gradients(const PoolView& p, const double2* w, const float2* w32,
                           const void* psi, int prec, const DevStep* step, double* partials,
@@ -409,7 +410,10 @@ struct tq_ctx {
     int grouped_lanes[2] = {1, 1};         // grouped-layout update: lanes per row (C128, C64)
     int grouped_ppt[2] = {1, 1};           // and pairs per lane
     int l2_fetch_default = 0;              // the CUDA context's L2 fetch granularity at creation (bytes)
-    int spmv_lanes = tq::SPMV_AUTO;        // energy SpMV: CSR lanes per row, 0 for XOR-ELL, or by precision
+    // energy SpMV (C128, C64): CSR lanes per row, TQ_SPMV_XELL or TQ_SPMV_AUTO;
+    // tuned: set by tq_autotune_spmv, which times the pass with H psi only
+    int spmv_lanes[2] = {TQ_SPMV_AUTO, TQ_SPMV_AUTO};
+    bool spmv_tuned[2] = {false, false};
     int test_flags = 0;                    // TQ_TEST_* (tests of the failure paths only)
     std::vector<tq_trace_rec> trace;      // recorded, not yet reported
     std::vector<cudaEvent_t> event_pool;  // reusable events

@@ -1588,9 +1588,9 @@ int launch_energy_half(const HamView& h, const void* psi, double* partials, unsi
 }
 
 int launch_energy_few(const HamView& h, const void* psi, double2* w, double* partials, unsigned* ticket, DevStep* step,
-                      DevStep* host, cudaStream_t s) {
+                      DevStep* host, cudaStream_t s, int lanes) {
     const auto* p = static_cast<const double2*>(psi);
-    if (h.D <= ENERGY_FEW16)
+    if (lanes == 16)
         k_energy_few<16><<<(int)((h.D + 15) / 16), 256, 0, s>>>(h, p, w, partials, ticket, step, host);
     else
         k_energy_few<8><<<(int)((h.D + 31) / 32), 256, 0, s>>>(h, p, w, partials, ticket, step, host);

@@ -739,13 +739,13 @@ int launch_build_fill(const BuildView& v, long long D, long long B, long long nn
     const size_t sx = (size_t)FILL_BW * v.W * (8 * vb + 1);
     const size_t sc = (size_t)FILL_BW * (v.W * (8 * vb + 1) + 2 * (size_t)v.H);
     if (prec == TQ_C128) {
-        cudaFuncSetAttribute(k_build_xell<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sx);
-        cudaFuncSetAttribute(k_build_csr<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
+        allow_smem(k_build_xell<double>);
+        allow_smem(k_build_csr<double>);
         k_build_xell<double><<<grid, FILL_BW * 32, sx, s>>>(v, D, B, tol, xptr, xmask, static_cast<double*>(xval));
         k_build_csr<double><<<grid, FILL_BW * 32, sc, s>>>(v, D, B, nnz, tol, rowptr, col, static_cast<double*>(val));
     } else {
-        cudaFuncSetAttribute(k_build_xell<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sx);
-        cudaFuncSetAttribute(k_build_csr<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
+        allow_smem(k_build_xell<float>);
+        allow_smem(k_build_csr<float>);
         k_build_xell<float><<<grid, FILL_BW * 32, sx, s>>>(v, D, B, tol, xptr, xmask, static_cast<float*>(xval));
         k_build_csr<float><<<grid, FILL_BW * 32, sc, s>>>(v, D, B, nnz, tol, rowptr, col, static_cast<float*>(val));
     }

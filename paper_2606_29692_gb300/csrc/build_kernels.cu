@@ -256,10 +256,10 @@ int launch_csr_fill(const HamView& h, double tol, int max_row, int* col, void* v
     const int bs = wpb * 32;
     const int grid = grid_for(h.D * 32, bs, sms, 8);
     if (prec == TQ_C128) {
-        cudaFuncSetAttribute(k_csr_fill<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_csr_fill<double>);
         k_csr_fill<double><<<grid, bs, smem, s>>>(h, tol, cap, col, static_cast<double*>(val));
     } else {
-        cudaFuncSetAttribute(k_csr_fill<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_csr_fill<float>);
         k_csr_fill<float><<<grid, bs, smem, s>>>(h, tol, cap, col, static_cast<float*>(val));
     }
     return 1;

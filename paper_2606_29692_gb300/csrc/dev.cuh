@@ -40,6 +40,20 @@ void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaSt
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
 }
 
+// Lets a kernel be launched with as much dynamic shared memory as there is
+// beside its static.  The limit belongs to the kernel, not to a launch: set to
+// each launch's own size, a call on another thread may lower it between this
+// one's setting and its launch, which is then refused.
+template <typename K>
+cudaError_t allow_smem(K kernel) {
+    constexpr int kPerBlock = 227 * 1024;
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kPerBlock - (int)at.sharedSizeBytes);
+}
+
 // complex type per precision: float2 (TQ_C64) or double2 (TQ_C128)
 template <typename T> struct C2;
 template <> struct C2<float> { using type = float2; };

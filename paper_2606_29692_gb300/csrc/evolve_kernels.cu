@@ -341,7 +341,7 @@ cudaError_t launch_cluster(int nq, int csize, const int* rowptr, const int* col,
     using V = typename C2<T>::type;
     auto kern = k_taylor5_csr_cluster<T, VT>;
     const size_t smem = (size_t)3 * ((1ll << nq) / csize) * sizeof(V);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     if (csize > 8) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

@@ -384,7 +384,7 @@ void sweep_shape(int nq, int* cs, int* tpb) {
 template <typename K>
 cudaError_t sweep_config(K kern, int cs, int tpb, size_t smem, cudaStream_t s, cudaLaunchConfig_t* cfg,
                          cudaLaunchAttribute* attr) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e == cudaSuccess && cs > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3(cs);

@@ -50,9 +50,14 @@ enum { TQ_JW = 0, TQ_BK = 1 };
 #define TQ_MAPPING_FIRST_RELABELLED 16
 
 /* Precisions: TQ_C128 runs every product and sum in float64.  TQ_C64 keeps
- * states and sparse products in complex64 (float32) while Hamiltonian
- * diagonals, energy and gradient dot reductions, norms and the convergence
- * test stay in float64. */
+ * states and sparse products in complex64 (float32).  Hamiltonian diagonals
+ * and the convergence test are float64; energy and gradient dot reductions
+ * and norms are float64 or, inside a kernel, float32 (hi, lo) pairs joined by
+ * TwoSum (about 48 bits) and widened at the end: pool gradients, ansatz
+ * gradients (products exact), norms of single states, and the row sums of the
+ * energy without H psi.  The ansatz gradients' pairs differ from float64 sums by
+ * 1e-16 to 1e-15 (8 to 18 qubits, 10 to 40 factors), where complex64 states leave
+ * 6e-8 to 1.1e-7. */
 enum { TQ_C128 = 0, TQ_C64 = 1 };
 
 enum {

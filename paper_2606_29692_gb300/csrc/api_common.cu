@@ -137,7 +137,9 @@ int update_tiles(const tq_pool* p, int prec, int upt) {
 }
 
 // Taylor-5 on n states (ops and angles from k/theta arrays, or k_fixed and
-// theta_fixed, or the step record when `gate` is set).  Returns true when
+// theta_fixed, or, in a sector, the step record when `gate` is set; the full
+// space's gated updates are the one-cluster and the large one, since every pool
+// generator's entries are +-1).  Returns true when
 // the launch also wrote the float64 norms (norm2[i] and/or *step_norm2);
 // otherwise they are in `part`, for launch_norm_reduce.
 bool launch_update(tq_ctx* c, const tq_pool* p, long long n, int prec, int upt, void* psi, const int* k,
@@ -150,13 +152,9 @@ bool launch_update(tq_ctx* c, const tq_pool* p, long long n, int prec, int upt, 
         });
         return sector_in_smem(p->view.sdim, prec);
     }
-    if (gate) {
-        launch(c, "taylor5_pair_gated", s, [&] { return launch_taylor5_pair_gated(p->view, prec, upt, psi, gate, part,
-                                                  c->sm_count, s); });
-    } else {
-        launch(c, "taylor5_pair", s, [&] { return launch_taylor5_pair(p->view, (int)n, prec, upt, psi, k, theta, k_fixed,
-                                                                      theta_fixed, part, c->sm_count, s); });
-    }
+    TQ_REQUIRE(!gate, "a gated update of the full space needs generators with entries +-1");
+    launch(c, "taylor5_pair", s, [&] { return launch_taylor5_pair(p->view, (int)n, prec, upt, psi, k, theta, k_fixed,
+                                                                  theta_fixed, part, c->sm_count, s); });
     return false;
 }
 

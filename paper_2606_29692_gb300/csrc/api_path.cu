@@ -113,7 +113,7 @@ extern "C" int tq_energy_matrix_free(tq_ctx* c, const tq_ham* h, const tq_state*
     cudaStream_t s = as_stream(stream);
     double* part = prepare(c, h->D, nullptr, h->nq);
     launch(c, "energy_matrix_free", s, [&] { return launch_energy_matrix_free(h->view, psi->data, psi->prec, part, c->tickets + 1,
-                                              c->step, nullptr, c->sm_count, s); });
+                                              c->step, c->sm_count, s); });
     *E = read_step(c, 0, s)->energy;
     API_END
 }

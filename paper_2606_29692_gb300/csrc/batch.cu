@@ -44,7 +44,7 @@
 namespace tq {
 
 struct TrajDev {
-    int nq, M, len, nch, chunk;
+    int nq, M, len;
     int eoff, ecnt;          // energy items of this trajectory
     int nslab, wslab;        // slabs of about wslab units of work each (kb_energy_smem):
     const int* cut;          // slab i is rows cut[i] .. cut[i + 1] - 1
@@ -998,8 +998,6 @@ extern "C" int tq_batch_create(tq_ctx* c, int n_traj, tq_ham* const* hams, tq_po
             d.xmask = h->view.xmask;
             d.xval = h->view.xval;
             d.pool = p->view;
-            d.chunk = 0;
-            d.nch = 0;
             d.eoff = (int)ei.size();
             for (long long r = 0; r < d.D; r += ROWS_PER_ITEM)
                 ei.push_back(make_int4(t, (int)r, (int)std::min<long long>(ROWS_PER_ITEM, d.D - r), 0));

@@ -264,8 +264,7 @@ int launch_energy_csr(const HamView& h, const void* psi, int psi_prec, double2* 
                       double* partials, unsigned* ticket, DevStep* step, int sms,
                       cudaStream_t s);
 int launch_energy_matrix_free(const HamView& h, const void* psi, int psi_prec,
-                              double* partials, unsigned* ticket, DevStep* step, DevStep* host,
-                              int sms, cudaStream_t s);
+                              double* partials, unsigned* ticket, DevStep* step, int sms, cudaStream_t s);
 int launch_energy_xell(const HamView& h, const void* psi, int psi_prec, double2* w, float2* w32,
                        double* partials, unsigned* ticket, DevStep* step, DevStep* host, cudaStream_t s,
                        int withhold_chunk = -1);
@@ -331,8 +330,6 @@ int launch_taylor5_single(const PoolView& p, int prec, bool unit_pool, int k, do
 int large_parts(int sms);
 int launch_taylor5_large(const PoolView& p, int prec, int k, double theta, const DevStep* gate, void* psi, int renorm,
                          double2* part, double* norm2, int sms, cudaStream_t s);
-int launch_taylor5_pair_gated(const PoolView& p, int prec, int upt, void* psi, const DevStep* step,
-                              double* partials, int sms, cudaStream_t s);
 int launch_scale_gated(void* psi, int prec, long long D, const double* norm2,
                        const DevStep* gate, cudaStream_t s);
 // The line search's three products in one pass over H: y_i = H x_i, x_i

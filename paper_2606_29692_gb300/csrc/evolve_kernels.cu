@@ -40,11 +40,10 @@ template <typename T, int UPT>
 __global__ void __launch_bounds__(PAIR_BS)
 k_taylor5_pair(PoolView p, int n_states, typename C2<T>::type* psi, const int* kk,
                const double* th, int k_imm, double th_imm, double* partials,
-               int tiles_per_state, const DevStep* gate) {
+               int tiles_per_state) {
     using V = typename C2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     OpRec<T>* ops = reinterpret_cast<OpRec<T>*>(smem_raw);
-    if (gate && gate->converged) return;
     // the vectorised pool layout, staged once per CTA
     for (int i = threadIdx.x; i < p.M; i += blockDim.x) ops[i] = make_rec<T>(p, i);
     __syncthreads();
@@ -415,7 +414,7 @@ int pair_grid(int M, int sms) {
 
 template <typename T, int UPT>
 int launch_pair(const PoolView& p, int n_states, void* psi, const int* k, const double* theta,
-                int k_imm, double theta_imm, double* partials, const DevStep* gate, int sms,
+                int k_imm, double theta_imm, double* partials, int sms,
                 cudaStream_t s) {
     using V = typename C2<T>::type;
     const long long units = (1ll << p.nq) >> 2;
@@ -427,7 +426,7 @@ int launch_pair(const PoolView& p, int n_states, void* psi, const int* k, const 
     if (grid < 1) grid = 1;
     const size_t smem = (size_t)p.M * sizeof(OpRec<T>);
     k_taylor5_pair<T, UPT><<<(int)grid, PAIR_BS, smem, s>>>(p, n_states, static_cast<V*>(psi), k, theta,
-                                                            k_imm, theta_imm, partials, tiles, gate);
+                                                            k_imm, theta_imm, partials, tiles);
     return 1;
 }
 
@@ -445,13 +444,13 @@ namespace {
 
 template <typename T>
 int dispatch_pair(int upt, const PoolView& p, int n_states, void* psi, const int* k, const double* theta,
-                  int k_imm, double theta_imm, double* partials, const DevStep* gate, int sms,
+                  int k_imm, double theta_imm, double* partials, int sms,
                   cudaStream_t s) {
     switch (upt) {
-        case 1: return launch_pair<T, 1>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, gate, sms, s);
-        case 2: return launch_pair<T, 2>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, gate, sms, s);
-        case 4: return launch_pair<T, 4>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, gate, sms, s);
-        case 8: return launch_pair<T, 8>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, gate, sms, s);
+        case 1: return launch_pair<T, 1>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, sms, s);
+        case 2: return launch_pair<T, 2>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, sms, s);
+        case 4: return launch_pair<T, 4>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, sms, s);
+        case 8: return launch_pair<T, 8>(p, n_states, psi, k, theta, k_imm, theta_imm, partials, sms, s);
         default: return -1;
     }
 }
@@ -462,15 +461,8 @@ int launch_taylor5_pair(const PoolView& p, int n_states, int prec, int upt, void
                         const double* theta, int k_imm, double theta_imm, double* partials, int sms,
                         cudaStream_t s) {
     if (prec == TQ_C128)
-        return dispatch_pair<double>(upt, p, n_states, psi, k, theta, k_imm, theta_imm, partials, nullptr, sms, s);
-    return dispatch_pair<float>(upt, p, n_states, psi, k, theta, k_imm, theta_imm, partials, nullptr, sms, s);
-}
-
-int launch_taylor5_pair_gated(const PoolView& p, int prec, int upt, void* psi, const DevStep* step,
-                              double* partials, int sms, cudaStream_t s) {
-    if (prec == TQ_C128)
-        return dispatch_pair<double>(upt, p, 1, psi, &step->selected, &step->theta, 0, 0.0, partials, step, sms, s);
-    return dispatch_pair<float>(upt, p, 1, psi, &step->selected, &step->theta, 0, 0.0, partials, step, sms, s);
+        return dispatch_pair<double>(upt, p, n_states, psi, k, theta, k_imm, theta_imm, partials, sms, s);
+    return dispatch_pair<float>(upt, p, n_states, psi, k, theta, k_imm, theta_imm, partials, sms, s);
 }
 
 int launch_norm_reduce(const double* partials, int prec, int n_states, int tiles_per_state,

@@ -669,7 +669,7 @@ k_energy_half(HamView h, const float2* __restrict__ psi, double* partials, unsig
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_energy_mf(HamView h, const typename C2<T>::type* __restrict__ psi, double* partials,
-            unsigned* ticket, DevStep* step, DevStep* host) {
+            unsigned* ticket, DevStep* step) {
     __shared__ double sh[2 * 8];
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -706,11 +706,9 @@ k_energy_mf(HamView h, const typename C2<T>::type* __restrict__ psi, double* par
         double a, b;
         block_sum_pairs(partials, 0, (int)gridDim.x, sh, a, b);
         if (threadIdx.x == 0) {
-            const double e = a / b;
             step->e_num = a;
             step->e_den = b;
-            step->energy = e;
-            if (host) publish(host, step, e);
+            step->energy = a / b;
             *ticket = 0u;
         }
     }
@@ -1000,28 +998,17 @@ k_line_dots(const typename C2<T>::type* z, const double2* w0, const double2* w1,
         a[4] += x1.x * v2.x + x1.y * v2.y;
         a[5] += x2.x * v2.x + x2.y * v2.y;
     }
-    // two-stage block sum (block_sum handles up to 4 values)
-    double lo[4] = {a[0], a[1], a[2], a[3]};
-    double hi[2] = {a[4], a[5]};
-    block_sum<4>(lo, sh);
-    block_sum<2>(hi, sh + 32);
-    if (threadIdx.x == 0) {
-        for (int j = 0; j < 4; ++j) partials[6 * blockIdx.x + j] = lo[j];
-        partials[6 * blockIdx.x + 4] = hi[0];
-        partials[6 * blockIdx.x + 5] = hi[1];
-    }
+    block_sum<6>(a, sh);
+    if (threadIdx.x == 0)
+        for (int j = 0; j < 6; ++j) partials[6 * blockIdx.x + j] = a[j];
     if (last_block(ticket, gridDim.x)) {
         // every thread sums a fixed stride of the blocks, then a fixed tree
         double f[6] = {0, 0, 0, 0, 0, 0};
         for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
             for (int j = 0; j < 6; ++j) f[j] += __ldcg(partials + 6 * b + j);
-        double lo2[4] = {f[0], f[1], f[2], f[3]};
-        double hi2[2] = {f[4], f[5]};
-        block_sum<4>(lo2, sh);
-        block_sum<2>(hi2, sh + 32);
+        block_sum<6>(f, sh);
         if (threadIdx.x == 0) {
-            const double tot[6] = {lo2[0], lo2[1], lo2[2], lo2[3], hi2[0], hi2[1]};
-            for (int j = 0; j < 6; ++j) step->dots[j] = tot[j] / step->e_den;
+            for (int j = 0; j < 6; ++j) step->dots[j] = f[j] / step->e_den;
             *ticket = 0u;
         }
     }
@@ -1598,13 +1585,13 @@ int launch_energy_few(const HamView& h, const void* psi, double2* w, double* par
 }
 
 int launch_energy_matrix_free(const HamView& h, const void* psi, int psi_prec, double* partials,
-                              unsigned* ticket, DevStep* step, DevStep* host, int sms, cudaStream_t s) {
+                              unsigned* ticket, DevStep* step, int sms, cudaStream_t s) {
     const long long blocks = (h.D + 255) / 256;                 // one row per thread
     const int grid = (int)(blocks < (long long)sms * 8 ? blocks : (long long)sms * 8);
     if (psi_prec == TQ_C128)
-        k_energy_mf<double><<<grid, 256, 0, s>>>(h, static_cast<const double2*>(psi), partials, ticket, step, host);
+        k_energy_mf<double><<<grid, 256, 0, s>>>(h, static_cast<const double2*>(psi), partials, ticket, step);
     else
-        k_energy_mf<float><<<grid, 256, 0, s>>>(h, static_cast<const float2*>(psi), partials, ticket, step, host);
+        k_energy_mf<float><<<grid, 256, 0, s>>>(h, static_cast<const float2*>(psi), partials, ticket, step);
     return 1;
 }
 

@@ -17,7 +17,9 @@ all 2 GiB, is reported beside it.
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
 Under torchrun every rank runs its own 8192 states (weak scaling, no
-collective on the data path); rank 0 prints one JSON line.
+collective on the data path); rank 0 prints one JSON line with the headline
+(under 3 KB) and writes the whole record, sections and tuning tables included,
+to a file (--record, bench_record.json in the working directory).
 """
 
 from __future__ import annotations
@@ -67,6 +69,29 @@ def workload_config(n_states):
                      "lines and sectors, in place)",
         "norm": "float64 squared norm per state, carried across steps",
     }
+
+
+# what of the record goes on the printed line (None: whole)
+LINE_KEYS = {
+    "metric": None, "value": None, "unit": None, "impl": None, "n_gpus": None, "steps": None, "warmup": None,
+    "ms_per_step": None, "higher_is_better": None, "scaling": None, "vs_baseline": None, "dtype": None, "data": None,
+    "gpu_launches": None, "clocks": None, "norms_finite": None,
+    "config": ("workload", "n_states", "n_qubits", "pool_size", "mapping", "state_precision", "l2_policy", "norm"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "algorithmic_bytes_per_launch",
+                 "sector_frac", "kernel_ms_per_launch", "update_over_touch_floor", "peak_source"),
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "api"),
+}
+
+
+def headline_line(out):
+    """The record's headline as one JSON line (the sections stay in the record)."""
+    line = {}
+    for key, keep in LINE_KEYS.items():
+        if key in out:
+            v = out[key]
+            line[key] = {k: v[k] for k in keep if k in v} if keep and isinstance(v, dict) else v
+    return json.dumps(line)
 
 
 # ------------------------------------------------------------------ helpers
@@ -1871,6 +1896,8 @@ def main():
                     help="headline states checked against the oracle after the run (0 skips)")
     ap.add_argument("--pair-schedule", type=int, default=0,
                     help="support pairs per thread of the update (0 = autotune)")
+    ap.add_argument("--record", default="bench_record.json",
+                    help="file for the whole record: the line's headline, every section, the tuning tables ('' skips)")
     args = ap.parse_args()
     rank = int(os.environ.get("RANK", "0"))
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -1940,7 +1967,11 @@ def main():
                 out["rates_14q"]["oracle"] = oracle_rates(seconds=2.0)
         else:
             out["cpu_baseline"] = None
-        print(json.dumps(out))
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(out, f)
+                f.write("\n")
+        print(headline_line(out), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

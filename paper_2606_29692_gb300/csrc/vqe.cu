@@ -265,8 +265,19 @@ k_ansatz_forward(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
     for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) psi_end[((size_t)rank << slice_log) + i] = st[i];
 }
 
-// chi_in null: chi = w - E psi at the end of the ansatz (the first launch of
-// the sweep), else the chi an earlier launch left.  part: [SWEEP_OPS][CTAs].
+// complex64 carries chi divided by 4^k, about <psi|psi>: the dots' float32
+// products of chi and phi are then near 1 whatever the state's norm (at norm
+// 1e-18 they fell below float32's range), and every other step is linear in
+// chi, so the scaling changes no bit.  Returns k (0 for complex128).
+template <typename T>
+__device__ __forceinline__ int sweep_scale(double den) {
+    const int e = ((__double2hiint(den) >> 20) & 0x7ff) - 1023;
+    return sizeof(T) == 8 || e < -250 || e > 250 ? 0 : e >> 1;
+}
+
+// chi_in null: chi = (w - E psi) / 4^k at the end of the ansatz (the first
+// launch of the sweep), else the chi an earlier launch left.  part:
+// [SWEEP_OPS][CTAs].
 template <typename T>
 __global__ void __launch_bounds__(SWEEP_MAX_TPB)
 k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int slice_log,
@@ -282,6 +293,8 @@ k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
     V* st = reinterpret_cast<V*>(wsum + (size_t)SWEEP_OPS * nw);
     const uint32_t per = 1u << slice_log, lo = per - 1u, rank = cl.block_rank();
     const double E = step->energy;
+    const int k = sweep_scale<T>(step->e_den);
+    const T sc = (T)__int_as_float((127 - k) << 23);             // 2^-k, applied twice: 4^-k may leave the range
     for (uint32_t i = threadIdx.x; i < per; i += blockDim.x) {
         const size_t r = ((size_t)rank << slice_log) + i;
         if (chi_in) {
@@ -290,6 +303,7 @@ k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
             const double2 wr = w[r];
             const V pr = psi[r];
             st[i] = {(T)(wr.x - E * (double)pr.x), (T)(wr.y - E * (double)pr.y)};
+            if (sizeof(T) == 4) st[i] = {st[i].x * sc * sc, st[i].y * sc * sc};
         }
     }
     sweep_prepare<T>(p, ops, n, true, op);
@@ -351,7 +365,7 @@ k_ansatz_adjoint(PoolView p, const __grid_constant__ SweepOps ops, int n, int sl
         for (int j = threadIdx.x; j < n; j += blockDim.x) {
             double v = 0.0;
             for (unsigned i = 0; i < cl.num_blocks(); ++i) v += __ldcg(part + (size_t)j * SWEEP_MAX_CLUSTER + i);
-            grad[j] = 2.0 * v / step->e_den;
+            grad[j] = 2.0 * v / (step->e_den * __hiloint2double((1023 - 2 * k) << 20, 0));
         }
 }
 

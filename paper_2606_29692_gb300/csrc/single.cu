@@ -513,7 +513,7 @@ k_large_update(PoolView p, int k_imm, double th_imm, const DevStep* gate, typena
             if (threadIdx.x == 0) {
                 const double n = t.norm2(growth), sc = 1.0 / sqrt(n);
                 scale_sh[0] = (T)sc;
-                scale_sh[1] = (T)(sc - (double)scale_sh[0]);
+                scale_sh[1] = isinf(sc) ? T(0) : (T)(sc - (double)scale_sh[0]);   // a norm below the range: as one factor
                 if (blockIdx.x == 0 && norm2_out) *norm2_out = n;
             }
         }

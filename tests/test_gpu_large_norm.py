@@ -32,3 +32,16 @@ def test_norm_after_rescale(scale, pick, th):
     sums = 0.5 * np.sqrt(24 / 3) / np.sqrt(D / 8)
     rescale = np.sqrt(2 / 3 / D)
     assert abs(norm - 1) <= 6 * u * (sums + rescale)
+
+
+def test_norm_below_the_range():
+    """Squares below float32's range: the factor is infinite, as it is for the batched update's norm."""
+    ctx = tq.Context(0)
+    pool = tq.build_pool(ctx, Q // 2, 4, tq.TQ_JW)
+    psi = np.zeros(1 << Q, complex)
+    psi[5], psi[9] = 1e-30, -1e-30j
+    st = to_state(ctx, psi, Q, tq.TQ_C64)
+    tq.evolve_taylor5(ctx, pool, 0, 0.0, st, renormalize=True)
+    got = st.numpy()
+    assert got[5].real == np.inf and got[9].imag == -np.inf
+    assert np.all(np.isnan(got[[5, 9]].view(float)[[1, 2]])) and np.all(np.isnan(got[10:20]))

@@ -10,8 +10,8 @@ doubles) and angle.  One step = one launch of the support-only update over
 all 8192 states: each state's generator support (D/2 rows for a single,
 D/8 for a double) is read and written in place, rows off the support are
 left as they are (every term of the series past the first vanishes there),
-and each state's float64 squared norm is carried (about 0.83 GB of DRAM
-traffic per step, larger than L2).  The full-state kernel, which streams
+and each state's float64 squared norm is carried (about 0.44 GB of DRAM
+sectors per step, larger than L2).  The full-state kernel, which streams
 all 2 GiB, is reported beside it.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -65,8 +65,8 @@ def workload_config(n_states):
         "pool_size": 204,
         "mapping": "BK",
         "state_precision": "complex64 (float32 products), float64 norm reduction",
-        "l2_policy": "inputs larger than L2 (1 GiB of states; each step moves about 0.83 GB of support "
-                     "lines and sectors, in place)",
+        "l2_policy": "inputs larger than L2 (1 GiB of states; each step moves about 0.44 GB of support "
+                     "sectors, in place)",
         "norm": "float64 squared norm per state, carried across steps",
     }
 
